@@ -184,7 +184,7 @@ def dmr_quantize(W: torch.Tensor, fmt: QFormat, stream=None, check: bool = True)
     qweight = torch.empty((N, K * fmt.bits // 32), dtype=torch.int32, device=W.device)
     scales = torch.empty((N, G), dtype=torch.bfloat16, device=W.device)
     zeros = torch.empty((N, G), dtype=torch.uint8, device=W.device)
-    status = torch.zeros(1, dtype=torch.int32, device=W.device)
+    status = torch.zeros(1, dtype=torch.int32, device=W.device) if check else None  # nobody could read it otherwise
     _check(L.dmr_quantize(_ptr(W), N, K, fmt, _ptr(qweight), _ptr(scales), _ptr(zeros), _ptr(status), _stream(stream)))
     if check:
         code = int(status.item())
