@@ -25,6 +25,14 @@ inline dmr_status_t check_launch() {
     return DMR_OK;
 }
 
+inline dmr_status_t launch_failed(cudaError_t e) {
+    g_last_cuda_error = (int)e;
+    (void)cudaGetLastError();
+    return DMR_ERR_CUDA;
+}
+
+int device_sm_count();  // SMs of the current device
+
 inline bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 inline int group_of(int K, dmr_qformat_t f) { return f.group_size == 0 ? K : f.group_size; }

@@ -97,6 +97,18 @@ bool ensure_dynamic_smem(const void *kernel, size_t bytes) {
     return true;
 }
 
+int device_sm_count() {
+    static int cached[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+    if (cached[dev] == 0) {
+        int n = 0;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) cached[dev] = n;
+        else cached[dev] = 148;
+    }
+    return cached[dev];
+}
+
 bool tc_pdl_enabled() {
     static int v = -1;
     if (v < 0) {
