@@ -169,6 +169,12 @@ size_t router_attention_smem(int L, int dh);
 dmr_status_t launch_router_forward(const float *params, const dmr_router_cfg_t &c, const float *Z, const int32_t *lengths, int B,
                                    int L, float *probs, float *scores, int score_class, float *ws, cudaStream_t st);
 
+// The same forward pass as one cooperative launch, for calls of up to this many (padded) tokens; `ws` as above.
+constexpr long long kRouterFusedMaxTokens = 4096;
+bool router_fused_supported(const dmr_router_cfg_t &c, int B, int L);
+dmr_status_t launch_router_fused(const float *params, const dmr_router_cfg_t &c, const float *Z, const int32_t *lengths, int B, int L,
+                                 float *probs, float *scores, int score_class, float *ws, cudaStream_t st);
+
 // One warp waits on a barrier nobody arrives at, with a short limit: *status becomes DMR_ERR_TIMEOUT, *returned 2.
 dmr_status_t launch_wait_timeout_selftest(int32_t *status, int32_t *returned, cudaStream_t st);
 

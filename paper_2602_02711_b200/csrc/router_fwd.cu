@@ -13,8 +13,10 @@
 // Arithmetic: fp32 throughout (CUDA cores; fused multiply-adds), so that the probabilities agree with a binary64
 // evaluation to about 1e-6 and the comparison against a threshold is stable.  The model is small (14 M parameters at
 // d = 384 and 8 layers) and runs once per agent step, next to a language-model call of tens of milliseconds.
-// Kernels: positions added; per layer a linear (QKV; tiled, or one feature per warp when there are at most 32 tokens), one CTA per (sequence, head) for the attention, a linear
-// with the residual added, a layer norm, two linears (ReLU; residual), a layer norm; then pooling, head and softmax.
+// Calls of up to kRouterFusedMaxTokens tokens with a head width of 16, 32, 64 or 128 are one launch (router_fused.cu); this file has the
+// layer-by-layer kernels for the others: positions added; per layer a linear (QKV; tiled, or one feature per warp when there are at
+// most 32 tokens), one CTA per (sequence, head) for the attention, a linear with the residual added, a layer norm, two linears (ReLU;
+// residual), a layer norm; then pooling, head and softmax.
 #include "sm100.cuh"
 
 namespace dmr {
@@ -305,13 +307,19 @@ size_t router_param_floats(const dmr_router_cfg_t &c) {
 
 size_t router_workspace_bytes(const dmr_router_cfg_t &c, int B, int L) {
     const size_t T = (size_t)B * L;
-    return round_up(T * (size_t)(6 * c.d + c.ffn) * sizeof(float), 256);
+    const size_t fused = 7 * T * (size_t)c.d * sizeof(float) + 256;  // input rows, two buffers of QKV, a counter
+    const size_t layered = T * (size_t)(6 * c.d + c.ffn) * sizeof(float);
+    return round_up(fused > layered ? fused : layered, 256);
 }
 
 size_t router_attention_smem(int L, int dh) { return ((size_t)2 * L * (dh + 1) + (size_t)kAttWarps * L + (size_t)kAttWarps * dh) * sizeof(float); }
 
 dmr_status_t launch_router_forward(const float *params, const dmr_router_cfg_t &c, const float *Z, const int32_t *lengths, int B,
                                    int L, float *probs, float *scores, int score_class, float *ws, cudaStream_t st) {
+    if (router_fused_supported(c, B, L)) {
+        const dmr_status_t rf = launch_router_fused(params, c, Z, lengths, B, L, probs, scores, score_class, ws, st);
+        if (rf != DMR_ERR_UNSUPPORTED) return rf;
+    }
     const int d = c.d, f = c.ffn, T = B * L, dh = c.d / c.heads;
     float *H = ws;                        // [T][d]   the layer's input and output
     float *QKV = H + (size_t)T * d;       // [T][3 d]
