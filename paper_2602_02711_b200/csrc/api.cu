@@ -98,7 +98,7 @@ Scratch carve(void *workspace, dmr_op_t op, int M, int N, int K, dmr_qformat_t f
         s.prefill_scratch = base + off;
         off += round_up(prefill_scratch_bytes(M, K), 256);
     }
-    const size_t partial_low = !low_gemm ? 0 : (prefill_supported(M, N, K, f.bits, g) ? prefill_partial_bytes(M, N, K) : gemm_plan(M, N, K, f.bits).partial_bytes);
+    const size_t partial_low = !low_gemm ? 0 : (prefill_supported(M, N, K, f.bits, g) ? prefill_partial_bytes(M, N, K, f.bits, g) : gemm_plan(M, N, K, f.bits).partial_bytes);
     const size_t partial_dense = dense_gemm ? gemm_plan(M, N, K, 0).partial_bytes : 0;
     if (op == DMR_OP_ROUTED_LINEAR) {
         if (partial_low) {
@@ -477,6 +477,11 @@ int dmr_describe_dispatch(dmr_op_t op, int M, int N, int K, dmr_qformat_t f, cha
     if (!dense && !format_ok(K, f)) return -1;
     const int bits = dense ? 0 : f.bits, g = dense ? K : group_of(K, f);
     if (use_gemm(M, N, K, bits, g)) {
+        if (!dense && pair_supported(M, N, K, bits, g)) {  // tiles counted per CTA: 128 features each
+            const PairPlan p = pair_plan(M, N, K, bits);
+            return snprintf(buf, buf_bytes, "prefill bits=%d bn=256 rows=%d splits=%d tiles=%d ctas=%d", bits, p.rows, p.splits,
+                            (N + 127) / 128 * (p.tiles / p.n_tiles), p.ctas);
+        }
         if (!dense && prefill_supported(M, N, K, bits, g)) {
             int bn, splits, ctas;
             long long tiles;

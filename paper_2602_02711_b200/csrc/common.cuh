@@ -108,17 +108,29 @@ void decode_w3_plan(int M, int *nt, int *r, int *warps);
 void stream_plan(int M, int N, int K, int bits, int *tiles, long long *steps, int *cluster);
 void prefill_plan(int M, int N, int K, int *bn, int *splits, long long *tiles, int *ctas);
 
-// Persistent prefill GEMM (M > 32, low-bit weights); sel.idx maps batch slots to rows of X and Y, sel.count
+// Low-bit linears on the tensor cores (M > 32; batches of more than 128 rows go on to launch_pair); sel.idx maps batch slots to rows of X and Y, sel.count
 // says how many slots are valid.
 bool prefill_supported(int M, int N, int K, int bits, int g);
 // X is the caller's activation matrix (for a routed call the rows sel.idx lists are gathered);
 // `scratch` holds prefill_scratch_bytes(M, K) bytes for the prepared fp16 activations and their row scales, `partial`
 // prefill_partial_bytes(M, N, K) bytes of fp32 partial sums (0 unless the call is split along k).
 size_t prefill_scratch_bytes(int M, int K);
-size_t prefill_partial_bytes(int M, int N, int K);
+size_t prefill_partial_bytes(int M, int N, int K, int bits, int g);
 dmr_status_t launch_prefill(const uint16_t *X, int M, RowSel sel, const void *qweight, const uint16_t *scales,
                             const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out,
                             void *scratch, float *partial, int32_t *status, cudaStream_t st);
+
+// Large batches (M > 128) on pairs of SMs: bf16 weights (bits == 0) and packed codes.  X is the bf16 matrix, or for codes the
+// prepared fp16 one with its row scales.
+struct PairPlan {
+    int n_tiles, rows, splits, kb_per_split, tiles, ctas;
+    size_t partial_bytes;
+};
+bool pair_supported(int M, int N, int K, int bits, int g);
+PairPlan pair_plan(int M, int N, int K, int bits);
+dmr_status_t launch_pair(const uint16_t *X, int M, RowSel sel, const float *xscale, const void *weights, const uint16_t *scales,
+                         const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out, float *partial, int32_t *status,
+                         cudaStream_t st);
 
 // Tensor-core GEMM family (M > 16): tcgen05 MMA with TMA-staged operands.
 struct GemmPlan {

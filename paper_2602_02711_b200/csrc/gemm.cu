@@ -407,8 +407,6 @@ dmr_status_t launch_gemm_bn(int BN, const CUtensorMap &map_w, const CUtensorMap 
     switch (BN) {
         case 32: return launch_gemm_t<MODE, 32>(map_w, map_x, a, splits, out, st);
         case 64: return launch_gemm_t<MODE, 64>(map_w, map_x, a, splits, out, st);
-        case 256:
-            if constexpr (MODE == 0) return launch_gemm_t<MODE, 256>(map_w, map_x, a, splits, out, st);
         default: return launch_gemm_t<MODE, 128>(map_w, map_x, a, splits, out, st);
     }
 }
@@ -425,8 +423,15 @@ bool gemm_supported(int M, int N, int K, int bits /*0 = dense*/, int g) {
 
 GemmPlan gemm_plan(int M, int N, int K, int bits) {
     GemmPlan p;
+    if (bits == 0 && pair_supported(M, N, K, 0, K)) {  // handed on by launch_gemm
+        const PairPlan q = pair_plan(M, N, K, 0);
+        p.bn = q.rows;
+        p.splits = q.splits;
+        p.kblocks_per_split = q.kb_per_split;
+        p.partial_bytes = q.partial_bytes;
+        return p;
+    }
     p.bn = M <= 32 ? 32 : (M <= 64 ? 64 : 128);
-    if (bits == 0 && M > 128) p.bn = 256;
     const int tiles = ((N + BM - 1) / BM) * ((M + p.bn - 1) / p.bn);
     const int kb = K / BK;
     // Split-K factor: the one with the shortest longest path - waves of CTAs (one CTA per SM at a time) times the k blocks
@@ -454,6 +459,8 @@ GemmPlan gemm_plan(int M, int N, int K, int bits) {
 dmr_status_t launch_gemm(const uint16_t *X, int M, RowSel sel, const void *weights, const uint16_t *scales,
                          const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out,
                          float *partial, int32_t *status, cudaStream_t st) {
+    if (bits == 0 && pair_supported(M, N, K, 0, K))
+        return launch_pair(X, M, sel, nullptr, weights, nullptr, nullptr, N, K, 0, K, Y, out, partial, status, st);
     const GemmPlan p = gemm_plan(M, N, K, bits);
     CUtensorMap map_w, map_x;
     if (!make_tensor_map_2d(&map_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)K, (uint64_t)K * 2,

@@ -1,20 +1,21 @@
-// Prefill-sized low-bit linear layers (M in the hundreds and above; 3-, 4- and 8-bit codes): a persistent, warp-specialised
+// Low-bit linear layers on the tensor cores (3-, 4- and 8-bit codes): activation preparation for all batches, and for 33 to 128 rows
+// (more go to pair.cu) a persistent, warp-specialised
 // tcgen05 GEMM with the dequantisation fused into the operand pipeline.  Prefill is a dense
 // contraction (its cost is folded into the per-token latency, App. "Latency coefficients"), so it
 // belongs on the tensor cores.
 //
 // Orientation: the weights are the 128-row operand (D[n][m] = sum_k W^[n][k] X[m][k]), one
-// tensor-memory lane per output feature, BN (64, 128 or 256) activation rows as the N operand.
+// tensor-memory lane per output feature, BN (64 or 128) activation rows as the N operand.
 //
 // Per 64-wide k block and stage of the ring:
 //   warp 0      TMA: the packed code tile [128 features x 32 or 64 bytes] and the activation tile
 //               [BN rows x 128 bytes, 128-byte swizzle] land in shared memory (one mbarrier);
-//   warps 2..9 (2..13 for the 64- and 128-row tiles)  one thread per feature row turns its codes into the fp16 weights s' * (q - zero)
+//   warps 2..13  one thread per feature row turns its codes into the fp16 weights s' * (q - zero)
 //               (exact integer q - zero, then ONE rounding of the product to 11 significant bits)
 //               and stores them as the swizzled K-major A tile;
 //   warp 1      one lane issues four tcgen05.mma (128 x BN x 16) that accumulate into one of two
 //               fp32 accumulators in tensor memory, and commits the stage back to the producer;
-//   the last four warps (eight for the 256-row tile, two per lane quadrant with half of the columns each)
+//   the last four warps
 //               drain the finished accumulator of the previous tile (tcgen05.ld) into Y while the
 //               next tile's MMAs run into the other accumulator (a block of 32 rows at a time: the rows' scales and
 //               output rows come from one coalesced load each, never from loads inside the store loop).
@@ -32,6 +33,7 @@
 #include <type_traits>
 
 #include "sm100.cuh"
+#include "unpack.cuh"
 
 namespace dmr {
 
@@ -51,36 +53,14 @@ struct PrefillCfg {
     static constexpr int S_RAW = (212 * 1024) / STAGE;
     static constexpr int S = S_RAW > 8 ? 8 : S_RAW;
     static constexpr int TMEM_COLS = 2 * BN;                 // two accumulators
-    // unpack warps: UW / 4 groups of four, group i takes every (UW / 4)-th stage of the ring.  Three groups for the
-    // 64- and 128-row tiles (small batches: a stage's MMAs are short and the unpack chain's latency is what is left), two for 256.
-    static constexpr int UW = BN == 256 ? 8 : 12;
-    // epilogue warps: four (one per tensor-memory lane quadrant), eight for the 256-row tile (two per quadrant, each draining
-    // half of the accumulator's columns: what is left after a CTA's last MMA is its last tile's epilogue)
-    static constexpr int EW = BN == 256 ? 8 : 4;
+    // unpack warps: three groups of four, group i takes every third stage of the ring (small batches: a stage's MMAs are short and the
+    // unpack chain's latency is what is left)
+    static constexpr int UW = 12;
+    // epilogue warps: one per tensor-memory lane quadrant (eight would make the 704 threads spill)
+    static constexpr int EW = 4;
     static constexpr int THREADS = 32 * (2 + UW + EW);
     static constexpr size_t SMEM = (size_t)S * STAGE + 1024 /*alignment*/ + 512 /*barriers*/;
 };
-
-// Largest magnitude pattern among a feature's G bf16 scales (sign bit cleared): eight scales per 16-byte load when the
-// row of the table allows it, so that a work item's set-up is a handful of independent loads, not a chain of G.
-__device__ __forceinline__ uint32_t scale_row_max(const uint16_t *sp, int G) {
-    uint32_t m0 = 0, m1 = 0;
-    int gi = 0;
-    // scalar loads up to the first 16-byte boundary, 16-byte loads over the aligned middle, scalar loads for the rest
-    const int head = (int)(((16u - (uint32_t)(reinterpret_cast<uintptr_t>(sp) & 15u)) & 15u) >> 1);
-    for (; gi < G && gi < head; ++gi) m0 = max(m0, (uint32_t)__ldg(sp + gi) & 0x7FFFu);
-    for (; gi + 8 <= G; gi += 8) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(sp + gi));
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            m0 = max(m0, w[i] & 0x7FFFu);
-            m1 = max(m1, (w[i] >> 16) & 0x7FFFu);
-        }
-    }
-    for (; gi < G; ++gi) m1 = max(m1, (uint32_t)__ldg(sp + gi) & 0x7FFFu);
-    return max(m0, m1);
-}
 
 struct PrefillArgs {
     const uint16_t *scales;
@@ -307,169 +287,31 @@ prefill_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         // at the same time: group i takes the stages whose running number is i modulo NG.
         const int r = ((warp - 2) & 3) * 32 + lane;  // feature row of the tile
         constexpr int NG = Cfg::UW / 4;
-        constexpr int CH = 8, c_lo = 0;               // 16-byte chunks (8 weights each) per thread and stage
         const int grp_id = (warp - 2) >> 2;
-        const uint32_t swz = (uint32_t)(r & 7);
         uint32_t it0 = 0;  // running number of the work item's first stage
         bool ok = true;
         for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
             const int split = SPLITK ? tile % n_splits : 0, tl = SPLITK ? tile / n_splits : tile;
             const int kb_lo = SPLITK ? split * a.kb_per_split : 0, kb_hi = SPLITK ? min(nkb, kb_lo + a.kb_per_split) : nkb;
             const int n = min((tl % a.n_tiles) * PM + r, a.N - 1);
-            const uint16_t *sp = a.scales + (size_t)n * G;
-            const uint8_t *zp = a.zeros + (size_t)n * G;
-            // power of two of the feature's largest scale: s' = s * 2^-f lies in (0, 2)
-            const uint32_t smax = scale_row_max(sp, G);
-            int fb = (int)(smax >> 7);
-            fb = fb < 1 ? 1 : (fb > 253 ? 253 : fb);
-            const float fdown = __uint_as_float((uint32_t)(254 - fb) << 23);  // 2^-(fb - 127)
+            UnpackRow<BITS> row;
+            row.begin(a.scales + (size_t)n * G, a.zeros + (size_t)n * G, G, BITS == 3 ? a.qweight3 + (size_t)n * (size_t)(a.K / 32 * 3) : nullptr);
             int kb = kb_lo + (int)(((uint32_t)grp_id + (uint32_t)NG - it0 % (uint32_t)NG) % (uint32_t)NG);  // this group's first k block of the item
-            uint32_t sb = 0, zb = 0;
-            if (kb < kb_hi) {
-                sb = __ldg(sp + kb / kb_per_group);
-                zb = __ldg(zp + kb / kb_per_group);
-            }
-            // 3-bit codes: this row's six words of the stage, read from global memory one stage of this group ahead
-            const uint32_t *wrow = a.qweight3 + (size_t)n * (size_t)(a.K / 32 * 3);
-            uint2 w3a = make_uint2(0u, 0u), w3b = w3a, w3c = w3a;
-            if (BITS == 3 && kb < kb_hi) {
-                w3a = __ldg(reinterpret_cast<const uint2 *>(wrow + kb * 6));
-                w3b = __ldg(reinterpret_cast<const uint2 *>(wrow + kb * 6 + 2));
-                w3c = __ldg(reinterpret_cast<const uint2 *>(wrow + kb * 6 + 4));
-            }
+            if (kb < kb_hi) row.fetch(kb, kb / kb_per_group);
             for (; kb < kb_hi; kb += NG) {
                 const uint32_t it = it0 + (uint32_t)(kb - kb_lo);
                 const int s = it % S;
-                uint2 n3a = w3a, n3b = w3b, n3c = w3c;
-                if (BITS == 3 && kb + NG < kb_hi) {
-                    n3a = __ldg(reinterpret_cast<const uint2 *>(wrow + (kb + NG) * 6));
-                    n3b = __ldg(reinterpret_cast<const uint2 *>(wrow + (kb + NG) * 6 + 2));
-                    n3c = __ldg(reinterpret_cast<const uint2 *>(wrow + (kb + NG) * 6 + 4));
-                }
-                // scale / zero of this group's next k block, fetched while this block is unpacked
-                uint32_t sb_next = sb, zb_next = zb;
-                if (kb + NG < kb_hi) {
-                    const int grp = (kb + NG) / kb_per_group;
-                    sb_next = __ldg(sp + grp);
-                    zb_next = __ldg(zp + grp);
-                }
+                row.take();
+                // what this group's next k block needs from global memory, fetched while this block is unpacked
+                if (kb + NG < kb_hi) row.fetch(kb + NG, (kb + NG) / kb_per_group);
                 if (!mbar_wait(full_bar(s), (it / S) & 1, a.status)) {
                     ok = false;
                     break;
                 }
-                const uint32_t src = p_tile(s) + r * Cfg::P_ROW;
-                const uint32_t dst = a_tile(s) + r * 128;
-                if (BITS == 3) {
-                    // fp16 patterns: a half-word holds five codes at bits 0, 3, 6, 9, 12.  0x6400 | (bits 0..2) = 1024 + q,
-                    // 0x6400 | (bits 3..5) = 1024 + 8 q, 0x6400 | (bits 6..8) = 1024 + 64 q without a shift (10 mantissa
-                    // bits); one shift by 9 brings the last two down.  Minus the matching 1024 + zero is exact, then one
-                    // rounding of the product with s', s'/8 or s'/64.
-                    const float sf = __uint_as_float(sb << 16) * fdown;
-                    uint32_t s2, s2_8, s2_64;
-                    asm("cvt.rn.f16x2.f32 %0, %1, %1;" : "=r"(s2) : "f"(sf));
-                    asm("cvt.rn.f16x2.f32 %0, %1, %1;" : "=r"(s2_8) : "f"(sf * 0.125f));
-                    asm("cvt.rn.f16x2.f32 %0, %1, %1;" : "=r"(s2_64) : "f"(sf * 0.015625f));
-                    const uint32_t z1 = 0x6400u | zb, z8 = 0x6400u | (zb << 3), z64 = 0x6400u | (zb << 6);
-                    const uint32_t zo1 = z1 | (z1 << 16), zo8 = z8 | (z8 << 16), zo64 = z64 | (z64 << 16);
-                    const uint32_t words[6] = {w3a.x, w3a.y, w3b.x, w3b.y, w3c.x, w3c.y};
-#pragma unroll
-                    for (int blk = 0; blk < 2; ++blk) {  // 32 codes = three words = four 16-byte chunks of fp16 weights
-                        uint32_t D[16];  // pair 5 j + i = codes (10 j + i, 10 j + 5 + i); pair 15 = codes (30, 31)
-#pragma unroll
-                        for (int j = 0; j < 3; ++j) {
-                            const uint32_t u = words[3 * blk + j], u9 = u >> 9;
-                            D[5 * j + 0] = f16x2_mul(f16x2_sub(lop3_and_or(u, 0x00070007u, 0x64006400u), zo1), s2);
-                            D[5 * j + 1] = f16x2_mul(f16x2_sub(lop3_and_or(u, 0x00380038u, 0x64006400u), zo8), s2_8);
-                            D[5 * j + 2] = f16x2_mul(f16x2_sub(lop3_and_or(u, 0x01C001C0u, 0x64006400u), zo64), s2_64);
-                            D[5 * j + 3] = f16x2_mul(f16x2_sub(lop3_and_or(u9, 0x00070007u, 0x64006400u), zo1), s2);
-                            D[5 * j + 4] = f16x2_mul(f16x2_sub(lop3_and_or(u9, 0x00380038u, 0x64006400u), zo8), s2_8);
-                        }
-                        {
-                            uint32_t t = lop3_and_or(words[3 * blk] >> 15, 0x00010001u, 0x64006400u);
-                            t = lop3_and_or(words[3 * blk + 1] >> 14, 0x00020002u, t);
-                            t = lop3_and_or(words[3 * blk + 2] >> 13, 0x00040004u, t);
-                            D[15] = f16x2_mul(f16x2_sub(t, zo1), s2);
-                        }
-                        // code a of the block: pair and half it sits in; the tile wants neighbours (2 v, 2 v + 1) side by side
-                        auto pair_of = [](int a) { return a >= 30 ? 15 : 5 * (a / 10) + (a % 10) % 5; };
-                        auto high_of = [](int a) { return a >= 30 ? a - 30 : ((a % 10) >= 5 ? 1 : 0); };
-#pragma unroll
-                        for (int c4 = 0; c4 < 4; ++c4) {
-                            uint32_t o[4];
-#pragma unroll
-                            for (int v4 = 0; v4 < 4; ++v4) {
-                                const int a0 = 8 * c4 + 2 * v4, a1 = a0 + 1;
-                                o[v4] = prmt(D[pair_of(a0)], D[pair_of(a1)], (high_of(a1) ? 0x7600u : 0x5400u) | (high_of(a0) ? 0x32u : 0x10u));
-                            }
-                            const uint32_t addr = dst + ((((uint32_t)(4 * blk + c4)) ^ swz) << 4);
-                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
-                        }
-                    }
-                } else if (BITS == 4) {
-                    uint32_t w[CH];
-#pragma unroll
-                    for (int c4 = 0; c4 < CH; c4 += 4)
-                        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
-                                     : "=r"(w[c4]), "=r"(w[c4 + 1]), "=r"(w[c4 + 2]), "=r"(w[c4 + 3])
-                                     : "r"(src + 4 * (c_lo + c4)));
-                    // fp16 patterns: 0x6400 | q = 1024 + q and 0x6400 | (q << 4) = 1024 + 16 q (no shift needed
-                    // for the odd codes); minus 1024 + zero (or 1024 + 16 zero) is exact; then one rounding
-                    const float sf = __uint_as_float(sb << 16) * fdown;
-                    uint32_t s2, s2_16;
-                    asm("cvt.rn.f16x2.f32 %0, %1, %1;" : "=r"(s2) : "f"(sf));
-                    asm("cvt.rn.f16x2.f32 %0, %1, %1;" : "=r"(s2_16) : "f"(sf * 0.0625f));
-                    const uint32_t zz = 0x6400u | zb, zz16 = 0x6400u | (zb << 4);
-                    const uint32_t zoff = zz | (zz << 16), zoff16 = zz16 | (zz16 << 16);
-#pragma unroll
-                    for (int cc = 0; cc < CH; ++cc) {  // word c = codes 8c .. 8c+7 = 16-byte chunk c of the row
-                        const int c = c_lo + cc;
-                        const uint32_t w8 = w[cc] >> 8;
-                        const uint32_t d04 = f16x2_mul(f16x2_sub(lop3_and_or(w[cc], 0x000F000Fu, 0x64006400u), zoff), s2);
-                        const uint32_t d15 = f16x2_mul(f16x2_sub(lop3_and_or(w[cc], 0x00F000F0u, 0x64006400u), zoff16), s2_16);
-                        const uint32_t d26 = f16x2_mul(f16x2_sub(lop3_and_or(w8, 0x000F000Fu, 0x64006400u), zoff), s2);
-                        const uint32_t d37 = f16x2_mul(f16x2_sub(lop3_and_or(w8, 0x00F000F0u, 0x64006400u), zoff16), s2_16);
-                        const uint32_t o01 = prmt(d04, d15, 0x5410), o45 = prmt(d04, d15, 0x7632);
-                        const uint32_t o23 = prmt(d26, d37, 0x5410), o67 = prmt(d26, d37, 0x7632);
-                        const uint32_t addr = dst + ((((uint32_t)c) ^ swz) << 4);
-                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(o01), "r"(o23), "r"(o45), "r"(o67) : "memory");
-                    }
-                } else {
-                    const float zf = __uint_as_float(0x4B000000u | zb);  // 2^23 + zero
-                    const float sf = __uint_as_float(sb << 16) * fdown;
-                    // A row of codes is 64 bytes = four 16-byte pieces.  Lane r starts at piece (r / 2) % 4, so that the eight
-                    // lanes of a load phase read eight different bank groups (all starting at piece 0 would meet in two).
-                    // Piece q holds codes 16 q .. 16 q + 15 = chunks 2 q and 2 q + 1 of the fp16 row.
-#pragma unroll
-                    for (int j = 0; j < CH / 2; ++j) {
-                        const uint32_t q = ((uint32_t)j + (uint32_t)(r >> 1)) & 3u;
-                        uint32_t wq[4];
-                        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(wq[0]), "=r"(wq[1]), "=r"(wq[2]), "=r"(wq[3]) : "r"(src + 16u * q));
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            uint32_t o[4];
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const uint32_t u = wq[2 * e + h];
-                                float f[4];
-#pragma unroll
-                                for (int b = 0; b < 4; ++b)  // (q - zero) exactly, times the scale exactly (8 x 8 bits)
-                                    f[b] = __fmul_rn(__fsub_rn(__uint_as_float(prmt(u, 0x4B000000u, 0x7650u + (uint32_t)b)), zf), sf);
-                                o[2 * h] = pack_f16x2_rn(f[0], f[1]);  // the one rounding
-                                o[2 * h + 1] = pack_f16x2_rn(f[2], f[3]);
-                            }
-                            const uint32_t addr = dst + (((2u * q + (uint32_t)e) ^ swz) << 4);
-                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
-                        }
-                    }
-                }
+                row.unpack(p_tile(s) + r * Cfg::P_ROW, a_tile(s) + r * 128, r);
                 fence_proxy_async_smem();  // the tile must be visible to the tensor core's reads
                 __syncwarp();
                 if (lane == 0) mbar_arrive(ready_bar(s));
-                sb = sb_next;
-                zb = zb_next;
-                w3a = n3a;
-                w3b = n3b;
-                w3c = n3c;
             }
             it0 += (uint32_t)(kb_hi - kb_lo);
         }
@@ -486,10 +328,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             const int split = SPLITK ? tile % n_splits : 0, tl = SPLITK ? tile / n_splits : tile;
             const int n = (tl % a.n_tiles) * PM + r, m0 = (tl / a.n_tiles) * BN;
             // the power of two the unpack threads divided this feature's scales by, undone here
-            const uint32_t smax = scale_row_max(a.scales + (size_t)min(n, a.N - 1) * G, G);
-            int fb = (int)(smax >> 7);
-            fb = fb < 1 ? 1 : (fb > 253 ? 253 : fb);
-            const float fscale = __uint_as_float((uint32_t)fb << 23);  // 2^(fb - 127)
+            const float fscale = feature_scale(a.scales + (size_t)min(n, a.N - 1) * G, G);
             if (!mbar_wait(tfull_bar(buf), (tile_it >> 1) & 1, a.status)) break;
             tcgen05_fence_after();
 #pragma unroll 1
@@ -568,33 +407,8 @@ dmr_status_t launch_prefill_t(const CUtensorMap &map_w, const CUtensorMap &map_x
     return launch(prefill_kernel<BITS, BN, false, false>);
 }
 
-int prefill_sm_count() {
-    static int cached = 0;
-    if (cached == 0) {
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
-            cached = n;
-        else
-            cached = 148;
-    }
-    return cached;
-}
-
-// Activation rows per tile.  A k block costs a CTA about the same time whatever the tile's width (hand-overs between the
-// roles, not MMA time, set the pace), so the wide tile does about twice the work per unit of time; the narrow one is
-// for batches it covers alone and for shapes whose last wave it fills much better.  Depends on (M, N) only.
-int prefill_bn(int M, int N, int sms) {
-    if (M <= 64) return 64;    // one tile of rows: the smaller the activation tile, the more stages are in flight
-    if (M <= 128) return 128;
-    const int n_tiles = (N + PM - 1) / PM;
-    auto score = [&](int bn, double rate) {
-        const long long t = (long long)n_tiles * ((M + bn - 1) / bn);
-        if (t < sms) return rate;  // fewer tiles than SMs: split along k fills the SMs (prefill_splits)
-        const long long waves = (t + sms - 1) / sms;
-        return rate * (double)t / (double)(waves * sms);
-    };
-    return score(256, 1.0) >= score(128, 0.7) ? 256 : 128;  // (measured: the narrow tile wins between 0.67 and 0.75)
-}
+// Activation rows per tile: the smaller the activation tile, the more stages are in flight.
+int prefill_bn(int M) { return M <= 64 ? 64 : 128; }
 
 }  // namespace
 
@@ -606,49 +420,44 @@ bool prefill_supported(int M, int N, int K, int bits, int g) {
     return M > 32 && (N + PM - 1) / PM >= 16;
 }
 
-// Split-K factor: for shapes whose tiles leave SMs idle.  As many splits as give every SM at most one work item, each
-// with at least sixteen k blocks; with more than one row tile the fp32 partial sums are large, and a split is taken only
-// if it shortens a work item by at least 48 k blocks.  Depends on (M, N, K) only.
+// Split-K factor: for layers whose tiles leave SMs idle.  As many splits as give every SM at most one work item, each
+// with at least sixteen k blocks.  Depends on (M, N, K) only.
 static int prefill_splits(int M, int N, int K, int sms, int *kb_per_split) {
-    const int bn = prefill_bn(M, N, sms);
-    const int nkb = K / PK, tiles = ((N + PM - 1) / PM) * ((M + bn - 1) / bn);
+    const int nkb = K / PK, bn = prefill_bn(M), tiles = (N + PM - 1) / PM * ((M + bn - 1) / bn);
     int splits = 1;
     if (tiles < sms) {
         splits = sms / tiles;
         if (splits > nkb / 16) splits = nkb / 16;  // a work item pays for its set-up (the feature's scale range) once
         if (splits < 1) splits = 1;
-        if (M > 128 && nkb - (nkb + splits - 1) / splits < 48) splits = 1;
     }
     *kb_per_split = (nkb + splits - 1) / splits;
     return (nkb + *kb_per_split - 1) / *kb_per_split;  // no empty split
 }
 
-size_t prefill_partial_bytes(int M, int N, int K) {
+size_t prefill_partial_bytes(int M, int N, int K, int bits, int g) {
+    if (pair_supported(M, N, K, bits, g)) return pair_plan(M, N, K, bits).partial_bytes;
     int kbps;
-    const int splits = prefill_splits(M, N, K, prefill_sm_count(), &kbps);
+    const int splits = prefill_splits(M, N, K, device_sm_count(), &kbps);
     return splits > 1 ? (size_t)splits * M * N * sizeof(float) : 0;
 }
 
 void prefill_plan(int M, int N, int K, int *bn, int *splits, long long *tiles, int *ctas) {
-    const int sms = prefill_sm_count();
+    const int sms = device_sm_count();
     int kbps;
-    *bn = prefill_bn(M, N, sms);
+    *bn = prefill_bn(M);
     *splits = prefill_splits(M, N, K, sms, &kbps);
     *tiles = (long long)((N + PM - 1) / PM) * ((M + *bn - 1) / *bn);
     const long long items = *tiles * *splits;
     *ctas = (int)(items < sms ? items : sms);
 }
 
-size_t prefill_scratch_bytes(int M, int K) { return round_up((size_t)M * K * 2, 256) + round_up((size_t)M * 4, 256); }
+// (32 entries more: the epilogue warps read the row scales in blocks of 32)
+size_t prefill_scratch_bytes(int M, int K) { return round_up((size_t)M * K * 2, 256) + round_up((size_t)M * 4 + 128, 256); }
 
 dmr_status_t launch_prefill(const uint16_t *X, int M, RowSel sel, const void *qweight, const uint16_t *scales,
                             const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out,
                             void *scratch, float *partial, int32_t *status, cudaStream_t st) {
-    const int sms = prefill_sm_count();
-    const int bn = prefill_bn(M, N, sms);
-    int kb_per_split;
-    const int splits = prefill_splits(M, N, K, sms, &kb_per_split);
-    if (splits > 1 && !partial) return DMR_ERR_WORKSPACE;
+    const int sms = device_sm_count();
     // activations: gather (routed calls), rescale each row by a power of two and convert to fp16
     uint16_t *Xh = reinterpret_cast<uint16_t *>(scratch);
     float *xscale = reinterpret_cast<float *>(reinterpret_cast<char *>(scratch) + round_up((size_t)M * K * 2, 256));
@@ -667,6 +476,11 @@ dmr_status_t launch_prefill(const uint16_t *X, int M, RowSel sel, const void *qw
         dmr_status_t r = check_launch();
         if (r != DMR_OK) return r;
     }
+    if (pair_supported(M, N, K, bits, g)) return launch_pair(Xh, M, sel, xscale, qweight, scales, zeros, N, K, bits, g, Y, out, partial, status, st);
+    const int bn = prefill_bn(M);
+    int kb_per_split;
+    const int splits = prefill_splits(M, N, K, sms, &kb_per_split);
+    if (splits > 1 && !partial) return DMR_ERR_WORKSPACE;
     CUtensorMap map_w, map_x;
     if (!make_tensor_map_2d(&map_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, Xh, (uint64_t)M, (uint64_t)K, (uint64_t)K * 2,
                             (uint32_t)bn, PK, TmaSwizzle::k128B))
@@ -701,7 +515,6 @@ dmr_status_t launch_prefill(const uint16_t *X, int M, RowSel sel, const void *qw
     dmr_status_t r;
     auto by_rows = [&](auto bits_tag) -> dmr_status_t {
         constexpr int B = decltype(bits_tag)::value;
-        if (bn == 256) return launch_prefill_t<B, 256>(map_w, map_x, a, grid, out, st);
         if (bn == 128) return launch_prefill_t<B, 128>(map_w, map_x, a, grid, out, st);
         return launch_prefill_t<B, 64>(map_w, map_x, a, grid, out, st);
     };
