@@ -48,12 +48,19 @@ struct PairCfg {
     static constexpr int STAGE = A_BYTES + B_BYTES + (BITS == 3 ? 0 : P_BYTES);
     static constexpr int S_RAW = (225 * 1024) / STAGE;
     static constexpr int S = BITS == 3 ? 6 : S_RAW > 8 ? 8 : S_RAW;
+    // Barriers the copies of the k blocks complete on, in turn.  Where a stage comes round to the unpack groups alternately there are two per
+    // stage, so that each is always waited for by the same group, phase after phase: a group that did not wait for the phase before takes
+    // a parity it waits for as already there.  (An even number of stages would do too: 8-bit, 32B layer, M = 500, 4 stages for 5: 381 us
+    // instead of 345; 3-bit, 7B layer, M = 1024, 4 for 6: 423 instead of 395.)
+    static constexpr int F = BITS == 8 || BITS == 3 ? 2 * S : S;
     static constexpr int RING = S * STAGE + (BITS == 3 ? S / 2 * P_BYTES : 0);
     static constexpr int UW = BITS == 0 ? 0 : 8;                        // unpack warps
     static constexpr int EW = 8;                                        // epilogue warps
     static constexpr int THREADS = 32 * (2 + UW + EW);
     static constexpr size_t SMEM = (size_t)RING + 1024 /*alignment*/ + 512 /*barriers*/;
     static_assert(SMEM <= 227 * 1024, "stages exceed an SM's shared memory");
+    static_assert(UW == 0 || F / (BITS == 3 ? 2 : 1) % (UW / 4) == 0, "a barrier belongs to one group of unpack warps");
+    static_assert(S <= 8 && F <= 32, "room for the barriers");
 };
 
 struct PairArgs {
@@ -118,7 +125,7 @@ template <int BITS, bool OUT_F32, bool SPLITK>
 __global__ void __launch_bounds__(PairCfg<BITS>::THREADS, 1)
 pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const PairArgs a) {
     using Cfg = PairCfg<BITS>;
-    constexpr int S = Cfg::S;
+    constexpr int S = Cfg::S, F = Cfg::F;
     extern __shared__ uint8_t smem_dyn[];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -132,7 +139,7 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
         return BITS == 3 ? base + (uint32_t)(S * Cfg::STAGE + s / 2 * Cfg::P_BYTES) : base + (uint32_t)s * Cfg::STAGE + Cfg::A_BYTES + Cfg::B_BYTES;
     };
     const uint32_t bar_base = base + (uint32_t)Cfg::RING;
-    auto full_bar = [&](int s) { return bar_base + 8u * s; };            // this CTA's copies of the stage have landed
+    auto full_bar = [&](int f) { return bar_base + 256u + 8u * f; };     // this CTA's copies have landed, k block it: f = it % F
     auto empty_bar = [&](int s) { return bar_base + 64u + 8u * s; };     // the MMAs have read the stage (both CTAs get it)
     auto ready_bar = [&](int s) { return bar_base + 128u + 8u * s; };    // first CTA: operands in place (codes: both CTAs; bf16: the second)
     auto tfull_bar = [&](int b) { return bar_base + 192u + 8u * b; };    // an accumulator is finished (both CTAs get it)
@@ -141,8 +148,8 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
     volatile uint32_t *tmem_slot_ptr = reinterpret_cast<volatile uint32_t *>(base_ptr + Cfg::RING + 224);
 
     if (threadIdx.x == 0) {
+        for (int f = 0; f < F; ++f) mbar_init(full_bar(f), 1);
         for (int s = 0; s < S; ++s) {
-            mbar_init(full_bar(s), 1);
             mbar_init(empty_bar(s), 1);
             mbar_init(ready_bar(s), BITS == 0 ? 1 : 8);  // codes: four unpack warps of each CTA
         }
@@ -191,10 +198,11 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
                         break;
                     }
                     const bool weights = BITS != 3 || (kb & 1) == 0;  // work items start at an even k block and have an even number of them
-                    mbar_expect_tx(full_bar(s), tx_x + (weights ? tx_w : 0u));
-                    tma_load_2d(b_tile(s), &map_x, full_bar(s), kb * kPk, m0);
-                    if constexpr (BITS == 0) tma_load_2d(a_tile(s), &map_w, full_bar(s), kb * kPk, n0);
-                    else if (weights) tma_load_2d(p_tile(s), &map_w, full_bar(s), BITS == 3 ? kb * (Cfg::P_ROW / 2) : kb * Cfg::P_ROW, n0);
+                    const uint32_t full = full_bar(it % F);
+                    mbar_expect_tx(full, tx_x + (weights ? tx_w : 0u));
+                    tma_load_2d(b_tile(s), &map_x, full, kb * kPk, m0);
+                    if constexpr (BITS == 0) tma_load_2d(a_tile(s), &map_w, full, kb * kPk, n0);
+                    else if (weights) tma_load_2d(p_tile(s), &map_w, full, BITS == 3 ? kb * (Cfg::P_ROW / 2) : kb * Cfg::P_ROW, n0);
                 }
             }
         }
@@ -281,7 +289,7 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
                     next = next_kb(kb);
                     row.take();
                     if (next < kb_hi) row.fetch(next, next / kb_per_group);
-                    if (!mbar_wait(full_bar(s), (it / S) & 1, a.status)) {
+                    if (!mbar_wait(full_bar(it % F), (it / F) & 1, a.status)) {
                         ok = false;
                         break;
                     }
