@@ -663,7 +663,7 @@ def run_extra_sections(sections, rank, dev, torch, dmr, inputs, fmt, peaks, l2_b
         # with the library's default dispatch (decode kernels up to 32 rows, tensor-core kernels above): where
         # the bandwidth-bound family hands over to the compute-bound one.  Two weight copies exceed 3 x L2 for INT8
         # (141 MB each) and come close for INT4 g64 (77 MB each; three copies are used).
-        cx = {"dispatch": f"DMR_DECODE_MAX_M={os.environ.get('DMR_DECODE_MAX_M', '32')}"}
+        cx = {"dispatch": f"DMR_DECODE_MAX_M={os.environ.get('DMR_DECODE_MAX_M', 'default')}"}
         summary = {}
         for lname, (N, K) in inputs.LAYER_32B.items():
             for fname, f5 in (("int4_g64", QF(4, 64)), ("int8_pc", QF(8, 0))):

@@ -111,8 +111,8 @@ dmr_status_t dmr_dequantize(const void *qweight, const void *scales, const void 
 
 /*
  * Low-precision linear layer (the W4A16 model's Linear, Sec. 5; also 8-bit and 3-bit codes): Y = X . dequant(Wq)^T
- * with fp32 accumulation.  Up to 32 rows run the bandwidth-bound decode kernels, larger M the tensor-core
- * kernels (3-bit codes: the persistent tensor-core kernel where it applies, otherwise the decode kernel, 16 rows per launch).  The decode kernels start fetching qweight, scales and zeros before the preceding kernel
+ * with fp32 accumulation.  Up to 16 rows of 3- and 4-bit codes run the decode kernels, larger batches and 8-bit codes the tensor-core
+ * kernels.  Kernels of up to 64 rows start fetching qweight, scales and zeros before the preceding kernel
  * of `stream` has finished (programmatic dependent launch): these three must be complete when the
  * call is enqueued, or be written by kernels that do not release their dependents early (dmr_quantize
  * and every ordinary kernel launch qualify).  X may be produced by the preceding kernel.
@@ -123,7 +123,8 @@ dmr_status_t dmr_lowbit_linear(const void *X_bf16, int M, const void *qweight, c
                                dmr_out_t out, void *workspace, size_t workspace_bytes,
                                void *stream);
 
-/* High-precision linear layer (the bf16 reference model, Sec. 5): Y = X . W^T, fp32 accumulation. */
+/* High-precision linear layer (the bf16 reference model, Sec. 5): Y = X . W^T, fp32 accumulation.  W is fetched ahead of the preceding
+ * kernel's end as the codes above are. */
 dmr_status_t dmr_dense_linear(const void *X_bf16, int M, const void *W_bf16, int N, int K, void *Y,
                               dmr_out_t out, void *workspace, size_t workspace_bytes, void *stream);
 
@@ -133,9 +134,9 @@ dmr_status_t dmr_dense_linear(const void *X_bf16, int M, const void *W_bf16, int
  * with the bf16 weights W, the others with the low-bit weights; every row's result is written
  * at its own index m, so Y is in step order.  The mask is read on the device only.  Row m equals,
  * bit for bit, row m of dmr_dense_linear (mask != 0) or dmr_lowbit_linear (mask == 0) called
- * on the same M rows.  The two halves run concurrently: the library forks a helper stream after the
- * partition and joins it back into `stream` before returning (also under stream capture).  The
- * helper stream and its two events are created by the first routed call on a device; make that
+ * on the same M rows.  The two halves run concurrently: in one launch where one kernel takes both (up to 64 rows, more than 16 or 8-bit
+ * codes), otherwise the library forks a helper stream after the partition and joins it back into `stream` before returning (also under stream capture).  The
+ * helper stream and its two events are created by the first such call on a device; make that
  * first call outside any capture.
  */
 dmr_status_t dmr_routed_linear(const void *X_bf16, int M, const uint8_t *mask, const void *W_bf16,

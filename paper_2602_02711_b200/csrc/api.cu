@@ -26,6 +26,7 @@ struct Scratch {
     uint16_t *xg_low = nullptr, *xg_high = nullptr;
     void *prefill_scratch = nullptr;  // prepared fp16 activations and row scales of the prefill kernel
     float *partial = nullptr;
+    int32_t *counters = nullptr, *counters_high = nullptr;  // small-batch kernel: shares of a tile that are done
     void *stream_scratch = nullptr;  // counters + partial sums of the streaming decode kernel
     uint16_t *xg_stream = nullptr;   // routed, decode path: the gathered activation rows of one chunk
     // routed calls run their two halves on two streams: the high-precision half gets its own scratch
@@ -36,18 +37,6 @@ struct Scratch {
 };
 
 constexpr int kStreamChunk = 32;  // rows one launch of the streaming decode kernel takes at most
-
-// Batches of up to this many rows stay on the streaming decode kernel (in chunks of 32 rows).  The
-// default is 32 (two chunks; measured faster than the tensor-core kernels up to there); the environment variable DMR_DECODE_MAX_M moves the crossover for measurements.
-int decode_max_m() {
-    static int v = -1;
-    if (v < 0) {
-        const char *e = getenv("DMR_DECODE_MAX_M");
-        const int x = e ? atoi(e) : 32;
-        v = x < 16 ? 16 : x;
-    }
-    return v;
-}
 
 // The warp-ring decode kernel takes the 4-bit decode batches unless the environment says DMR_DECODE_KERNEL=stream
 // (the shared-memory ring kernel, kept for 8-bit codes, bf16 weights and for comparison).
@@ -60,24 +49,48 @@ bool decode_w4_enabled() {
     return v != 0;
 }
 
-constexpr int kDecodeChunk = 16;  // rows one launch of the 4-bit decode kernel takes at most
+constexpr int kDecodeChunk = 16;  // rows one launch of the 3- and 4-bit decode kernels takes at most
 
-// Whether a call goes to the tensor-core kernels.  For 3-bit codes that family is the persistent prefill kernel alone
-// (no split-K kernel): batches it does not take stay on the decode kernel, 16 rows per launch.
-bool use_gemm(int M, int N, int K, int bits, int g) {
-    if (M <= decode_max_m()) return false;
-    if (bits == 3) return prefill_supported(M, N, K, bits, g);
-    return gemm_supported(M, N, K, bits, g);
+// Batches of up to this many rows stay on the decode kernels (in chunks); the environment variable DMR_DECODE_MAX_M moves the crossover
+// (to 16 rows or more, for all weights) for measurements.  Measured on the four linears of the 7B layer, us, decode kernels against small.cu's:
+// 4-bit codes 1 row 41 / 82, 16 rows 58 / 80, 17 rows 107 / 77, 32 rows 114 / 83; bf16 1 row 85.7 / 78, 3 rows 87.5 / 78.5, 16 rows
+// 95 / 87; 8-bit codes (32B layer) 1 row 85.7 / 65.6, 13 rows 112.5 / 67, 32 rows 146 / 77.  The kernels for 3- and 4-bit
+// codes multiply few rows in registers and need no hand-over between warps per unit of weights: they are the better ones as long as one
+// launch takes all rows.
+int decode_max_m(int bits) {
+    static int v = -1;
+    if (v < 0) {
+        const char *e = getenv("DMR_DECODE_MAX_M");
+        const int x = e ? atoi(e) : 0;
+        v = !e ? 0 : x < 16 ? 16 : x;
+    }
+    return v ? v : (bits == 3 || bits == 4) ? kDecodeChunk : 0;
+}
+
+// Which batches the small-batch tensor-core kernel takes (bits 0: bf16 weights), and which go to the one for large batches (a pair of SMs
+// per tile).  The latter rounds the weights of codes to fp16, the others multiply exact integers; narrow layers of up to 128 rows stay exact.
+// (65 to 128 rows on pairs of SMs, us, against tiles of one SM: bf16 M = 128 7B layer 135 -> 119, 14B layer 215 -> 164; 4-bit 7B layer
+// M = 128 148 -> 136; 8-bit 32B layer M = 65 191 -> 155; 3-bit 7B layer M = 128 174 -> 141.)
+bool use_small(int M, int N, int K, int bits, int g) { return M > decode_max_m(bits) && small_supported(M, N, K, bits, g); }
+bool use_pair(int M, int N, int K, int bits, int g) {
+    const bool exact = (bits == 4 || bits == 8) && M <= 128 && N <= kNarrow;
+    return M > decode_max_m(bits) && !exact && !use_small(M, N, K, bits, g) && pair_supported(M, N, K, bits, g);
 }
 
 Scratch carve(void *workspace, dmr_op_t op, int M, int N, int K, dmr_qformat_t f) {
     Scratch s;
     char *base = reinterpret_cast<char *>(workspace);
     size_t off = kWsStatusBytes;
+    // at a place of their own in every layout, so that no other call's scratch ever lies on them
+    s.counters = reinterpret_cast<int32_t *>(base + off);
+    s.counters_high = s.counters + kSmallMaxTiles;
+    off += 2 * (size_t)kSmallMaxTiles * sizeof(int32_t);
     s.status = reinterpret_cast<int32_t *>(base);
     const int g = format_ok(K, f) ? group_of(K, f) : K;
-    const bool low_gemm = op != DMR_OP_DENSE_LINEAR && use_gemm(M, N, K, f.bits, g);
-    const bool dense_gemm = op != DMR_OP_LOWBIT_LINEAR && use_gemm(M, N, K, 0, K);
+    const bool low_pair = op != DMR_OP_DENSE_LINEAR && use_pair(M, N, K, f.bits, g);
+    const bool dense_pair = op != DMR_OP_LOWBIT_LINEAR && use_pair(M, N, K, 0, K);
+    const bool low_small = op != DMR_OP_DENSE_LINEAR && format_ok(K, f) && use_small(M, N, K, f.bits, g);
+    const bool dense_small = op != DMR_OP_LOWBIT_LINEAR && use_small(M, N, K, 0, K);
     if (op == DMR_OP_ROUTED_LINEAR) {
         const size_t list = round_up((size_t)(M > 0 ? M : 1) * 4, 256);
         s.counts = reinterpret_cast<int32_t *>(base + off);
@@ -85,21 +98,21 @@ Scratch carve(void *workspace, dmr_op_t op, int M, int N, int K, dmr_qformat_t f
         s.idx_low = reinterpret_cast<int32_t *>(base + off + 256 + list);
         off += 256 + 2 * list;
         const size_t xg = round_up((size_t)M * K * 2, 256);
-        if (low_gemm) {
+        if (low_small) {
             s.xg_low = reinterpret_cast<uint16_t *>(base + off);
             off += xg;
         }
-        if (dense_gemm) {
+        if (dense_pair || dense_small) {
             s.xg_high = reinterpret_cast<uint16_t *>(base + off);
             off += xg;
         }
     }
-    if (low_gemm && prefill_supported(M, N, K, f.bits, g)) {
+    if (low_pair) {
         s.prefill_scratch = base + off;
         off += round_up(prefill_scratch_bytes(M, K), 256);
     }
-    const size_t partial_low = !low_gemm ? 0 : (prefill_supported(M, N, K, f.bits, g) ? prefill_partial_bytes(M, N, K, f.bits, g) : gemm_plan(M, N, K, f.bits).partial_bytes);
-    const size_t partial_dense = dense_gemm ? gemm_plan(M, N, K, 0).partial_bytes : 0;
+    const size_t partial_low = low_small ? small_plan(M, N, K).partial_bytes : low_pair ? pair_plan(M, N, K, f.bits).partial_bytes : 0;
+    const size_t partial_dense = dense_small ? small_plan(M, N, K).partial_bytes : dense_pair ? pair_plan(M, N, K, 0).partial_bytes : 0;
     if (op == DMR_OP_ROUTED_LINEAR) {
         if (partial_low) {
             s.partial = reinterpret_cast<float *>(base + off);
@@ -113,8 +126,8 @@ Scratch carve(void *workspace, dmr_op_t op, int M, int N, int K, dmr_qformat_t f
         s.partial = reinterpret_cast<float *>(base + off);
         off += round_up(partial_low > partial_dense ? partial_low : partial_dense, 256);
     }
-    const bool low_stream = op != DMR_OP_DENSE_LINEAR && !low_gemm;
-    const bool dense_stream = op != DMR_OP_LOWBIT_LINEAR && !dense_gemm;
+    const bool low_stream = op != DMR_OP_DENSE_LINEAR && !low_pair && !low_small;
+    const bool dense_stream = op != DMR_OP_LOWBIT_LINEAR && !dense_pair && !dense_small;
     if (low_stream || dense_stream) {
         s.stream_scratch = base + off;
         off += round_up(stream_scratch_bytes(N), 256);
@@ -147,17 +160,17 @@ dmr_status_t run_lowbit(const uint16_t *X, int M, RowSel sel, const uint32_t *qw
                         const Scratch &ws, cudaStream_t st) {
     const int g = group_of(K, f);
     const size_t ysz = out == DMR_OUT_F32 ? 4 : 2;
-    if (use_gemm(M, N, K, f.bits, g)) {
-        if (prefill_supported(M, N, K, f.bits, g))  // gathers the listed rows itself
-            return launch_prefill(X, M, sel, qweight, scales, zeros, N, K, f.bits, g, Y, out, ws.prefill_scratch, ws.partial, ws.status, st);
+    if (use_small(M, N, K, f.bits, g)) {
         const uint16_t *Xin = X;
         if (sel.idx) {
             dmr_status_t r = launch_gather_rows(X, K, M, sel.idx, sel.count, 0, ws.xg_low, st);
             if (r != DMR_OK) return r;
             Xin = ws.xg_low;
         }
-        return launch_gemm(Xin, M, sel, qweight, scales, zeros, N, K, f.bits, g, Y, out, ws.partial, ws.status, st);
+        return launch_small(Xin, M, sel, qweight, scales, zeros, N, K, f.bits, g, Y, out, ws.partial, ws.counters, ws.status, st);
     }
+    if (use_pair(M, N, K, f.bits, g))  // gathers the listed rows itself
+        return launch_prefill(X, M, sel, qweight, scales, zeros, N, K, f.bits, g, Y, out, ws.prefill_scratch, ws.partial, ws.status, st);
     const bool dec3 = f.bits == 3 && decode_w3_supported(M < kDecodeChunk ? M : kDecodeChunk, N, K, g);
     if (dec3 || (f.bits == 4 && decode_w4_enabled() && decode_w4_supported(M < kDecodeChunk ? M : kDecodeChunk, N, K, g))) {
         // chunks of up to 16 rows; the kernel gathers the rows of a routed call itself
@@ -208,14 +221,23 @@ dmr_status_t run_lowbit(const uint16_t *X, int M, RowSel sel, const uint32_t *qw
 dmr_status_t run_dense(const uint16_t *X, int M, RowSel sel, const uint16_t *W, int N, int K, void *Y,
                        dmr_out_t out, const Scratch &ws, cudaStream_t st) {
     const size_t ysz = out == DMR_OUT_F32 ? 4 : 2;
-    if (use_gemm(M, N, K, 0, K)) {
+    if (use_small(M, N, K, 0, K)) {
         const uint16_t *Xin = X;
         if (sel.idx) {
             dmr_status_t r = launch_gather_rows(X, K, M, sel.idx, sel.count, 0, ws.xg_high, st);
             if (r != DMR_OK) return r;
             Xin = ws.xg_high;
         }
-        return launch_gemm(Xin, M, sel, W, nullptr, nullptr, N, K, 0, K, Y, out, ws.partial, ws.status, st);
+        return launch_small(Xin, M, sel, W, nullptr, nullptr, N, K, 0, K, Y, out, ws.partial, ws.counters, ws.status, st);
+    }
+    if (use_pair(M, N, K, 0, K)) {
+        const uint16_t *Xin = X;
+        if (sel.idx) {
+            dmr_status_t r = launch_gather_rows(X, K, M, sel.idx, sel.count, 0, ws.xg_high, st);
+            if (r != DMR_OK) return r;
+            Xin = ws.xg_high;
+        }
+        return launch_pair(Xin, M, sel, nullptr, W, nullptr, nullptr, N, K, 0, K, Y, out, ws.partial, ws.status, st);
     }
     if (!stream_supported(M < kStreamChunk ? M : kStreamChunk, N, K, 16, K)) return launch_simple_dense(X, M, sel, W, N, K, Y, out, st);
     for (int m0 = 0; m0 < M; m0 += kStreamChunk) {
@@ -378,6 +400,15 @@ dmr_status_t dmr_routed_linear(const void *X_bf16, int M, const uint8_t *mask, c
     if (!aligned16(workspace)) return DMR_ERR_ALIGNMENT;
     cudaStream_t st = (cudaStream_t)stream;
     const Scratch ws = carve(workspace, DMR_OP_ROUTED_LINEAR, M, N, K, f);
+    if (use_small(M, N, K, 0, K) && use_small(M, N, K, f.bits, group_of(K, f))) {
+        // one launch for the split, one for both halves
+        r = launch_route_split(mask, M, reinterpret_cast<const uint16_t *>(X_bf16), K, ws.idx_high, ws.idx_low, ws.counts, ws.xg_high, ws.xg_low, st);
+        if (r != DMR_OK) return r;
+        const RowSel high = {ws.idx_high, ws.counts + 0, 0}, low = {ws.idx_low, ws.counts + 1, 0};
+        return launch_small_routed(ws.xg_high, ws.xg_low, M, high, low, reinterpret_cast<const uint16_t *>(W_bf16), qweight,
+                                   reinterpret_cast<const uint16_t *>(scales), reinterpret_cast<const uint8_t *>(zeros), N, K, f.bits, group_of(K, f), Y, out,
+                                   ws.partial_high, ws.partial, ws.counters_high, ws.counters, ws.status, st);
+    }
     std::lock_guard<std::mutex> routed_lock(g_routed_mutex);
     r = launch_route_partition(mask, M, ws.idx_high, ws.idx_low, ws.counts, st);
     if (r != DMR_OK) return r;
@@ -394,6 +425,7 @@ dmr_status_t dmr_routed_linear(const void *X_bf16, int M, const uint8_t *mask, c
     }
     Scratch wh = ws;
     wh.partial = ws.partial_high;
+    wh.counters = ws.counters_high;
     wh.stream_scratch = ws.stream_scratch_high;
     wh.xg_stream = ws.xg_stream_high;
     RowSel high = {ws.idx_high, ws.counts + 0, 0};
@@ -476,20 +508,18 @@ int dmr_describe_dispatch(dmr_op_t op, int M, int N, int K, dmr_qformat_t f, cha
     if (op != DMR_OP_LOWBIT_LINEAR && op != DMR_OP_DENSE_LINEAR) return -1;
     if (!dense && !format_ok(K, f)) return -1;
     const int bits = dense ? 0 : f.bits, g = dense ? K : group_of(K, f);
-    if (use_gemm(M, N, K, bits, g)) {
-        if (!dense && pair_supported(M, N, K, bits, g)) {  // tiles counted per CTA: 128 features each
-            const PairPlan p = pair_plan(M, N, K, bits);
-            return snprintf(buf, buf_bytes, "prefill bits=%d bn=256 rows=%d splits=%d tiles=%d ctas=%d", bits, p.rows, p.splits,
-                            (N + 127) / 128 * (p.tiles / p.n_tiles), p.ctas);
-        }
-        if (!dense && prefill_supported(M, N, K, bits, g)) {
-            int bn, splits, ctas;
-            long long tiles;
-            prefill_plan(M, N, K, &bn, &splits, &tiles, &ctas);
-            return snprintf(buf, buf_bytes, "prefill bits=%d bn=%d splits=%d tiles=%lld ctas=%d", bits, bn, splits, tiles, ctas);
-        }
-        const GemmPlan p = gemm_plan(M, N, K, bits);
-        return snprintf(buf, buf_bytes, "gemm bits=%d bn=%d splits=%d", bits, p.bn, p.splits);
+    if (use_pair(M, N, K, bits, g)) {  // tiles counted per CTA: 128 features each
+        const PairPlan p = pair_plan(M, N, K, bits);
+        return snprintf(buf, buf_bytes, "%s bits=%d bn=256 rows=%d splits=%d tiles=%d ctas=%d", dense ? "gemm" : "prefill", bits, p.rows, p.splits,
+                        (N + 127) / 128 * (p.tiles / p.n_tiles), p.ctas);
+    }
+    if (use_small(M, N, K, bits, g)) {
+        // the family a batch of this size belongs to; one kernel serves them all, one unit of 128 features x 128 inputs after the other
+        const SmallPlan p = small_plan(M, N, K);
+        if (!dense && M > 32) return snprintf(buf, buf_bytes, "prefill bits=%d bn=%d splits=1 tiles=%d ctas=%d", bits, p.bn, p.tiles, p.shares);
+        if (dense && M > 32) return snprintf(buf, buf_bytes, "gemm bits=0 bn=%d splits=1 tiles=%d ctas=%d", p.bn, p.tiles, p.shares);
+        if (!dense && bits != 8) return snprintf(buf, buf_bytes, "decode_w%d rows=%d tile=128 ctas=%d chunks=1", bits, p.bn, p.shares);
+        return snprintf(buf, buf_bytes, "stream bits=%d rows=%d steps=%d cluster=0 chunks=1", dense ? 16 : 8, p.bn, dense ? 2 * p.units : p.units);
     }
     if (!dense && bits == 3 && decode_w3_supported(M < kDecodeChunk ? M : kDecodeChunk, N, K, g)) {
         int nt, r, warps;

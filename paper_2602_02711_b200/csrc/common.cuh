@@ -106,21 +106,33 @@ dmr_status_t launch_decode_w3(const uint16_t *X, int M, RowSel sel, const uint32
 void decode_w4_plan(int M, int g, int *nt, int *r, int *warps);
 void decode_w3_plan(int M, int *nt, int *r, int *warps);
 void stream_plan(int M, int N, int K, int bits, int *tiles, long long *steps, int *cluster);
-void prefill_plan(int M, int N, int K, int *bn, int *splits, long long *tiles, int *ctas);
 
-// Low-bit linears on the tensor cores (M > 32; batches of more than 128 rows go on to launch_pair); sel.idx maps batch slots to rows of X and Y, sel.count
-// says how many slots are valid.
-bool prefill_supported(int M, int N, int K, int bits, int g);
-// X is the caller's activation matrix (for a routed call the rows sel.idx lists are gathered);
-// `scratch` holds prefill_scratch_bytes(M, K) bytes for the prepared fp16 activations and their row scales, `partial`
-// prefill_partial_bytes(M, N, K) bytes of fp32 partial sums (0 unless the call is split along k).
+// Low-bit linears of the sizes pair_supported() takes: the activations are prepared (for a routed call the rows sel.idx lists are
+// gathered), then launch_pair() runs.  `scratch` holds prefill_scratch_bytes(M, K) bytes for the prepared fp16 activations and their row
+// scales, `partial` pair_plan().partial_bytes.
 size_t prefill_scratch_bytes(int M, int K);
-size_t prefill_partial_bytes(int M, int N, int K, int bits, int g);
 dmr_status_t launch_prefill(const uint16_t *X, int M, RowSel sel, const void *qweight, const uint16_t *scales,
                             const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out,
                             void *scratch, float *partial, int32_t *status, cudaStream_t st);
 
-// Large batches (M > 128) on pairs of SMs: bf16 weights (bits == 0) and packed codes.  X is the bf16 matrix, or for codes the
+// Batches of up to 64 rows, and of up to 128 on layers of up to kNarrow features with 4- and 8-bit codes (bits == 0: bf16 weights).  X holds M rows (for a routed call: the gathered rows); `partial` holds
+// small_plan().partial_bytes, `counters` kSmallMaxTiles words that are zero before and after every call.
+constexpr int kSmallMaxTiles = 4096;
+constexpr int kNarrow = 15 * 128;  // k and v projections
+struct SmallPlan {
+    int bn, tiles, units, shares;
+    size_t partial_bytes;
+};
+bool small_supported(int M, int N, int K, int bits, int g);
+SmallPlan small_plan(int M, int N, int K);
+dmr_status_t launch_small(const uint16_t *X, int M, RowSel sel, const void *weights, const uint16_t *scales, const uint8_t *zeros, int N, int K,
+                          int bits, int g, void *Y, dmr_out_t out, float *partial, int32_t *counters, int32_t *status, cudaStream_t st);
+// Both halves of a routed call of up to 64 rows in one launch; Xh / Xl: the gathered rows.
+dmr_status_t launch_small_routed(const uint16_t *Xh, const uint16_t *Xl, int M, RowSel high, RowSel low, const uint16_t *W, const void *qweight,
+                                 const uint16_t *scales, const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out, float *partial_high,
+                                 float *partial_low, int32_t *counters_high, int32_t *counters_low, int32_t *status, cudaStream_t st);
+
+// Large batches (M > 32) on pairs of SMs: bf16 weights (bits == 0) and packed codes.  X is the bf16 matrix, or for codes the
 // prepared fp16 one with its row scales.
 struct PairPlan {
     int n_tiles, rows, splits, kb_per_split, tiles, ctas;
@@ -132,20 +144,6 @@ dmr_status_t launch_pair(const uint16_t *X, int M, RowSel sel, const float *xsca
                          const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out, float *partial, int32_t *status,
                          cudaStream_t st);
 
-// Tensor-core GEMM family (M > 16): tcgen05 MMA with TMA-staged operands.
-struct GemmPlan {
-    int bn;                 // activation rows per CTA (MMA N)
-    int splits;             // split-K factor (partials are added in split order)
-    int kblocks_per_split;  // 64-wide k blocks per split
-    size_t partial_bytes;   // fp32 partial-sum scratch needed (0 when splits == 1)
-};
-bool gemm_supported(int M, int N, int K, int bits /*0 = bf16 weights*/, int g);
-GemmPlan gemm_plan(int M, int N, int K, int bits);
-// `weights` is W (bits == 0) or qweight.  X holds M rows (for a routed call: the gathered rows,
-// sel.count of them valid); sel.idx maps batch slots to output rows.
-dmr_status_t launch_gemm(const uint16_t *X, int M, RowSel sel, const void *weights, const uint16_t *scales,
-                         const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out,
-                         float *partial, int32_t *status, cudaStream_t st);
 // Y[row(m)][n] = sum over z < splits of partial[z][m][n], in split order (fp32 partial sums by batch slot).
 dmr_status_t launch_splitk_reduce(const float *partial, int splits, int M, int N, RowSel sel, void *Y, dmr_out_t out,
                                   cudaStream_t st);
@@ -164,6 +162,9 @@ dmr_status_t launch_simple_dense(const uint16_t *X, int M, RowSel sel, const uin
 // Route partition.
 dmr_status_t launch_route_partition(const uint8_t *mask, int M, int32_t *idx_high, int32_t *idx_low,
                                     int32_t *counts, cudaStream_t st);
+// The same for up to 128 rows, with the rows themselves: Xh / Xl [M][K] receive the two halves' rows (slots past the counts stay as they are).
+dmr_status_t launch_route_split(const uint8_t *mask, int M, const uint16_t *X, int K, int32_t *idx_high, int32_t *idx_low, int32_t *counts,
+                                uint16_t *Xh, uint16_t *Xl, cudaStream_t st);
 
 // Step-wise KL divergence: kl_token[i] = KL(softmax(high[i]) || softmax(low[i])) for T rows of V logits
 // (bf16 or fp32), kl_step[s] = mean of kl_token over [offsets[s], offsets[s + 1]).

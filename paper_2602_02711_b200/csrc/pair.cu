@@ -421,8 +421,7 @@ dmr_status_t launch_pair_bits(const CUtensorMap &map_w, const CUtensorMap &map_x
 
 bool pair_supported(int M, int N, int K, int bits, int g) {
     (void)N;
-    // 3-bit codes: rows of whole 48-byte boxes (the others stay on the single-SM kernel)
-    if (M <= 128 || K % (bits == 3 ? 2 * kPk : kPk) != 0) return false;
+    if (M <= 32 || K % (bits == 3 ? 2 * kPk : kPk) != 0) return false;  // (3-bit codes: rows of whole 48-byte boxes)
     return bits == 0 || ((bits == 3 || bits == 4 || bits == 8) && g % kPk == 0 && K <= 32768);
 }
 

@@ -14,7 +14,7 @@ namespace dmr {
 // Host: 2-D tiled tensor maps.  The driver entry point is fetched through the runtime, so the
 // library does not link against libcuda.
 // ---------------------------------------------------------------------------------------------
-enum class TmaSwizzle { kNone, k128B };
+enum class TmaSwizzle { kNone, k64B, k128B };
 
 // rows x cols elements, row-major with `row_stride_bytes` between rows; box = box_rows x box_cols.
 // Out-of-range parts of a box read as zero.  Returns false (and records the error) on failure.

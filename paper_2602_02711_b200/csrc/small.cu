@@ -1,0 +1,750 @@
+// Linears of up to 64 rows on the tensor cores, bf16 weights and 3-, 4- and 8-bit codes: the weights are streamed once, in equal
+// shares over the SMs.
+//
+// What bounds it.  HBM, if everything else keeps out of the way: 128 features x 128 inputs are 8 KB of 4-bit codes (360 cycles of an
+// SM's share of the HBM rate) or 32 KB of bf16 (1430).  Turning codes into a shared-memory operand moves 32 KB in and out of shared
+// memory for them, 500 cycles of its bandwidth; so the unpacked weights go to TENSOR MEMORY (tcgen05.st) and the MMA
+// reads its first operand there.  What the codes become are the exact integers code - zero in bf16: no rounding, no
+// multiplication per weight, activations used as they are; a quantization group's sums are scaled once, in fp32, on their way out of the
+// accumulator (one fma per feature, row and group).
+// Measured (four linears of the 7B layer, us; in brackets the kernels that ran before, a streaming kernel up to 32 rows and tensor-core kernels
+// with unpacked tiles in shared memory above): 4-bit M = 17 77 (107), 32 83 (114), 64 96 (128); 3-bit M = 32 86 (116); bf16 M = 3 79 (88),
+// 16 87 (95), 64 106 (116); 8-bit, 32B layer, M = 1 66 (86), 13 67 (113), 64 92 (147).  A unit of codes still takes 700 to 900 cycles:
+// the chain of wait, unpack, store, MMA and commit of the units in flight, not the HBM rate.
+// Tried and dropped: one MMA warp (1380 cycles per unit); tiles of 128 rows for all layers (routed M = 128 402 against pair.cu's 375).
+//
+// Work split.  A unit is 128 features x 128 inputs; CTA c takes units [c U / n, (c + 1) U / n) of the U units, counted along k first: every SM
+// streams the same number of bytes, whatever the layer.  A 128-feature tile whose units belong to several CTAs is summed by the one
+// that finishes last: the others leave their fp32 sums in the workspace and count themselves; nobody waits.  The sums are added in
+// CTA order, so the result does not depend on who is last; the split depends on (N, K) only.
+//
+// Roles.  Unpack warps (codes only) in groups of four that take alternate units; scale warps, one per lane quadrant: group
+// sums from the accumulators into registers, at the end of a tile to memory; MMA warps, each with an accumulator of its own; one warp
+// of copies (weights run ahead of the preceding kernel's end, activations wait for it).  Every wait is bounded.
+#include <cuda_bf16.h>
+
+#include "sm100.cuh"
+
+namespace dmr {
+
+namespace {
+
+constexpr int kSm = 128;        // features per tile
+constexpr int kSk = 128;        // inputs per unit
+constexpr int kABufs = 4;       // unpacked units in tensor memory, 64 columns each
+constexpr int kMaxSums = 8;     // shared tiles of a CTA at most: two for each of its shares
+constexpr int kMinUnits = 8;    // units per CTA at least: below, the exchange costs more than the SMs bring (1024 x 5120, routed, M = 64, 14B layer: 4 / 8 / 12: 289 / 279 / 289 us)
+
+template <int BITS, int BN>  // BITS 0: bf16 weights
+struct SmallCfg {
+    static constexpr int W_ROW = BITS == 0 ? 256 : kSk * BITS / 8;   // bytes of a feature's weights in a unit
+    static constexpr int W_BYTES = kSm * W_ROW;
+    static constexpr int X_HALF = BN * 128;                            // activations of 64 inputs
+    static constexpr int STAGE = W_BYTES + 2 * X_HALF;
+    static constexpr int MW = BITS == 8 && BN < 64 ? 4 : 2;            // MMA warps
+    static constexpr int UW = BITS == 0 ? 0 : BITS == 8 && BN < 64 ? 16 : 8;  // unpack warps
+    // A stage, and an unpacked unit's buffer, come round to the same MMA warp and the same group of unpack warps every time: each
+    // barrier's phases are then waited for one after the other by whoever waits for them, and none is taken for the one after it.
+    static constexpr int TURN = UW / 4 > MW ? UW / 4 : MW;
+    static constexpr int S_RAW = (216 * 1024) / STAGE / TURN * TURN;
+    static constexpr int S = S_RAW > 16 ? 16 : S_RAW;
+    static constexpr int EW = BN == 128 ? 8 : 4;                       // scale warps, at most 64 rows of the batch each
+    // warps: unpack first, so that groups of four cover the lane quadrants, then scale, MMA, copies
+    static constexpr int THREADS = 32 * (UW + EW + MW + 1);
+    static constexpr size_t SMEM = (size_t)S * STAGE + 1024 /*alignment*/ + 1024 /*barriers*/;
+    static_assert(STAGE % 1024 == 0 && W_BYTES % 1024 == 0, "tiles on swizzle boundaries");
+    static_assert(S >= TURN && S % TURN == 0 && S % MW == 0 && (UW == 0 || (S % (UW / 4) == 0 && kABufs % (UW / 4) == 0)) && kABufs % MW == 0, "turns");
+};
+
+struct SmallArgs {
+    const uint16_t *scales;
+    const uint8_t *zeros;
+    void *Y;
+    const int32_t *idx, *count;  // routed: output row of batch slot m; valid slots (nullptr: identity, M)
+    float *partial;              // [share][2][BN][128]
+    int32_t *counters;           // [tiles], zero between calls
+    int32_t *status;
+    int M, N, K, G;
+    int g_units, half;           // units per quantization group; half: two groups per unit
+    uint32_t g_mul;              // group of a tile's unit k = k g_mul / 2^32 (0: k itself)
+    int units, k_units;          // in all; per tile
+    int shares;                  // the units are cut into this many equal shares; a CTA works through one or, in a routed call, two
+};
+
+__device__ __forceinline__ void tmem_st_x32(uint32_t taddr, const uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,"
+        "%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]),
+        "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
+        "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// D[tmem] (+)= A * B, bf16; A in tensor or shared memory, B in shared memory.  Descriptors as low words (the address field, which is all
+// that changes) and a high word that all of them share.
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc, bool add) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 b, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"((uint32_t)add)
+        : "memory");
+}
+__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, bool add) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 a, {%1, %3};\n\t"
+        "mov.b64 b, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"((uint32_t)add)
+        : "memory");
+}
+__device__ __forceinline__ uint4 lds_v4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+
+// Eight 4-bit codes -> the bf16 integers code - zero, in order (zz = 128 + zero, twice).
+__device__ __forceinline__ void ints_of_nibbles(uint32_t u, uint32_t zz, uint32_t *o) {
+    const uint32_t u4 = u >> 4;
+    const uint32_t d04 = bf16x2_sub(lop3_and_or(u, 0x000F000Fu, 0x43004300u), zz), d15 = bf16x2_sub(lop3_and_or(u4, 0x000F000Fu, 0x43004300u), zz);
+    const uint32_t d26 = bf16x2_sub(lop3_and_or(prmt(u, 0u, 0x4321), 0x000F000Fu, 0x43004300u), zz);
+    const uint32_t d37 = bf16x2_sub(lop3_and_or(prmt(u4, 0u, 0x4321), 0x000F000Fu, 0x43004300u), zz);
+    o[0] = prmt(d04, d15, 0x5410);
+    o[1] = prmt(d26, d37, 0x5410);
+    o[2] = prmt(d04, d15, 0x7632);
+    o[3] = prmt(d26, d37, 0x7632);
+}
+// Four 8-bit codes (zf = 2^23 + zero).
+__device__ __forceinline__ void ints_of_bytes(uint32_t u, float zf, uint32_t *o) {
+    float f[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) f[b] = __fsub_rn(__uint_as_float(prmt(u, 0x4B000000u, 0x7650u + (uint32_t)b)), zf);
+    o[0] = pack_bf16x2_rn(f[0], f[1]);  // exact: at most 255 in magnitude
+    o[1] = pack_bf16x2_rn(f[2], f[3]);
+}
+// Thirty-two 3-bit codes in three words: pair 5 j + i = codes (10 j + i, 10 j + 5 + i), pair 15 = codes (30, 31).
+__device__ __forceinline__ void ints_of_block3(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t zb, uint32_t *o) {
+    const uint32_t zz = (0x4300u | zb) * 0x00010001u;         // 128 + zero
+    const uint32_t z8 = (0xC180u | (zb << 3)) * 0x00010001u;  // -(16 + zero)
+    uint32_t D[16];
+    const uint32_t w[3] = {w0, w1, w2};
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const uint32_t u = w[j], u6 = u >> 6;
+        D[5 * j + 0] = bf16x2_sub(lop3_and_or(u, 0x00070007u, 0x43004300u), zz);
+        D[5 * j + 1] = bf16x2_fma(lop3_and_or(u, 0x00380038u, 0x43004300u), 0x3E003E00u, z8);  // (128 + 8 q) / 8 - (16 + zero)
+        D[5 * j + 2] = bf16x2_sub(lop3_and_or(u6, 0x00070007u, 0x43004300u), zz);
+        D[5 * j + 3] = bf16x2_fma(lop3_and_or(u6, 0x00380038u, 0x43004300u), 0x3E003E00u, z8);
+        D[5 * j + 4] = bf16x2_sub(lop3_and_or(u >> 12, 0x00070007u, 0x43004300u), zz);
+    }
+    uint32_t t = lop3_and_or(w0 >> 15, 0x00010001u, 0x43004300u);
+    t = lop3_and_or(w1 >> 14, 0x00020002u, t);
+    t = lop3_and_or(w2 >> 13, 0x00040004u, t);
+    D[15] = bf16x2_sub(t, zz);
+    auto pair_of = [](int a) { return a >= 30 ? 15 : 5 * (a / 10) + (a % 10) % 5; };
+    auto high_of = [](int a) { return a >= 30 ? a - 30 : ((a % 10) >= 5 ? 1 : 0); };
+#pragma unroll
+    for (int v = 0; v < 16; ++v)
+        o[v] = prmt(D[pair_of(2 * v)], D[pair_of(2 * v + 1)], (high_of(2 * v + 1) ? 0x7600u : 0x5400u) | (high_of(2 * v) ? 0x32u : 0x10u));
+}
+
+// CTA `cta` of the `ctas` that work on one linear.
+template <int BITS, int BN, bool OUT_F32>
+__device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUtensorMap &map_x, const SmallArgs &a, uint32_t tmem_base, int cta, int ctas) {
+    using Cfg = SmallCfg<BITS, BN>;
+    constexpr int S = Cfg::S, MW = Cfg::MW;
+    constexpr int W_SCALE = Cfg::UW, W_MMA = Cfg::UW + Cfg::EW, W_COPY = W_MMA + MW;  // first warp of each role
+    extern __shared__ uint8_t smem_dyn[];
+    __shared__ int sum_tile[kMaxSums], to_sum;  // shared tiles that this CTA finished last
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    auto w_tile = [&](int s) { return base + (uint32_t)s * Cfg::STAGE; };
+    auto x_tile = [&](int s, int h) { return base + (uint32_t)s * Cfg::STAGE + Cfg::W_BYTES + (uint32_t)h * Cfg::X_HALF; };
+    const uint32_t bar_base = base + (uint32_t)S * Cfg::STAGE;
+    auto wfull_bar = [&](int s) { return bar_base + 8u * s; };              // weights of a unit have landed
+    auto xfull_bar = [&](int s) { return bar_base + 128u + 8u * s; };       // activations of a unit have landed
+    auto done_bar = [&](int s) { return bar_base + 256u + 8u * s; };        // the unit's MMAs have completed: its stage is free
+    auto afull_bar = [&](int i) { return bar_base + 384u + 8u * i; };       // an unpacked unit is in tensor memory, its activations have landed
+    auto tempty_bar = [&](int i) { return bar_base + 448u + 8u * i; };      // the scale warps have read MMA warp i's accumulator
+    auto tfull_bar = [&](int i) { return bar_base + 480u + 8u * i; };       // MMA warp i is through with its units of a longer group
+
+    auto first_unit = [&](int share) { return (int)((uint32_t)a.units * (uint32_t)share / (uint32_t)a.shares); };  // (units x shares fit in 32 bits)
+    // the shares that have units of a tile, and where their sums of it are kept: a share's first tile uses its first slot
+    auto sharers = [&](int tile, int &c_first, int &c_last) {
+        auto owner = [&](int unit) { return (int)((((uint32_t)unit + 1) * (uint32_t)a.shares - 1) / (uint32_t)a.units); };
+        c_first = owner(tile * a.k_units);
+        c_last = owner(tile * a.k_units + a.k_units - 1);
+    };
+    auto slot_of = [&](int tile, int c) -> float * {
+        return a.partial + ((size_t)c * 2 + (first_unit(c) >= tile * a.k_units ? 0 : 1)) * (size_t)(BN * kSm);
+    };
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(wfull_bar(s), 1);
+            mbar_init(xfull_bar(s), 1);
+            mbar_init(done_bar(s), 1);
+        }
+        for (int i = 0; i < kABufs; ++i) mbar_init(afull_bar(i), 4);
+        for (int i = 0; i < 4; ++i) {
+            mbar_init(tempty_bar(i), Cfg::EW);
+            mbar_init(tfull_bar(i), 1);
+        }
+        to_sum = 0;
+        fence_barrier_init();
+        prefetch_tensor_map(&map_w);
+        prefetch_tensor_map(&map_x);
+    }
+    __syncthreads();
+    const uint32_t tmem_a = tmem_base + 256;  // columns 0 .. 255: the accumulators
+    auto copy_w = [&](int s, int tile, int ku) {
+        mbar_expect_tx(wfull_bar(s), Cfg::W_BYTES);
+        if constexpr (BITS == 0) {
+            tma_load_2d(w_tile(s), &map_w, wfull_bar(s), ku * kSk, tile * kSm);
+            tma_load_2d(w_tile(s) + Cfg::W_BYTES / 2, &map_w, wfull_bar(s), ku * kSk + 64, tile * kSm);
+        } else {
+            tma_load_2d(w_tile(s), &map_w, wfull_bar(s), ku * Cfg::W_ROW, tile * kSm);
+        }
+    };
+    auto group_of = [&](int ku) -> int { return a.g_mul ? (int)__umulhi((uint32_t)ku, a.g_mul) : ku; };
+    // Unit i of the CTA's share belongs to MMA warp and accumulator i % nd.  A quantization group that ends with its unit is read when the unit
+    // is done; a longer one (or a tile of bf16 weights) when all warps are through with their units of it, their accumulators added in order; a
+    // group of half a unit has an accumulator of its own beside the other half's.
+    const bool half_groups = BITS != 0 && a.half, long_groups = BITS == 0 || a.g_units > 1;
+    const int nd = half_groups && BN >= 64 ? 128 / BN : MW;
+    const uint32_t d_cols = 256u / (uint32_t)nd, half_cols = d_cols / 2;
+    // this CTA's shares and units (consecutive ones), and the first unit's tile and place in it
+    const int share_lo = (int)((uint32_t)a.shares * (uint32_t)cta / (uint32_t)ctas), share_hi = (int)((uint32_t)a.shares * (uint32_t)(cta + 1) / (uint32_t)ctas);
+    const int lo = first_unit(share_lo), hi = first_unit(share_hi);
+    const int lo_tile = lo / a.k_units, lo_ku = lo - lo_tile * a.k_units;
+
+    // the first weights run ahead of the preceding kernel's end, in a routed call ahead of the number of rows as well
+    const int first = min(hi - lo, S);
+    if (warp == W_COPY && lane == 0) {
+        for (int i = 0; i < first; ++i) {
+            const int u = lo + i, tile = u / a.k_units;
+            copy_w(i, tile, u - tile * a.k_units);
+        }
+    }
+    __syncwarp();
+    int rows = a.M;
+    if (a.count) {
+        pdl_wait();
+        rows = min(*a.count, a.M);
+    }
+    const bool work = rows > 0;
+
+    if (warp == W_COPY) {
+        // ================= copies =================
+        if (lane == 0) {
+            int issued = first, x_issued = 0;
+            if (work) {
+                int tile = (lo + first) / a.k_units, ku = lo + first - tile * a.k_units, xku = lo_ku;  // the next unit's weights, and activations
+                auto copy_x = [&](int s) {
+                    mbar_expect_tx(xfull_bar(s), 2 * Cfg::X_HALF);
+                    tma_load_2d(x_tile(s, 0), &map_x, xfull_bar(s), xku * kSk, 0);
+                    tma_load_2d(x_tile(s, 1), &map_x, xfull_bar(s), xku * kSk + 64, 0);
+                    if (++xku == a.k_units) xku = 0;
+                };
+                pdl_wait();
+                for (int i = 0; i < first; ++i) copy_x(i);
+                for (int u = lo + first, s = 0, par = 0; u < hi; ++u) {
+                    if (!mbar_wait(done_bar(s), (uint32_t)par, a.status)) break;
+                    copy_w(s, tile, ku);
+                    if (++ku == a.k_units) {
+                        ku = 0;
+                        ++tile;
+                    }
+                    copy_x(s);
+                    if (++s == S) {
+                        s = 0;
+                        par ^= 1;
+                    }
+                    issued = u + 1 - lo;
+                }
+                x_issued = issued;
+            }
+            // no copy is left in flight, even where a wait has run out
+            for (int i = max(0, issued - S); i < issued; ++i) {
+                (void)mbar_wait(wfull_bar(i % S), (uint32_t)((i / S) & 1), a.status);
+                if (i < x_issued) (void)mbar_wait(xfull_bar(i % S), (uint32_t)((i / S) & 1), a.status);
+            }
+        }
+        __syncwarp();
+    } else if (warp >= W_MMA && warp < W_COPY) {
+        // ================= MMAs =================
+        // Several warps, because a unit's eight small MMAs take 370 cycles but waiting for operands, issuing and committing take one warp
+        // about 1400, most of it latency.
+        const int w = warp - W_MMA;
+        if (work && w < nd) {
+            constexpr uint32_t IDESC = umma_idesc_bf16(kSm, BN);
+            const uint32_t desc_x0 = (uint32_t)umma_desc_sw128(x_tile(0, 0)), desc_w0 = (uint32_t)umma_desc_sw128(w_tile(0));
+            const uint32_t desc_hi = (uint32_t)(umma_desc_sw128(0) >> 32);
+            const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+            const uint32_t d0 = tmem_u + (uint32_t)w * d_cols, d1 = half_groups ? d0 + half_cols : d0;
+            // the warp's current run - units of one quantization group and one share - ends before unit `end`
+            int share = share_lo, share_end = first_unit(share_lo + 1), end = 0;
+            auto run_end = [&](int u) {
+                while (share_end <= u) share_end = first_unit(++share + 1);
+                return a.g_units == 1 ? u + 1 : min((u / a.g_units + 1) * a.g_units, share_end);
+            };
+            int starts = 0, last = -1;
+            for (int i = w; lo + i < hi; i += nd) {
+                const int s = i % S, ab = i % kABufs;
+                const uint32_t par = (uint32_t)((i / S) & 1);
+                if (BITS == 0) {
+                    if (!mbar_wait(xfull_bar(s), par, a.status) || !mbar_wait(wfull_bar(s), par, a.status)) break;
+                } else if (!mbar_wait(afull_bar(ab), (uint32_t)((i / kABufs) & 1), a.status)) {
+                    break;
+                }
+                const bool start = lo + i >= end;
+                if (start) {
+                    end = run_end(lo + i);
+                    if (starts > 0 && !mbar_wait(tempty_bar(w), (uint32_t)((starts - 1) & 1), a.status)) break;
+                    ++starts;
+                }
+                tcgen05_fence_after();
+                const uint32_t off = ((uint32_t)s * (uint32_t)Cfg::STAGE) >> 4;
+                const uint32_t dx = desc_x0 + off, dw = desc_w0 + off, ta = tmem_u + 256u + (uint32_t)(ab * 64);
+                if (lane == 0) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const uint32_t jx = (uint32_t)((j >> 2) * (Cfg::X_HALF >> 4) + 2 * (j & 3)), jw = (uint32_t)((j >> 2) * (Cfg::W_BYTES >> 5) + 2 * (j & 3));
+                        const bool add = j == 0 ? !start : j == 4 ? !half_groups : true;
+                        if constexpr (BITS == 0) umma_ss(j < 4 ? d0 : d1, dw + jw, dx + jx, desc_hi, IDESC, add);
+                        else umma_ts(j < 4 ? d0 : d1, ta + (uint32_t)(8 * j), dx + jx, desc_hi, IDESC, add);
+                    }
+                    umma_commit(done_bar(s));
+                    if (long_groups && lo + i + nd >= end) umma_commit(tfull_bar(w));  // this warp's last unit of the run
+                }
+                __syncwarp();
+                last = i;
+            }
+            if (last >= 0) (void)mbar_wait(done_bar(last % S), (uint32_t)((last / S) & 1), a.status);  // no MMA is left in flight
+        }
+        __syncwarp();
+    } else if (warp < Cfg::UW) {
+        if constexpr (BITS != 0) {
+            // ================= unpack: codes -> integers in tensor memory =================
+            if (work) {
+                constexpr int NG = Cfg::UW / 4;
+                const int q = warp & 3, r = q * 32 + lane, grp = warp >> 2;
+                const uint32_t dst0 = tmem_a + ((uint32_t)(q * 32) << 16);
+                // the next unit of this group of warps: tile and unit within the tile, and its zero points (both halves)
+                int tile = lo_tile, ku = lo_ku;
+                auto skip = [&](int n) {
+                    ku += n;
+                    while (ku >= a.k_units) {
+                        ku -= a.k_units;
+                        ++tile;
+                    }
+                };
+                auto zeros_of = [&](uint32_t &z0, uint32_t &z1) {
+                    const uint8_t *zp = a.zeros + (size_t)min(tile * kSm + r, a.N - 1) * a.G;
+                    if (half_groups) {
+                        z0 = __ldg(zp + 2 * ku);
+                        z1 = __ldg(zp + min(2 * ku + 1, a.G - 1));
+                    } else {
+                        z0 = z1 = __ldg(zp + group_of(ku));
+                    }
+                };
+                skip(grp);
+                uint32_t z0 = 0, z1 = 0;
+                if (lo + grp < hi) zeros_of(z0, z1);
+                for (int i = grp; lo + i < hi; i += NG) {
+                    const int s = i % S, ab = i % kABufs;
+                    const uint32_t zc[2] = {z0, z1};
+                    skip(NG);
+                    if (lo + i + NG < hi) zeros_of(z0, z1);
+                    if (!mbar_wait(wfull_bar(s), (uint32_t)((i / S) & 1), a.status)) break;
+                    const uint32_t src = w_tile(s) + (uint32_t)(r * Cfg::W_ROW);
+                    bool ok = true;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t v[32];
+                        if constexpr (BITS == 4) {
+                            const uint32_t zz = (0x4300u | zc[h]) * 0x00010001u;
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) {  // 64-byte swizzle: 16-byte piece p of row r sits at p ^ (r / 2 % 4)
+                                const uint4 w = lds_v4(src + ((((uint32_t)(2 * h + c)) ^ ((uint32_t)(r >> 1) & 3u)) << 4));
+                                ints_of_nibbles(w.x, zz, &v[16 * c]);
+                                ints_of_nibbles(w.y, zz, &v[16 * c + 4]);
+                                ints_of_nibbles(w.z, zz, &v[16 * c + 8]);
+                                ints_of_nibbles(w.w, zz, &v[16 * c + 12]);
+                            }
+                        } else if constexpr (BITS == 8) {
+                            const float zf = __uint_as_float(0x4B000000u | zc[h]);
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {  // 128-byte swizzle
+                                const uint4 w = lds_v4(src + ((((uint32_t)(4 * h + c)) ^ ((uint32_t)r & 7u)) << 4));
+                                ints_of_bytes(w.x, zf, &v[8 * c]);
+                                ints_of_bytes(w.y, zf, &v[8 * c + 2]);
+                                ints_of_bytes(w.z, zf, &v[8 * c + 4]);
+                                ints_of_bytes(w.w, zf, &v[8 * c + 6]);
+                            }
+                        } else {
+                            uint32_t w[6];
+                            asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "r"(src + 24 * h));
+                            asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(w[2]), "=r"(w[3]) : "r"(src + 24 * h + 8));
+                            asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(w[4]), "=r"(w[5]) : "r"(src + 24 * h + 16));
+                            ints_of_block3(w[0], w[1], w[2], zc[h], &v[0]);
+                            ints_of_block3(w[3], w[4], w[5], zc[h], &v[16]);
+                        }
+                        if (h == 0) {  // the buffer's unit before has been read by the MMAs
+                            const int j = i - kABufs;
+                            if (j >= 0 && !(ok = mbar_wait(done_bar(j % S), (uint32_t)((j / S) & 1), a.status))) break;
+                            tcgen05_fence_after();
+                        }
+                        tmem_st_x32(dst0 + (uint32_t)(ab * 64 + h * 32), v);
+                    }
+                    if (!ok) break;
+                    tmem_st_wait();
+                    tcgen05_fence_before();
+                    if (!mbar_wait(xfull_bar(s), (uint32_t)((i / S) & 1), a.status)) break;  // so that the MMA warp has one barrier to wait on
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(afull_bar(ab));
+                }
+            }
+            __syncwarp();
+        }
+    } else if (warp < W_MMA) {
+        // ================= group sums, outputs =================
+        const int q = warp & 3, r = q * 32 + lane;
+        constexpr int CW = BN < 64 ? BN : 64;
+        const int m_lo = Cfg::EW == 4 ? 0 : ((warp - W_SCALE) >> 2) * CW;  // this warp's rows of the batch: m_lo .. m_lo + CW - 1
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)m_lo;
+        bool ok = true;
+        if (work) pdl_wait();  // outputs and partial sums may still be in use by the kernel before
+        int i = 0;  // units done
+        uint32_t phases = 0;  // bit w: phase of tfull w
+        int tile = lo_tile, ku = lo_ku, share = share_lo, share_end = first_unit(share_lo + 1);
+        for (int u = work ? lo : hi; u < hi;) {
+            while (share_end <= u) share_end = first_unit(++share + 1);
+            const int n = tile * kSm + r, nc = min(n, a.N - 1);
+            const int mine = min(share_end - u, a.k_units - ku), ku_end = ku + mine;  // the share's units of the tile
+            float acc[CW];
+#pragma unroll
+            for (int c = 0; c < CW; ++c) acc[c] = 0.f;
+            const uint16_t *sp = a.scales + (size_t)nc * a.G;
+            int grp = group_of(ku), left = a.g_units - (ku - grp * a.g_units);  // group, and units left in it
+            uint32_t sb0 = 0, sb1 = 0;
+            auto scale_of = [&](int k, int g) {
+                if (BITS == 0) return;
+                if (half_groups) {
+                    sb0 = __ldg(sp + 2 * k);
+                    sb1 = __ldg(sp + min(2 * k + 1, a.G - 1));
+                } else {
+                    sb0 = __ldg(sp + g);
+                }
+            };
+            scale_of(ku, grp);
+            while (ku < ku_end) {
+                const int run = min(left, ku_end - ku);
+                const float sc0 = __uint_as_float(sb0 << 16), sc1 = __uint_as_float(sb1 << 16);
+                ku += run;
+                ++grp;
+                left = a.g_units;
+                if (ku < ku_end) scale_of(ku, grp);  // of the next group
+                const int parts = min(run, nd);  // one accumulator per MMA warp that has units of the group
+                for (int j = i + run - parts; j < i + run; ++j) {
+                    const int w = j % nd;
+                    if (long_groups) {
+                        ok = mbar_wait(tfull_bar(w), (phases >> w) & 1u, a.status);
+                        phases ^= 1u << w;
+                    } else {
+                        ok = mbar_wait(done_bar(j % S), (uint32_t)((j / S) & 1), a.status);
+                    }
+                    if (!ok) break;
+                    tcgen05_fence_after();
+#pragma unroll
+                    for (int c0 = 0; c0 < CW; c0 += 16) {
+                        uint32_t v[16];
+                        tmem_ld_x16(lane_addr + (uint32_t)w * d_cols + (uint32_t)c0, v);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) acc[c0 + c] = BITS == 0 ? acc[c0 + c] + __uint_as_float(v[c]) : fmaf(sc0, __uint_as_float(v[c]), acc[c0 + c]);
+                    }
+                    if (half_groups) {
+#pragma unroll
+                        for (int c0 = 0; c0 < CW; c0 += 16) {
+                            uint32_t v[16];
+                            tmem_ld_x16(lane_addr + (uint32_t)w * d_cols + half_cols + (uint32_t)c0, v);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) acc[c0 + c] = fmaf(sc1, __uint_as_float(v[c]), acc[c0 + c]);
+                        }
+                    }
+                    tcgen05_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tempty_bar(w));
+                }
+                if (!ok) break;
+                i += run;
+            }
+            if (!ok) break;
+            if (mine < a.k_units) {
+                // one of several shares that have units of this tile
+                int c_first, c_last;
+                sharers(tile, c_first, c_last);
+                float *part = slot_of(tile, share) + r;
+#pragma unroll
+                for (int c = 0; c < CW; ++c)
+                    if (m_lo + c < rows) __stcg(part + (m_lo + c) * kSm, acc[c]);
+                __threadfence();
+                asm volatile("bar.sync 1, %0;" ::"n"(Cfg::EW * 32) : "memory");
+                if (warp == W_SCALE && lane == 0) {
+                    const bool last = atomicAdd(a.counters + tile, 1) == c_last - c_first;
+                    __threadfence();
+                    if (last) {
+                        a.counters[tile] = 0;
+                        if (to_sum < kMaxSums) sum_tile[to_sum++] = tile;
+                    }
+                }
+            } else if (n < a.N) {
+#pragma unroll
+                for (int c = 0; c < CW; ++c) {
+                    if (m_lo + c < rows) {
+                        const size_t at = (size_t)(a.idx ? a.idx[m_lo + c] : m_lo + c) * a.N + n;
+                        if (OUT_F32) reinterpret_cast<float *>(a.Y)[at] = acc[c];
+                        else reinterpret_cast<__nv_bfloat16 *>(a.Y)[at] = __float2bfloat16_rn(acc[c]);
+                    }
+                }
+            }
+            u += mine;
+            if (ku == a.k_units) {
+                ku = 0;
+                ++tile;
+            }
+        }
+        __syncwarp();
+    }
+
+    // every role's loop is bounded, and none leaves a copy or an MMA in flight
+    tcgen05_fence_before();
+    __syncthreads();
+    tcgen05_fence_after();
+
+    // The shared tiles that this CTA was the last one to finish, with all its warps: a warp for a few rows, four features per lane, several
+    // CTAs' sums requested at once.  (By the scale warps alone, at the time, it took 0.76 us per CTA of a tile of 64 rows: routed 14B layer, M = 64, 311 us instead of 279.)
+    constexpr int RW = BN >= 64 ? 4 : BN / 16, CU = BN >= 64 ? 4 : 8;  // rows of a warp, and CTAs, at a time
+    for (int e = 0; e < to_sum; ++e) {
+        const int tile = sum_tile[e], n4 = tile * kSm + 4 * lane;
+        int c_first, c_last;
+        sharers(tile, c_first, c_last);
+#pragma unroll 1
+        for (int m0 = warp * RW; m0 < rows; m0 += (int)(blockDim.x >> 5) * RW) {
+            float4 sum[RW];
+#pragma unroll
+            for (int r = 0; r < RW; ++r) sum[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+            for (int c0 = c_first; c0 <= c_last; c0 += CU) {
+                float4 v[CU][RW];
+#pragma unroll
+                for (int c = 0; c < CU; ++c) {
+                    const float4 *p = reinterpret_cast<const float4 *>(slot_of(tile, c0 + c) + (size_t)m0 * kSm) + lane;
+#pragma unroll
+                    for (int r = 0; r < RW; ++r) v[c][r] = c0 + c <= c_last && m0 + r < rows ? __ldcg(p + r * (kSm / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int c = 0; c < CU; ++c) {
+#pragma unroll
+                    for (int r = 0; r < RW; ++r) {
+                        sum[r].x += v[c][r].x;
+                        sum[r].y += v[c][r].y;
+                        sum[r].z += v[c][r].z;
+                        sum[r].w += v[c][r].w;
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                if (m0 + r >= rows) break;
+                const size_t at = (size_t)(a.idx ? a.idx[m0 + r] : m0 + r) * a.N + n4;
+                const float f[4] = {sum[r].x, sum[r].y, sum[r].z, sum[r].w};
+                if (a.N % 4 == 0 && n4 < a.N) {
+                    if (OUT_F32) *reinterpret_cast<float4 *>(reinterpret_cast<float *>(a.Y) + at) = sum[r];
+                    else *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(a.Y) + at) = make_uint2(pack_bf16x2_rn(f[0], f[1]), pack_bf16x2_rn(f[2], f[3]));
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (n4 + i < a.N) {
+                            if (OUT_F32) reinterpret_cast<float *>(a.Y)[at + i] = f[i];
+                            else reinterpret_cast<__nv_bfloat16 *>(a.Y)[at + i] = __float2bfloat16_rn(f[i]);
+                        }
+                }
+            }
+        }
+    }
+}
+
+__device__ __forceinline__ uint32_t small_begin(uint32_t *slot) {
+    if (threadIdx.x < 32) {
+        tmem_alloc(smem_u32(slot), 512);
+        tmem_relinquish();
+    }
+    tcgen05_fence_before();
+    __syncthreads();
+    tcgen05_fence_after();
+    pdl_launch_dependents();
+    return *reinterpret_cast<volatile uint32_t *>(slot);
+}
+
+template <int BITS, int BN, bool OUT_F32>
+__global__ void __launch_bounds__(SmallCfg<BITS, BN>::THREADS, 1)
+small_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const SmallArgs a) {
+    __shared__ uint32_t slot;
+    const uint32_t tmem = small_begin(&slot);
+    small_body<BITS, BN, OUT_F32>(map_w, map_x, a, tmem, (int)blockIdx.x, (int)gridDim.x);
+    if (threadIdx.x < 32) tmem_dealloc(tmem, 512);
+}
+
+// Both halves of a routed call in one launch: the first n_dense CTAs work on the bf16 weights, the others on the codes.  The shares, and with
+// them every sum, are those of the two calls by themselves.
+template <int BITS, int BN, bool OUT_F32>
+__global__ void __launch_bounds__(SmallCfg<BITS, BN>::THREADS, 1)
+small_routed_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_xh, const SmallArgs dense,
+                    const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_xl, const SmallArgs low, int n_dense) {
+    __shared__ uint32_t slot;
+    const uint32_t tmem = small_begin(&slot);
+    if ((int)blockIdx.x < n_dense) small_body<0, BN, OUT_F32>(map_w, map_xh, dense, tmem, (int)blockIdx.x, n_dense);  // (its spare warps idle)
+    else small_body<BITS, BN, OUT_F32>(map_q, map_xl, low, tmem, (int)blockIdx.x - n_dense, (int)gridDim.x - n_dense);
+    if (threadIdx.x < 32) tmem_dealloc(tmem, 512);
+}
+
+int small_bn(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 128; }
+
+template <int BITS, int BN>
+dmr_status_t launch_small_t(const CUtensorMap &map_w, const CUtensorMap &map_x, const SmallArgs &a, int ctas, dmr_out_t out, cudaStream_t st) {
+    using Cfg = SmallCfg<BITS, BN>;
+    auto kernel = out == DMR_OUT_F32 ? small_kernel<BITS, BN, true> : small_kernel<BITS, BN, false>;
+    if (!ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), Cfg::SMEM)) return DMR_ERR_CUDA;
+    const cudaError_t e = launch_pdl(kernel, dim3((unsigned)ctas), dim3(Cfg::THREADS), Cfg::SMEM, st, map_w, map_x, a);
+    if (e != cudaSuccess) return launch_failed(e);
+    return check_launch();
+}
+
+template <int BITS>
+dmr_status_t launch_small_bits(int bn, const CUtensorMap &map_w, const CUtensorMap &map_x, const SmallArgs &a, int ctas, dmr_out_t out, cudaStream_t st) {
+    switch (bn) {
+        case 16: return launch_small_t<BITS, 16>(map_w, map_x, a, ctas, out, st);
+        case 32: return launch_small_t<BITS, 32>(map_w, map_x, a, ctas, out, st);
+        case 64: return launch_small_t<BITS, 64>(map_w, map_x, a, ctas, out, st);
+        default:
+            if constexpr (BITS == 4 || BITS == 8) return launch_small_t<BITS, 128>(map_w, map_x, a, ctas, out, st);
+            return DMR_ERR_UNSUPPORTED;
+    }
+}
+
+struct SmallMaps {
+    CUtensorMap w, x;
+};
+
+template <int BITS, int BN>
+dmr_status_t launch_routed_t(const SmallMaps &md, const SmallArgs &d, const SmallMaps &ml, const SmallArgs &l, int n_dense, int ctas, dmr_out_t out, cudaStream_t st) {
+    constexpr size_t smem = SmallCfg<0, BN>::SMEM > SmallCfg<BITS, BN>::SMEM ? SmallCfg<0, BN>::SMEM : SmallCfg<BITS, BN>::SMEM;
+    static_assert(SmallCfg<0, BN>::THREADS <= SmallCfg<BITS, BN>::THREADS, "the spare warps of a CTA on bf16 weights idle");
+    auto kernel = out == DMR_OUT_F32 ? small_routed_kernel<BITS, BN, true> : small_routed_kernel<BITS, BN, false>;
+    if (!ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), smem)) return DMR_ERR_CUDA;
+    const cudaError_t e = launch_pdl(kernel, dim3((unsigned)ctas), dim3(SmallCfg<BITS, BN>::THREADS), smem, st, md.w, md.x, d, ml.w, ml.x, l, n_dense);
+    if (e != cudaSuccess) return launch_failed(e);
+    return check_launch();
+}
+template <int BITS>
+dmr_status_t launch_routed_bits(int bn, const SmallMaps &md, const SmallArgs &d, const SmallMaps &ml, const SmallArgs &l, int n_dense, int ctas, dmr_out_t out,
+                                cudaStream_t st) {
+    switch (bn) {
+        case 16: return launch_routed_t<BITS, 16>(md, d, ml, l, n_dense, ctas, out, st);
+        case 32: return launch_routed_t<BITS, 32>(md, d, ml, l, n_dense, ctas, out, st);
+        default: return launch_routed_t<BITS, 64>(md, d, ml, l, n_dense, ctas, out, st);
+    }
+}
+
+bool small_maps(SmallMaps *m, const uint16_t *X, int M, const void *weights, int N, int K, int bits, int bn) {
+    if (!make_tensor_map_2d(&m->x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)K, (uint64_t)K * 2, (uint32_t)bn, 64, TmaSwizzle::k128B)) return false;
+    const uint64_t row_bytes = (uint64_t)K * bits / 8;
+    if (bits == 0)
+        return make_tensor_map_2d(&m->w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, weights, (uint64_t)N, (uint64_t)K, (uint64_t)K * 2, kSm, 64, TmaSwizzle::k128B);
+    return make_tensor_map_2d(&m->w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, weights, (uint64_t)N, row_bytes, row_bytes, kSm, (uint32_t)(kSk * bits / 8),
+                              bits == 3 ? TmaSwizzle::kNone : bits == 4 ? TmaSwizzle::k64B : TmaSwizzle::k128B);
+}
+
+SmallArgs small_args(const SmallPlan &p, int M, RowSel sel, const uint16_t *scales, const uint8_t *zeros, int N, int K, int bits, int g, void *Y, float *partial,
+                     int32_t *counters, int32_t *status) {
+    SmallArgs a = {};
+    a.scales = scales;
+    a.zeros = zeros;
+    a.Y = Y;
+    a.idx = sel.idx;
+    a.count = sel.count;
+    a.partial = partial;
+    a.counters = counters;
+    a.status = status;
+    a.M = M;
+    a.N = N;
+    a.K = K;
+    a.units = p.units;
+    a.k_units = (K + kSk - 1) / kSk;  // (half a unit past the end: zero activations)
+    a.shares = p.shares;
+    a.G = bits == 0 ? 1 : K / g;
+    a.half = bits != 0 && g == 64 ? 1 : 0;
+    a.g_units = bits == 0 || g == K ? a.k_units : a.half ? 1 : g / kSk;
+    a.g_mul = a.g_units > 1 ? (uint32_t)((0x100000000ull + (uint64_t)a.g_units - 1) / (uint64_t)a.g_units) : 0u;  // exact for the unit numbers that occur
+    return a;
+}
+
+}  // namespace
+
+bool small_supported(int M, int N, int K, int bits, int g) {
+    const int tiles = (N + kSm - 1) / kSm;
+    // narrow layers (k and v projections) with 4- and 8-bit codes: up to 128 rows, so that they are multiplied exactly
+    if (M < 1 || M > ((bits == 4 || bits == 8) && N <= kNarrow ? 128 : 64)) return false;
+    if (K % (bits == 3 ? kSk : kSk / 2) != 0) return false;  // (3-bit codes: rows of whole 48-byte boxes)
+    if (tiles > kSmallMaxTiles || K > 131072) return false;  // (units x shares stay below 2^32)
+    // a unit is one group, part of one, or two; two of 64 have an accumulator each, which is as many as there are
+    return bits == 0 || ((bits == 3 || bits == 4 || bits == 8) && (g % 128 == 0 || g == 64 || g == K));
+}
+
+SmallPlan small_plan(int M, int N, int K) {
+    SmallPlan p;
+    p.bn = small_bn(M);
+    p.tiles = (N + kSm - 1) / kSm;
+    p.units = p.tiles * ((K + kSk - 1) / kSk);
+    const int sms = device_sm_count(), most = p.units / kMinUnits;
+    p.shares = most < 1 ? 1 : (most < sms ? most : sms);
+    p.partial_bytes = (size_t)p.shares * 2 * p.bn * kSm * sizeof(float);
+    return p;
+}
+
+dmr_status_t launch_small(const uint16_t *X, int M, RowSel sel, const void *weights, const uint16_t *scales, const uint8_t *zeros, int N, int K,
+                          int bits, int g, void *Y, dmr_out_t out, float *partial, int32_t *counters, int32_t *status, cudaStream_t st) {
+    const SmallPlan p = small_plan(M, N, K);
+    SmallMaps m;
+    if (!small_maps(&m, X, M, weights, N, K, bits, p.bn)) return DMR_ERR_CUDA;
+    const SmallArgs a = small_args(p, M, sel, scales, zeros, N, K, bits, g, Y, partial, counters, status);
+    if (bits == 0) return launch_small_bits<0>(p.bn, m.w, m.x, a, p.shares, out, st);
+    if (bits == 3) return launch_small_bits<3>(p.bn, m.w, m.x, a, p.shares, out, st);
+    if (bits == 4) return launch_small_bits<4>(p.bn, m.w, m.x, a, p.shares, out, st);
+    return launch_small_bits<8>(p.bn, m.w, m.x, a, p.shares, out, st);
+}
+
+dmr_status_t launch_small_routed(const uint16_t *Xh, const uint16_t *Xl, int M, RowSel high, RowSel low, const uint16_t *W, const void *qweight,
+                                 const uint16_t *scales, const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out, float *partial_high,
+                                 float *partial_low, int32_t *counters_high, int32_t *counters_low, int32_t *status, cudaStream_t st) {
+    const SmallPlan p = small_plan(M, N, K);
+    SmallMaps md, ml;
+    if (!small_maps(&md, Xh, M, W, N, K, 0, p.bn) || !small_maps(&ml, Xl, M, qweight, N, K, bits, p.bn)) return DMR_ERR_CUDA;
+    const SmallArgs d = small_args(p, M, high, nullptr, nullptr, N, K, 0, K, Y, partial_high, counters_high, status);
+    const SmallArgs l = small_args(p, M, low, scales, zeros, N, K, bits, g, Y, partial_low, counters_low, status);
+    // Half of the SMs each: both halves' shares go into two (or, on small layers, one) per CTA.
+    const int half = device_sm_count() / 2, n = p.shares < half ? p.shares : half;
+    if (bits == 3) return launch_routed_bits<3>(p.bn, md, d, ml, l, n, 2 * n, out, st);
+    if (bits == 4) return launch_routed_bits<4>(p.bn, md, d, ml, l, n, 2 * n, out, st);
+    return launch_routed_bits<8>(p.bn, md, d, ml, l, n, 2 * n, out, st);
+}
+
+}  // namespace dmr

@@ -64,7 +64,7 @@ bool make_tensor_map_2d(CUtensorMap *map, CUtensorMapDataType dtype, size_t elem
     cuuint32_t estr[2] = {1, 1};
     (void)elem_bytes;
     CUresult r = g_encode(map, dtype, 2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          swizzle == TmaSwizzle::k128B ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                          swizzle == TmaSwizzle::k128B ? CU_TENSOR_MAP_SWIZZLE_128B : swizzle == TmaSwizzle::k64B ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         g_last_cuda_error = 10000 + (int)r;

@@ -1,0 +1,88 @@
+"""Batches of up to 64 rows (and of up to 128 on narrow layers with 4- and 8-bit codes) against the oracle at the edges of the kernel that
+multiplies exact integers: row counts around its three row tiles, feature counts below, at and beyond one 128-feature tile and not multiples
+of four, half a unit of inputs, one unit, and more units than CTAs, groups of half a unit, one, several and the whole row; routed rows bit
+for bit against the unrouted calls; and repeated calls of several layers on one stream."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2602_02711_b200 as dmr
+from paper_2602_02711_b200 import inputs, QFormat, OUT_BF16, OUT_F32
+from paper_2602_02711_b200.binding import OP_DENSE, OP_LOWBIT, OP_ROUTED
+from helpers import to_dev_bf16, rel_err
+
+pytestmark = pytest.mark.gpu
+
+TOL = 5e-5  # exact products (integers times bf16, scaled in fp32), fp32 sums of up to 5120 terms
+
+SHAPES = [(1, 128, 128), (3, 100, 64), (16, 129, 192), (17, 257, 384), (32, 130, 576), (33, 640, 512), (63, 1024, 2048), (64, 2304, 1088)]
+
+
+@pytest.mark.parametrize("M,N,K", SHAPES)
+def test_dense(M, N, K):
+    W, X = inputs.weights(N, K, seed=M), inputs.activations(M, K, seed=M)
+    Y = dmr.dmr_dense_linear(to_dev_bf16(X), to_dev_bf16(W), OUT_F32)
+    assert rel_err(Y.cpu().numpy().astype(np.float64), oracle.dense_linear(X, W)) <= TOL
+    assert torch.equal(dmr.dmr_dense_linear(to_dev_bf16(X), to_dev_bf16(W), OUT_BF16), Y.to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("bits", [3, 4, 8])
+@pytest.mark.parametrize("M,N,K,group", [s + (g,) for s in SHAPES for g in (64, 0)] + [(20, 700, 1024, 128), (64, 129, 1536, 256), (33, 128, 768, 384),
+                                                                                        (65, 1024, 512, 128), (128, 1920, 384, 64), (100, 250, 576, 192)])
+def test_low_bit(M, N, K, bits, group):
+    if bits == 3 and (M > 64 or K % 128 != 0):
+        pytest.skip("other kernels")
+    W, X = inputs.weights(N, K, seed=K), inputs.activations(M, K, seed=N, outlier_frac=0.01)
+    q = dmr.dmr_quantize(to_dev_bf16(W), QFormat(bits, group))
+    want = oracle.lowbit_linear(X, *oracle.quantize(W, bits=bits, group=group), bits=bits, group=group)
+    Y = dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_F32)
+    assert rel_err(Y.cpu().numpy().astype(np.float64), want) <= TOL
+    assert torch.equal(dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_BF16), Y.to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("bits,group", [(4, 128), (4, 64), (8, 0), (3, 128)])
+@pytest.mark.parametrize("M,high,N", [(2, 1, 700), (16, 5, 128), (17, 0, 700), (40, 40, 130), (64, 63, 700), (64, 20, 2304), (100, 30, 700)])
+def test_routed_rows_equal_unrouted_ones(M, high, N, bits, group):
+    K = 1024
+    W, X = to_dev_bf16(inputs.weights(N, K, seed=1)), to_dev_bf16(inputs.activations(M, K, seed=2))
+    q = dmr.dmr_quantize(W, QFormat(bits, group))
+    mask = np.zeros(M, dtype=np.uint8)
+    mask[np.random.default_rng(M).permutation(M)[:high]] = 1
+    md = torch.from_numpy(mask).cuda()
+    ws = dmr.new_workspace(OP_ROUTED, M, N, K, q.fmt)
+    Y = dmr.dmr_routed_linear(X, md, W, q, OUT_F32, workspace=ws)
+    want = torch.where(md[:, None] != 0, dmr.dmr_dense_linear(X, W, OUT_F32), dmr.dmr_lowbit_linear(X, q, OUT_F32))
+    assert torch.equal(Y, want)
+    assert int(ws[:4].view(torch.int32).item()) == 0
+
+
+@pytest.mark.parametrize("M,N,K", [(65, 257, 320), (100, 2000, 512), (128, 1930, 1024)])
+def test_rows_between_the_small_and_the_large_batches(M, N, K):
+    W, X = inputs.weights(N, K, seed=M), inputs.activations(M, K, seed=M)
+    Y = dmr.dmr_dense_linear(to_dev_bf16(X), to_dev_bf16(W), OUT_F32)
+    assert rel_err(Y.cpu().numpy().astype(np.float64), oracle.dense_linear(X, W)) <= TOL
+    for bits in (3, 4, 8) if N > 1920 else ():
+        q = dmr.dmr_quantize(to_dev_bf16(W), QFormat(bits, 128))
+        want = oracle.lowbit_linear(X, *oracle.quantize(W, bits=bits, group=128), bits=bits, group=128)
+        Y = dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_F32)
+        # weights rounded to fp16: 2^-11 / sqrt(3) in the root mean square, independent errors
+        assert np.linalg.norm(Y.cpu().numpy() - want) <= 2.0 ** -11 / 3 ** 0.5 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("bits,M", [(0, 5), (0, 64), (4, 30), (8, 13), (8, 128)])
+def test_calls_one_after_the_other(bits, M):
+    """Each launch starts before the one ahead of it has ended: outputs, partial sums and counters must not meet."""
+    layers = []
+    for N, K in [(1024, 5120), (5120, 1024), (1024, 5120)]:
+        W, X = to_dev_bf16(inputs.weights(N, K, seed=N)), to_dev_bf16(inputs.activations(M, K, seed=K))
+        q = dmr.dmr_quantize(W, QFormat(bits, 0)) if bits else None
+        ws = dmr.new_workspace(OP_LOWBIT if bits else OP_DENSE, M, N, K, QFormat(bits or 4, 0))
+        layers.append(lambda X=X, W=W, q=q, ws=ws: dmr.dmr_lowbit_linear(X, q, OUT_F32, workspace=ws) if q else dmr.dmr_dense_linear(X, W, OUT_F32, workspace=ws))
+    first = []
+    for f in layers:
+        first.append(f())
+        torch.cuda.synchronize()
+    for _ in range(20):
+        again = [f() for f in layers for _ in range(2)]
+        assert all(torch.equal(y, first[i // 2]) for i, y in enumerate(again))
