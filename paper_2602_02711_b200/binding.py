@@ -1,4 +1,5 @@
-"""ctypes binding of libdmr.so: argument marshalling only, every step runs in the CUDA kernels.
+"""Binding of libdmr.so: argument marshalling only, every step runs in the CUDA kernels.  ctypes, and for the linears, which a decode step
+calls one after the other, a small extension module (csrc/calls.cpp) that takes the tensors apart natively.
 
 Functions carry the names of the C entry points (include/dmr.h) and take torch CUDA tensors
 (or, for the *_host call, pinned host tensors). There is no CPU fallback: if the library is
@@ -35,6 +36,7 @@ class QFormat(ctypes.Structure):
 
 
 _lib = None
+_calls = None
 
 
 class RouterCfg(ctypes.Structure):
@@ -49,7 +51,7 @@ def lib_path() -> str:
 
 def lib() -> ctypes.CDLL:
     """Loads libdmr.so (built in-tree by paper_2602_02711_b200.build). Raises if it is missing."""
-    global _lib
+    global _lib, _calls
     if _lib is not None:
         return _lib
     if not os.path.exists(_LIB_PATH):
@@ -102,7 +104,12 @@ def lib() -> ctypes.CDLL:
     L.dmr_status_string.argtypes = [i32]
     L.dmr_last_cuda_error.restype = i32
     L.dmr_launch_count.restype = ctypes.c_uint64
-    _lib = L
+    try:
+        from . import _calls as calls
+    except ImportError as e:
+        raise DmrError(-1, f"{e}: run `python -m paper_2602_02711_b200.build`") from e
+    calls.bind(*(ctypes.cast(getattr(L, f), vp).value for f in ("dmr_lowbit_linear", "dmr_dense_linear", "dmr_routed_linear")))
+    _calls, _lib = calls, L
     return L
 
 
@@ -214,6 +221,14 @@ def _out_tensor(M, N, out, device, Y):
 def dmr_lowbit_linear(X: torch.Tensor, q: QuantizedLinear, out: int = OUT_BF16, Y=None, workspace=None,
                       stream=None) -> torch.Tensor:
     """Y = X . dequant(Wq)^T."""
+    L = lib()
+    if Y is not None and workspace is not None:
+        f = q.fmt
+        r = _calls.lowbit(X, q.qweight, q.scales, q.zeros, q.N, q.K, f.bits, f.group_size, Y, out, workspace, None if stream is None else stream.cuda_stream)
+        if r >= 0:
+            if r:
+                _check(r)
+            return Y
     _dev(X, torch.bfloat16, "X")
     M, K = X.shape
     if K != q.K:
@@ -221,14 +236,21 @@ def dmr_lowbit_linear(X: torch.Tensor, q: QuantizedLinear, out: int = OUT_BF16, 
     Y = _out_tensor(M, q.N, out, X.device, Y)
     if workspace is None:
         workspace = new_workspace(OP_LOWBIT, M, q.N, K, q.fmt, X.device)
-    _check(lib().dmr_lowbit_linear(_ptr(X), M, _ptr(q.qweight), _ptr(q.scales), _ptr(q.zeros), q.N, K, q.fmt,
-                                   _ptr(Y), out, _ptr(workspace), workspace.numel(), _stream(stream)))
+    _check(L.dmr_lowbit_linear(_ptr(X), M, _ptr(q.qweight), _ptr(q.scales), _ptr(q.zeros), q.N, K, q.fmt,
+                               _ptr(Y), out, _ptr(workspace), workspace.numel(), _stream(stream)))
     return Y
 
 
 def dmr_dense_linear(X: torch.Tensor, W: torch.Tensor, out: int = OUT_BF16, Y=None, workspace=None,
                      stream=None) -> torch.Tensor:
     """Y = X . W^T with bf16 weights."""
+    L = lib()
+    if Y is not None and workspace is not None:
+        r = _calls.dense(X, W, Y, out, workspace, None if stream is None else stream.cuda_stream)
+        if r >= 0:
+            if r:
+                _check(r)
+            return Y
     _dev(X, torch.bfloat16, "X")
     _dev(W, torch.bfloat16, "W")
     M, K = X.shape
@@ -238,14 +260,21 @@ def dmr_dense_linear(X: torch.Tensor, W: torch.Tensor, out: int = OUT_BF16, Y=No
     Y = _out_tensor(M, N, out, X.device, Y)
     if workspace is None:
         workspace = new_workspace(OP_DENSE, M, N, K, QFormat(4, 0), X.device)
-    _check(lib().dmr_dense_linear(_ptr(X), M, _ptr(W), N, K, _ptr(Y), out, _ptr(workspace), workspace.numel(),
-                                  _stream(stream)))
+    _check(L.dmr_dense_linear(_ptr(X), M, _ptr(W), N, K, _ptr(Y), out, _ptr(workspace), workspace.numel(), _stream(stream)))
     return Y
 
 
 def dmr_routed_linear(X: torch.Tensor, mask: torch.Tensor, W: torch.Tensor, q: QuantizedLinear,
                       out: int = OUT_BF16, Y=None, workspace=None, stream=None) -> torch.Tensor:
     """Rows with mask != 0 use the bf16 weights, the others the low-bit weights; Y keeps step order."""
+    L = lib()
+    if Y is not None and workspace is not None:
+        f = q.fmt
+        r = _calls.routed(X, mask, W, q.qweight, q.scales, q.zeros, q.N, q.K, f.bits, f.group_size, Y, out, workspace, None if stream is None else stream.cuda_stream)
+        if r >= 0:
+            if r:
+                _check(r)
+            return Y
     _dev(X, torch.bfloat16, "X")
     _dev(W, torch.bfloat16, "W")
     _dev(mask, torch.uint8, "mask")
@@ -255,8 +284,8 @@ def dmr_routed_linear(X: torch.Tensor, mask: torch.Tensor, W: torch.Tensor, q: Q
     Y = _out_tensor(M, q.N, out, X.device, Y)
     if workspace is None:
         workspace = new_workspace(OP_ROUTED, M, q.N, K, q.fmt, X.device)
-    _check(lib().dmr_routed_linear(_ptr(X), M, _ptr(mask), _ptr(W), _ptr(q.qweight), _ptr(q.scales), _ptr(q.zeros),
-                                   q.N, K, q.fmt, _ptr(Y), out, _ptr(workspace), workspace.numel(), _stream(stream)))
+    _check(L.dmr_routed_linear(_ptr(X), M, _ptr(mask), _ptr(W), _ptr(q.qweight), _ptr(q.scales), _ptr(q.zeros),
+                               q.N, K, q.fmt, _ptr(Y), out, _ptr(workspace), workspace.numel(), _stream(stream)))
     return Y
 
 

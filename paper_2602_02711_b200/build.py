@@ -1,7 +1,7 @@
 """Builds libdmr.so in-tree with nvcc for sm_100a (cross-compiles without a GPU).
 
 Every .cu file is compiled to an object of its own (in parallel, only when it or a header changed)
-and the objects are linked into the shared library.
+and the objects are linked into the shared library.  csrc/calls.cpp becomes the extension module _calls.so beside it.
 """
 from __future__ import annotations
 
@@ -9,6 +9,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -16,6 +17,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdmr.so")
+CALLS_SRC = os.path.join(CSRC, "calls.cpp")
+CALLS = os.path.join(PKG, "_calls.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -43,7 +46,16 @@ def _stale(target: str, deps) -> bool:
 
 
 def needs_build() -> bool:
-    return _stale(LIB, sources() + headers())
+    return _stale(LIB, sources() + headers()) or _stale(CALLS, [CALLS_SRC] + headers())
+
+
+def _calls_command() -> list:
+    import torch  # for its paths
+    base = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            "-I" + os.path.join(ROOT, "include"), "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(cuda, "include"),
+            "-I" + os.path.join(base, "include"), CALLS_SRC, "-o", CALLS, "-L" + os.path.join(base, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -59,6 +71,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         return src, r
 
+    calls = subprocess.Popen(_calls_command()) if force or _stale(CALLS, [CALLS_SRC] + hdrs) else None
     with ThreadPoolExecutor(max_workers=min(8, max(1, len(todo)))) as pool:
         for src, r in pool.map(compile_one, todo):
             if verbose or r.returncode != 0:
@@ -67,6 +80,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
                 raise subprocess.CalledProcessError(r.returncode, f"nvcc {src}")
     objs = [_obj(s) for s in sources()]
     subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "--shared", "-o", LIB] + objs, check=True)
+    if calls is not None and calls.wait() != 0:
+        raise subprocess.CalledProcessError(calls.returncode, f"{calls.args[0]} {CALLS_SRC}")
     return LIB
 
 
