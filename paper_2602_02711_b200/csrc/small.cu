@@ -418,8 +418,16 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
         constexpr int CW = BN < 64 ? BN : 64;
         const int m_lo = Cfg::EW == 4 ? 0 : ((warp - W_SCALE) >> 2) * CW;  // this warp's rows of the batch: m_lo .. m_lo + CW - 1
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)m_lo;
+        constexpr int LW = CW < 32 ? CW : 32;  // accumulator columns per round trip to tensor memory
+        auto load_sums = [](uint32_t addr, uint32_t (&v)[LW]) {
+            tmem_ld_x16(addr, reinterpret_cast<uint32_t (&)[16]>(v[0]));
+            if constexpr (LW == 32) tmem_ld_x16(addr + 16, reinterpret_cast<uint32_t (&)[16]>(v[16]));
+            tmem_ld_wait();
+        };
         bool ok = true;
         if (work) pdl_wait();  // outputs and partial sums may still be in use by the kernel before
+        auto row_of = [&](int m) { return a.idx && work ? a.idx[min(m, rows - 1)] : m; };
+        const int row_lo = row_of(m_lo + lane), row_hi = CW > 32 ? row_of(m_lo + 32 + lane) : 0;  // output rows of this warp's batch slots
         int i = 0;  // units done
         uint32_t phases = 0;  // bit w: phase of tfull w
         int tile = lo_tile, ku = lo_ku, share = share_lo, share_end = first_unit(share_lo + 1);
@@ -462,21 +470,19 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
                     if (!ok) break;
                     tcgen05_fence_after();
 #pragma unroll
-                    for (int c0 = 0; c0 < CW; c0 += 16) {
-                        uint32_t v[16];
-                        tmem_ld_x16(lane_addr + (uint32_t)w * d_cols + (uint32_t)c0, v);
-                        tmem_ld_wait();
+                    for (int c0 = 0; c0 < CW; c0 += LW) {
+                        uint32_t v[LW];
+                        load_sums(lane_addr + (uint32_t)w * d_cols + (uint32_t)c0, v);
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) acc[c0 + c] = BITS == 0 ? acc[c0 + c] + __uint_as_float(v[c]) : fmaf(sc0, __uint_as_float(v[c]), acc[c0 + c]);
+                        for (int c = 0; c < LW; ++c) acc[c0 + c] = BITS == 0 ? acc[c0 + c] + __uint_as_float(v[c]) : fmaf(sc0, __uint_as_float(v[c]), acc[c0 + c]);
                     }
                     if (half_groups) {
 #pragma unroll
-                        for (int c0 = 0; c0 < CW; c0 += 16) {
-                            uint32_t v[16];
-                            tmem_ld_x16(lane_addr + (uint32_t)w * d_cols + half_cols + (uint32_t)c0, v);
-                            tmem_ld_wait();
+                        for (int c0 = 0; c0 < CW; c0 += LW) {
+                            uint32_t v[LW];
+                            load_sums(lane_addr + (uint32_t)w * d_cols + half_cols + (uint32_t)c0, v);
 #pragma unroll
-                            for (int c = 0; c < 16; ++c) acc[c0 + c] = fmaf(sc1, __uint_as_float(v[c]), acc[c0 + c]);
+                            for (int c = 0; c < LW; ++c) acc[c0 + c] = fmaf(sc1, __uint_as_float(v[c]), acc[c0 + c]);
                         }
                     }
                     tcgen05_fence_before();
@@ -505,13 +511,18 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
                         if (to_sum < kMaxSums) sum_tile[to_sum++] = tile;
                     }
                 }
-            } else if (n < a.N) {
+            } else {
+                // (Row numbers from the lanes that hold them, branches only around the stores: an address from each row's number in memory,
+                // in a branch of its own, costs 80 cycles a row: two tiles of 64 rows 12.7 us instead of 6.1.)
+                const uint32_t stride = (uint32_t)a.N * (OUT_F32 ? 4u : 2u);
+                char *y = reinterpret_cast<char *>(a.Y) + (size_t)n * (OUT_F32 ? 4 : 2);
+                const int m_n = n < a.N ? rows - m_lo : 0;
 #pragma unroll
                 for (int c = 0; c < CW; ++c) {
-                    if (m_lo + c < rows) {
-                        const size_t at = (size_t)(a.idx ? a.idx[m_lo + c] : m_lo + c) * a.N + n;
-                        if (OUT_F32) reinterpret_cast<float *>(a.Y)[at] = acc[c];
-                        else reinterpret_cast<__nv_bfloat16 *>(a.Y)[at] = __float2bfloat16_rn(acc[c]);
+                    char *at = y + (uint64_t)(uint32_t)__shfl_sync(0xffffffffu, c < 32 ? row_lo : row_hi, c & 31) * stride;
+                    if (c < m_n) {
+                        if (OUT_F32) *reinterpret_cast<float *>(at) = acc[c];
+                        else *reinterpret_cast<__nv_bfloat16 *>(at) = __float2bfloat16_rn(acc[c]);
                     }
                 }
             }
@@ -531,7 +542,7 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
 
     // The shared tiles that this CTA was the last one to finish, with all its warps: a warp for a few rows, four features per lane, several
     // CTAs' sums requested at once.  (By the scale warps alone, at the time, it took 0.76 us per CTA of a tile of 64 rows: routed 14B layer, M = 64, 311 us instead of 279.)
-    constexpr int RW = BN >= 64 ? 4 : BN / 16, CU = BN >= 64 ? 4 : 8;  // rows of a warp, and CTAs, at a time
+    constexpr int RW = BN >= 64 ? 4 : BN / 16, CU = BN == 16 ? 8 : BN == 128 ? 2 : 4;  // rows of a warp, and CTAs, at a time (as registers allow)
     for (int e = 0; e < to_sum; ++e) {
         const int tile = sum_tile[e], n4 = tile * kSm + 4 * lane;
         int c_first, c_last;
