@@ -8,8 +8,8 @@
 // multiplication per weight, activations used as they are; a quantization group's sums are scaled once, in fp32, on their way out of the
 // accumulator (one fma per feature, row and group).
 // Measured (four linears of the 7B layer, us; in brackets the kernels that ran before, a streaming kernel up to 32 rows and tensor-core kernels
-// with unpacked tiles in shared memory above): 4-bit M = 17 77 (107), 32 83 (114), 64 96 (128); 3-bit M = 32 86 (116); bf16 M = 3 79 (88),
-// 16 87 (95), 64 106 (116); 8-bit, 32B layer, M = 1 66 (86), 13 67 (113), 64 92 (147).  A unit of codes still takes 700 to 900 cycles:
+// with unpacked tiles in shared memory above): 4-bit M = 17 75 (107), 32 76 (114), 64 85 (128); 3-bit M = 32 79 (116); bf16 M = 3 79 (88),
+// 16 87 (95), 64 96 (116); 8-bit, 32B layer, M = 1 64 (86), 13 65 to 68 (113), 64 91 (147).  A unit of codes still takes 700 to 900 cycles:
 // the chain of wait, unpack, store, MMA and commit of the units in flight, not the HBM rate.
 // Tried and dropped: one MMA warp (1380 cycles per unit); tiles of 128 rows for all layers (routed M = 128 402 against pair.cu's 375).
 //
@@ -32,7 +32,7 @@ namespace {
 constexpr int kSm = 128;        // features per tile
 constexpr int kSk = 128;        // inputs per unit
 constexpr int kABufs = 4;       // unpacked units in tensor memory, 64 columns each
-constexpr int kMaxSums = 8;     // shared tiles of a CTA at most: two for each of its shares
+constexpr int kMaxShared = 8;    // shared tiles of a CTA at most: two for each of its shares
 constexpr int kMinUnits = 8;    // units per CTA at least: below, the exchange costs more than the SMs bring (1024 x 5120, routed, M = 64, 14B layer: 4 / 8 / 12: 289 / 279 / 289 us)
 
 template <int BITS, int BN>  // BITS 0: bf16 weights
@@ -50,7 +50,8 @@ struct SmallCfg {
     static constexpr int S = S_RAW > 16 ? 16 : S_RAW;
     static constexpr int EW = BN == 128 ? 8 : 4;                       // scale warps, at most 64 rows of the batch each
     // warps: unpack first, so that groups of four cover the lane quadrants, then scale, MMA, copies
-    static constexpr int THREADS = 32 * (UW + EW + MW + 1);
+    static constexpr int WARPS = UW + EW + MW + 1;
+    static constexpr int THREADS = 32 * (WARPS < 16 ? 16 : WARPS);     // (spare warps help with the sums of shared tiles: one turn for 16 groups of rows)
     static constexpr size_t SMEM = (size_t)S * STAGE + 1024 /*alignment*/ + 1024 /*barriers*/;
     static_assert(STAGE % 1024 == 0 && W_BYTES % 1024 == 0, "tiles on swizzle boundaries");
     static_assert(S >= TURN && S % TURN == 0 && S % MW == 0 && (UW == 0 || (S % (UW / 4) == 0 && kABufs % (UW / 4) == 0)) && kABufs % MW == 0, "turns");
@@ -158,9 +159,13 @@ template <int BITS, int BN, bool OUT_F32>
 __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUtensorMap &map_x, const SmallArgs &a, uint32_t tmem_base, int cta, int ctas) {
     using Cfg = SmallCfg<BITS, BN>;
     constexpr int S = Cfg::S, MW = Cfg::MW;
+    // Counting a CTA into a shared tile means a fence and the counter's way to the L2 and back, which hold the scale warps up, and with them the
+    // MMAs: it is left until all units are done (routed 14B layer, M = 64, 259 us instead of 278; bf16 M = 64 96 instead of 103).  The instances
+    // for few rows of 8-bit codes, whose scale warps have little to do, are the faster for counting at once (32B layer, M = 13, 65 instead of 67).
+    constexpr bool COUNT_NOW = BITS == 8 && BN < 64;
     constexpr int W_SCALE = Cfg::UW, W_MMA = Cfg::UW + Cfg::EW, W_COPY = W_MMA + MW;  // first warp of each role
     extern __shared__ uint8_t smem_dyn[];
-    __shared__ int sum_tile[kMaxSums], to_sum;  // shared tiles that this CTA finished last
+    __shared__ int shared_tile[kMaxShared], n_shared;  // tiles that this CTA has a part of, later those that it finished last
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -184,6 +189,15 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
     auto slot_of = [&](int tile, int c) -> float * {
         return a.partial + ((size_t)c * 2 + (first_unit(c) >= tile * a.k_units ? 0 : 1)) * (size_t)(BN * kSm);
     };
+    // counts this CTA into a tile whose sums it has stored: whether it is the last one
+    auto count_in = [&](int tile) {
+        int c_first, c_last;
+        sharers(tile, c_first, c_last);
+        const bool last = atomicAdd(a.counters + tile, 1) == c_last - c_first;
+        __threadfence();
+        if (last) a.counters[tile] = 0;
+        return last;
+    };
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(wfull_bar(s), 1);
@@ -195,7 +209,7 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
             mbar_init(tempty_bar(i), Cfg::EW);
             mbar_init(tfull_bar(i), 1);
         }
-        to_sum = 0;
+        n_shared = 0;
         fence_barrier_init();
         prefetch_tensor_map(&map_w);
         prefetch_tensor_map(&map_x);
@@ -495,21 +509,16 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
             if (!ok) break;
             if (mine < a.k_units) {
                 // one of several shares that have units of this tile
-                int c_first, c_last;
-                sharers(tile, c_first, c_last);
                 float *part = slot_of(tile, share) + r;
 #pragma unroll
                 for (int c = 0; c < CW; ++c)
                     if (m_lo + c < rows) __stcg(part + (m_lo + c) * kSm, acc[c]);
-                __threadfence();
-                asm volatile("bar.sync 1, %0;" ::"n"(Cfg::EW * 32) : "memory");
-                if (warp == W_SCALE && lane == 0) {
-                    const bool last = atomicAdd(a.counters + tile, 1) == c_last - c_first;
+                if constexpr (COUNT_NOW) {
                     __threadfence();
-                    if (last) {
-                        a.counters[tile] = 0;
-                        if (to_sum < kMaxSums) sum_tile[to_sum++] = tile;
-                    }
+                    asm volatile("bar.sync 1, %0;" ::"n"(Cfg::EW * 32) : "memory");
+                    if (warp == W_SCALE && lane == 0 && count_in(tile)) shared_tile[n_shared++] = tile;
+                } else {
+                    if (warp == W_SCALE && lane == 0) shared_tile[n_shared++] = tile;
                 }
             } else {
                 // (Row numbers from the lanes that hold them, branches only around the stores: an address from each row's number in memory,
@@ -532,6 +541,7 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
                 ++tile;
             }
         }
+        if constexpr (!COUNT_NOW) __threadfence();  // the partial sums, before the CTA counts itself
         __syncwarp();
     }
 
@@ -540,11 +550,18 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
     __syncthreads();
     tcgen05_fence_after();
 
-    // The shared tiles that this CTA was the last one to finish, with all its warps: a warp for a few rows, four features per lane, several
-    // CTAs' sums requested at once.  (By the scale warps alone, at the time, it took 0.76 us per CTA of a tile of 64 rows: routed 14B layer, M = 64, 311 us instead of 279.)
+    // The shared tiles that this CTA is the last one to finish are summed with all its warps: a warp for a few rows, four features per lane,
+    // several CTAs' sums requested at once.  (By the scale warps alone, at the time, it took 0.76 us per CTA of a tile of 64 rows: routed 14B
+    // layer, M = 64, 311 us instead of 279.)
+    if constexpr (!COUNT_NOW) {
+        if (n_shared == 0) return;
+        if ((int)threadIdx.x < n_shared && !count_in(shared_tile[threadIdx.x])) shared_tile[threadIdx.x] = -1;
+        __syncthreads();
+    }
     constexpr int RW = BN >= 64 ? 4 : BN / 16, CU = BN == 16 ? 8 : BN == 128 ? 2 : 4;  // rows of a warp, and CTAs, at a time (as registers allow)
-    for (int e = 0; e < to_sum; ++e) {
-        const int tile = sum_tile[e], n4 = tile * kSm + 4 * lane;
+    for (int e = 0; e < n_shared; ++e) {
+        if (shared_tile[e] < 0) continue;
+        const int tile = shared_tile[e], n4 = tile * kSm + 4 * lane;
         int c_first, c_last;
         sharers(tile, c_first, c_last);
 #pragma unroll 1
