@@ -298,7 +298,9 @@ __global__ void __launch_bounds__(kThreads, 1) router_fused_kernel(const FusedAr
     const size_t layer_floats = (size_t)4 * d * d + (size_t)2 * f * d + 9 * (size_t)d + f;
 
     if (threadIdx.x == 0) prefetch_l2(a.params + (size_t)a.l_max * d, layer_floats);
-    if (threadIdx.x < kTokBlock) fs[threadIdx.x * a.rf] = 0.f;  // a CTA without hidden features multiplies zeros with these
+    // A CTA without hidden features (sixteen shares of a multiple of four can be more than there are) runs the second linear's tasks with weights
+    // of zero and reads four floats of each of these rows for them: what an earlier kernel left there may not be finite.
+    if (threadIdx.x < kTokBlock) *reinterpret_cast<float4 *>(fs + threadIdx.x * a.rf) = make_float4(0.f, 0.f, 0.f, 0.f);
     if (warp == 0) {  // first rows: a running sum of the lengths
         int base = 0;
         for (int b0 = 0; b0 < a.B; b0 += 32) {

@@ -52,3 +52,20 @@ def test_inside_a_graph():
         g.replay()
         torch.cuda.synchronize()
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("ffn", [16, 80, 208, 400])
+def test_features_that_some_ctas_have_none_of_after_a_kernel_that_left_nans(ffn):
+    """Some of the sixteen CTAs of a cluster have no hidden features at these widths.  What the kernel before left in shared memory - here NaN
+    in every word - must not reach the probabilities."""
+    kw = dict(d=64, heads=4, ffn=ffn, layers=2, l_max=16, classes=2)
+    cfg = RouterCfg(**kw)
+    p = inputs.router_params(**kw, seed=3)
+    Z, n = inputs.router_embeddings(20, 16, 64, seed=3), inputs.router_lengths(20, 16, seed=3)
+    params, Zd, nd = dmr.pack_router_params(p, cfg), torch.from_numpy(Z).cuda(), torch.from_numpy(n).cuda()
+    X, W = torch.full((16, 4096), float("nan"), device="cuda").bfloat16(), torch.full((4096, 4096), float("nan"), device="cuda").bfloat16()
+    want = oracle.router_forward(Z, n, p, 4)
+    for _ in range(5):
+        dmr.dmr_dense_linear(X, W)
+        got, _ = dmr.dmr_router_forward(params, cfg, Zd, nd)
+        assert np.abs(got.cpu().numpy() - want).max() <= TOL
