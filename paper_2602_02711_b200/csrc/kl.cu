@@ -25,7 +25,11 @@ constexpr int kKlThreads = 512;
 constexpr int kKlWarps = kKlThreads / 32;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
-constexpr float kLogitFloor = -1.0e30f;  // -inf logits are raised to this: no inf - inf anywhere, e^(x - m) is still 0
+// Logits below this (-inf, a mask of the type's lowest value) are raised to it: no inf - inf anywhere, e^(x - m) is still 0.  A bf16 number whose
+// product with log2 e is rounded up: where a thread has met nothing but the floor so far, the fused multiply-add of its weight leaves that
+// rounding, 5e22 below zero, whose power of two is 0 (of a floor whose product is rounded down it would be infinite).
+constexpr float kLogitFloor = -9.953037915854457e29f;
+constexpr uint32_t kFloorPair = 0xF149F149u;  // the same as a bf16 pair
 
 // CTAs of a cluster that share a row: the two halves of a long row end together and few tokens reach twice as many SMs (9 tokens x
 // 151936: 20.5 us in one part, 18 in two; 777 tokens: 95 and 90); rows below 16384 entries would mostly pay for the exchange.
@@ -72,11 +76,15 @@ __device__ __forceinline__ void kl_raise(KlThread &st, float va, float vb) {
         st.mb = vb;
     }
 }
-// One 16-byte vector of each row.  Finite logits only: -inf or NaN anywhere leaves s1 or s2 not finite, which the caller looks at
-// once per part of a row (kl_redo) instead of once per element.
+// One 16-byte vector of each row.  Of a, finite logits only: -inf or NaN anywhere leaves s1 not finite, which the caller looks at once per
+// part of a row (kl_redo) instead of once per element; a finite one below the floor has weight 0, or leaves s1 not finite where the thread has
+// met no other.
 template <bool F32>
 __device__ __forceinline__ void kl_vector(KlThread &st, const uint4 &qa, const uint4 &qb) {
-    const uint32_t a[4] = {qa.x, qa.y, qa.z, qa.w}, b[4] = {qb.x, qb.y, qb.z, qb.w};
+    const uint32_t a[4] = {qa.x, qa.y, qa.z, qa.w};
+    uint32_t b[4] = {qb.x, qb.y, qb.z, qb.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) b[i] = F32 ? __float_as_uint(fmaxf(__uint_as_float(b[i]), kLogitFloor)) : bmax2(b[i], kFloorPair);
     if constexpr (F32) {
         const float va = fmaxf(fmaxf(__uint_as_float(a[0]), __uint_as_float(a[1])), fmaxf(__uint_as_float(a[2]), __uint_as_float(a[3])));
         const float vb = fmaxf(fmaxf(__uint_as_float(b[0]), __uint_as_float(b[1])), fmaxf(__uint_as_float(b[2]), __uint_as_float(b[3])));
@@ -96,7 +104,7 @@ __device__ __forceinline__ void kl_vector(KlThread &st, const uint4 &qa, const u
         st.s2[i & 1] += ex2(fmaf(y, kLog2e, -st.mb));
     }
 }
-// One element of any value: -inf and NaN count as the floor, and p_v = 0 contributes nothing whatever b_v is.
+// One element of any value: -inf, NaN and what lies below the floor count as the floor, and p_v = 0 contributes nothing whatever b_v is.
 __device__ __forceinline__ void kl_element(KlThread &st, float a, float b) {
     a = fmaxf(a, kLogitFloor);
     b = fmaxf(b, kLogitFloor);
@@ -238,7 +246,8 @@ kl_token_kernel(const void *__restrict__ high, const void *__restrict__ low, int
     kl_warp_sum(tot);
     // lse(b) - lse(a), differences first (exactly 0 for equal rows), from log2 to natural-log units
     const float dlse = ((tot.mb - tot.ma) + (log2f(tot.s2) - log2f(tot.s0))) * kLn2;
-    if (lane == 0) kl_token[tok] = tot.s1 / tot.s0 + dlse;
+    // a row of nothing but the floor is no distribution: undefined (0 / 0) as the first one, infinitely far as the second
+    if (lane == 0) kl_token[tok] = tot.s2 == 0.f && tot.s0 > 0.f ? INFINITY : tot.s1 / tot.s0 + dlse;
 }
 
 // kl_step[s] = mean of kl_token over [offsets[s], offsets[s + 1]), added in token order; 0 for an empty step.
