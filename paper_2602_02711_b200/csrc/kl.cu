@@ -35,6 +35,14 @@ constexpr uint32_t kFloorPair = 0xF149F149u;  // the same as a bf16 pair
 // 151936: 20.5 us in one part, 18 in two; 777 tokens: 95 and 90); rows below 16384 entries would mostly pay for the exchange.
 constexpr int kKlMaxParts = 2;
 __host__ __device__ constexpr int kl_parts(int V) { return V >= 16384 ? 2 : 1; }
+// CTAs that share a row: one for each part, except that one CTA takes a row of fp32 logits part after part (the same sums) where the halves need an
+// even number of rounds of CTAs over the chip.  Whole rows fill it as well then, and a round that is nearly empty, a row's latency long, costs half
+// as much of the time as they do (300 x 151936: 78 and 68 us; 444 x 99997: 91 and 68; but 250 x 151936 48 and 63, 700 x 151936 139 and 160).
+// With bf16 logits, half as many bytes for the same exponentials, such a round is hidden (300 x 151936: 45 and 48 us).
+inline int kl_ctas(int T, int parts, bool f32) {
+    const int resident = 4 * device_sm_count();
+    return f32 && parts == 2 && (T + (resident / 2 - 1)) / (resident / 2) % 2 == 0 ? 1 : parts;
+}
 static_assert(kKlMaxParts * kKlWarps <= 32, "the sums of a token's warps meet in one warp");
 
 __device__ __forceinline__ float ex2(float x) {
@@ -179,12 +187,12 @@ __device__ __noinline__ KlThread kl_redo(const uint8_t *ra, const uint8_t *rb, i
 // 250 x 151936 fp32: 64 -> 53 (5.8 TB/s).
 template <bool F32, bool ALIGNED>
 __global__ void __launch_bounds__(kKlThreads, 4)
-kl_token_kernel(const void *__restrict__ high, const void *__restrict__ low, int V, int parts, float *__restrict__ kl_token) {
+kl_token_kernel(const void *__restrict__ high, const void *__restrict__ low, int V, int parts, int ctas, float *__restrict__ kl_token) {
     constexpr int ES = F32 ? 4 : 2, VE = F32 ? 4 : 8;  // bytes per element, elements per vector
     __shared__ KlSums sums[kKlMaxParts * kKlWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rank = (int)(blockIdx.x % (unsigned)parts);
-    const size_t tok = blockIdx.x / (unsigned)parts;
+    const int rank = (int)(blockIdx.x % (unsigned)ctas);  // `ctas` CTAs share a row's parts: each takes one, or the only one takes all
+    const size_t tok = blockIdx.x / (unsigned)ctas;
     pdl_launch_dependents();
     asm volatile("barrier.cluster.arrive.relaxed.aligned;");  // every CTA of the cluster runs before its shared memory is written
 
@@ -194,48 +202,51 @@ kl_token_kernel(const void *__restrict__ high, const void *__restrict__ low, int
     const int vecs = (V + VE - 1) / VE, per = (vecs + parts - 1) / parts;
     // vectors that lie, with the 16 bytes after them where those are read too, inside the row
     const int whole = shift == 0 ? V / VE : max(0, (V - VE) / VE);
-    const int end = min(vecs, (rank + 1) * per), fast = min(end, whole), first = rank * per + (int)threadIdx.x;
-    KlThread st;
-    int v = first;
-    const uint8_t *pa = ra + (size_t)v * 16, *pb = rb + (size_t)v * 16;
 #pragma unroll 1
-    for (; v < fast; v += kKlThreads) {
-        kl_vector<F32>(st, load_shifted(pa, shift), load_shifted(pb, shift));
-        pa += kKlThreads * 16;
-        pb += kKlThreads * 16;
-    }
-    for (; v < end; v += kKlThreads) {
-        // the one or two vectors at the row's end; a whole one is added like every other, whatever `shift`
-        if ((v + 1) * VE > V) {
-            st = kl_elements<F32>(st, ra, rb, v, V);
-            continue;
+    for (int part = rank; part < (F32 && ctas == 1 ? parts : rank + 1); ++part) {
+        const int end = min(vecs, (part + 1) * per), fast = min(end, whole), first = part * per + (int)threadIdx.x;
+        KlThread st;
+        int v = first;
+        const uint8_t *pa = ra + (size_t)v * 16, *pb = rb + (size_t)v * 16;
+#pragma unroll 1
+        for (; v < fast; v += kKlThreads) {
+            kl_vector<F32>(st, load_shifted(pa, shift), load_shifted(pb, shift));
+            pa += kKlThreads * 16;
+            pb += kKlThreads * 16;
         }
-        uint32_t x[4], y[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if constexpr (F32) {
-                x[j] = reinterpret_cast<const uint32_t *>(ra)[v * 4 + j];
-                y[j] = reinterpret_cast<const uint32_t *>(rb)[v * 4 + j];
-            } else {
-                const uint16_t *p = reinterpret_cast<const uint16_t *>(ra) + v * 8 + 2 * j, *q = reinterpret_cast<const uint16_t *>(rb) + v * 8 + 2 * j;
-                x[j] = p[0] | ((uint32_t)p[1] << 16);
-                y[j] = q[0] | ((uint32_t)q[1] << 16);
+        for (; v < end; v += kKlThreads) {
+            // the one or two vectors at the row's end; a whole one is added like every other, whatever `shift`
+            if ((v + 1) * VE > V) {
+                st = kl_elements<F32>(st, ra, rb, v, V);
+                continue;
             }
+            uint32_t x[4], y[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if constexpr (F32) {
+                    x[j] = reinterpret_cast<const uint32_t *>(ra)[v * 4 + j];
+                    y[j] = reinterpret_cast<const uint32_t *>(rb)[v * 4 + j];
+                } else {
+                    const uint16_t *p = reinterpret_cast<const uint16_t *>(ra) + v * 8 + 2 * j, *q = reinterpret_cast<const uint16_t *>(rb) + v * 8 + 2 * j;
+                    x[j] = p[0] | ((uint32_t)p[1] << 16);
+                    y[j] = q[0] | ((uint32_t)q[1] << 16);
+                }
+            }
+            kl_vector<F32>(st, make_uint4(x[0], x[1], x[2], x[3]), make_uint4(y[0], y[1], y[2], y[3]));
         }
-        kl_vector<F32>(st, make_uint4(x[0], x[1], x[2], x[3]), make_uint4(y[0], y[1], y[2], y[3]));
-    }
-    if (!isfinite((st.s1[0] + st.s1[1]) + (st.s2[0] + st.s2[1]))) st = kl_redo<F32>(ra, rb, first, end, V);
-    KlSums s;
-    s.ma = st.ma;
-    s.mb = st.mb;
-    s.s0 = st.s0[0] + st.s0[1];
-    s.s1 = st.s1[0] + st.s1[1];
-    s.s2 = st.s2[0] + st.s2[1];
-    kl_warp_sum(s);
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if (lane < 5) {  // the warp's five numbers to the first CTA's shared memory
-        const float f = lane == 0 ? s.ma : lane == 1 ? s.s0 : lane == 2 ? s.s1 : lane == 3 ? s.mb : s.s2;
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_map(smem_u32(&sums[rank * kKlWarps + warp]) + 4u * lane, 0)), "f"(f) : "memory");
+        if (!isfinite((st.s1[0] + st.s1[1]) + (st.s2[0] + st.s2[1]))) st = kl_redo<F32>(ra, rb, first, end, V);
+        KlSums s;
+        s.ma = st.ma;
+        s.mb = st.mb;
+        s.s0 = st.s0[0] + st.s0[1];
+        s.s1 = st.s1[0] + st.s1[1];
+        s.s2 = st.s2[0] + st.s2[1];
+        kl_warp_sum(s);
+        if (part == rank) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (lane < 5) {  // the warp's five numbers to the first CTA's shared memory
+            const float f = lane == 0 ? s.ma : lane == 1 ? s.s0 : lane == 2 ? s.s1 : lane == 3 ? s.mb : s.s2;
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_map(smem_u32(&sums[part * kKlWarps + warp]) + 4u * lane, 0)), "f"(f) : "memory");
+        }
     }
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -274,16 +285,16 @@ dmr_status_t launch_stepwise_kl(const void *high, const void *low, bool f32, int
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (T > 0) {
-        const int parts = kl_parts(V);
+        const int parts = kl_parts(V), ctas = kl_ctas(T, parts, f32);
         const bool aligned = V % (f32 ? 4 : 8) == 0;
         auto kernel = f32 ? (aligned ? kl_token_kernel<true, true> : kl_token_kernel<true, false>)
                           : (aligned ? kl_token_kernel<false, true> : kl_token_kernel<false, false>);
-        cfg.gridDim = dim3((unsigned)T * (unsigned)parts, 1, 1);
+        cfg.gridDim = dim3((unsigned)T * (unsigned)ctas, 1, 1);
         cfg.blockDim = dim3(kKlThreads, 1, 1);
         attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)parts;
+        attr[0].val.clusterDim.x = (unsigned)ctas;
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, high, low, V, parts, kl_token);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, high, low, V, parts, ctas, kl_token);
         if (e != cudaSuccess) return launch_failed(e);
         dmr_status_t r = check_launch();
         if (r != DMR_OK || S == 0) return r;
