@@ -182,11 +182,14 @@ size_t router_attention_smem(int L, int dh);
 dmr_status_t launch_router_forward(const float *params, const dmr_router_cfg_t &c, const float *Z, const int32_t *lengths, int B,
                                    int L, float *probs, float *scores, int score_class, float *ws, cudaStream_t st);
 
-// The same forward pass as one cooperative launch, for calls of up to this many (padded) tokens; `ws` as above.
+// The same forward pass as one cooperative launch, for calls of up to this many (padded) tokens; `ws` as above, its last kRouterWordBytes
+// hold the kernel's barrier counter and `done` word.  DMR_ERR_UNSUPPORTED: layer by layer is the faster way.  *done: nullptr, or where the
+// number of valid tokens, which the device alone knows, decides, the word that is not 0 if the launch has taken the call.
 constexpr long long kRouterFusedMaxTokens = 4096;
+constexpr size_t kRouterWordBytes = 256;
 bool router_fused_supported(const dmr_router_cfg_t &c, int B, int L);
 dmr_status_t launch_router_fused(const float *params, const dmr_router_cfg_t &c, const float *Z, const int32_t *lengths, int B, int L,
-                                 float *probs, float *scores, int score_class, float *ws, cudaStream_t st);
+                                 float *probs, float *scores, int score_class, float *ws, const int32_t **done, cudaStream_t st);
 
 // One warp waits on a barrier nobody arrives at, with a short limit: *status becomes DMR_ERR_TIMEOUT, *returned 2.
 dmr_status_t launch_wait_timeout_selftest(int32_t *status, int32_t *returned, cudaStream_t st);

@@ -1,5 +1,5 @@
 // The router's forward pass (see router_fwd.cu for the method) as ONE cooperative launch of thread-block clusters, for calls of up
-// to some hundreds of tokens: an agent, or some tens of them, asking for the precision of their next step.
+// to some hundreds of tokens (fused_cost says how many): an agent, or some tens of them, asking for the precision of their next step.
 //
 // What bounds it.  One step of one agent (32 tokens, d = 384, 8 layers) reads 57 MB of parameters for 0.9 GFLOP: 9 us of HBM time.
 // As 58 dependent kernels it took 475 us on the device (580 with their launches): each paid a launch, a cold start and the latency of
@@ -43,11 +43,15 @@ struct FusedArgs {
     float *probs, *scores;
     float *H;              // [T][d] a layer's input, compact token rows
     float *QKV;            // two buffers [T][3 d]
-    uint32_t *counter;     // grid barrier; zero at launch
+    uint32_t *counter;     // grid barrier, then whether this launch takes the call; zero at launch
+    long long limit;       // work (see router_work) up to which it does
     int B, L, d, heads, dh, ffn, layers, l_max, classes, score_class;
     int rq, rd, rf;        // features per CTA of QKV, of the d-wide linears, of the hidden layer (multiples of 4)
     int off_ss, off_as, off_fs, off_par, off_part, off_tab;  // shared memory, in floats
 };
+
+// Tokens times layers: past the keys and values of the last layer there is one token per sequence.
+__host__ __device__ constexpr long long router_work(int layers, long long tokens, int B) { return (layers - 1) * tokens + B; }
 
 __device__ __forceinline__ int seq_len(int n, int L) { return n < 1 ? 1 : (n > L ? L : n); }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
@@ -318,6 +322,8 @@ __global__ void __launch_bounds__(kThreads, 1) router_fused_kernel(const FusedAr
     }
     __syncthreads();
     const int total = start[a.B];
+    if (router_work(a.layers, total, a.B) > a.limit) return;  // every CTA finds the same
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.counter[1] = 1u;
     const int row_lo = (int)((long long)total * cid / clusters), row_hi = (int)((long long)total * (cid + 1) / clusters);
     const int seq_lo = (int)((long long)a.B * cid / clusters), seq_hi = (int)((long long)a.B * (cid + 1) / clusters);
     const size_t buf = (size_t)a.B * a.L * 3 * d;
@@ -652,9 +658,24 @@ bool router_fused_supported(const dmr_router_cfg_t &c, int B, int L) {
     return fused_plan(c, B, L).smem <= 227 * 1024;
 }
 
-// ws: H [T][d], then two buffers of QKV [T][3 d], then the barrier's counter (7 T d floats and 256 bytes).
+// What either way takes, us.  A cluster takes its tokens in blocks of 32, and a block's steps through a layer cost about 28 us and 20 us per
+// million of the layer's weights, whatever the chip could do at once; a layer's kernels cost about their sums' length in launches and latency
+// and then 38 TFLOP/s of ALL tokens, the padded ones too.  Measured, one launch against layer by layer: d = 384, ffn 1536, 8 layers: 1024 tokens 2069 /
+// 1890, 2048 of which half are padding 2150 / 2892, none 4066; d = 96, ffn 96, 12 layers: 256 tokens 497 / 592, 512 tokens 815 / 613, 4096
+// 5568 / 937; d = 64, ffn 128, 2 layers: 512 tokens 102 / 107, 1024 tokens 167 / 118.
+struct FusedCost {
+    double layered, base, per_work;  // layer by layer; one launch: base + per_work * router_work()
+};
+FusedCost fused_cost(const dmr_router_cfg_t &c, long long T, int clusters) {
+    const double d = c.d, f = c.ffn, weights = (4.0 * d * d + 2.0 * d * f) * 1e-6;  // of a layer, millions
+    return {8.0 + c.layers * (30.0 + 0.055 * (3.0 * d + f) + (double)T * weights / 19.0), 20.0 + c.layers * (9.5 + 5.5 * weights),
+            (28.0 + 20.0 * weights) / (kTokBlock * clusters)};
+}
+
+// ws: H [T][d], then two buffers of QKV [T][3 d]; the words at its end.
 dmr_status_t launch_router_fused(const float *params, const dmr_router_cfg_t &c, const float *Z, const int32_t *lengths, int B, int L,
-                                 float *probs, float *scores, int score_class, float *ws, cudaStream_t st) {
+                                 float *probs, float *scores, int score_class, float *ws, const int32_t **done, cudaStream_t st) {
+    *done = nullptr;
     FusedPlan p = fused_plan(c, B, L);
     FusedArgs &a = p.a;
     const size_t T = (size_t)B * L;
@@ -666,7 +687,7 @@ dmr_status_t launch_router_fused(const float *params, const dmr_router_cfg_t &c,
     a.score_class = score_class;
     a.H = ws;
     a.QKV = ws + T * c.d;
-    a.counter = reinterpret_cast<uint32_t *>(ws + 7 * T * c.d);
+    a.counter = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(ws) + router_workspace_bytes(c, B, L) - kRouterWordBytes);
     FusedKernel kernel = fused_kernel(a.dh);
     static std::atomic<int> max_clusters[64][4];  // per device and kernel, at the largest shared memory: 0 = not asked yet
     int dev = 0;
@@ -678,9 +699,18 @@ dmr_status_t launch_router_fused(const float *params, const dmr_router_cfg_t &c,
         if (most < 1) return DMR_ERR_UNSUPPORTED;
         known.store(most);
     }
+    const FusedCost cost = fused_cost(c, (long long)T, most);
+    a.limit = cost.layered > cost.base ? (long long)((cost.layered - cost.base) / cost.per_work) : 0;
+    const bool sure = router_work(c.layers, (long long)T, B) <= a.limit;
+    if (!sure) {
+        // The lengths may decide, on the device: the kernels of the other way are enqueued behind this one and return at once where it has taken the
+        // call.  That is worth their microsecond each where sequences of evenly spread lengths, half the work of full ones, gain a tenth.
+        const long long even = router_work(c.layers, ((long long)T + B) / 2, B);
+        if (even > a.limit || cost.base + cost.per_work * (double)even + 1.3 * (2 + 7 * c.layers) > 0.9 * cost.layered) return DMR_ERR_UNSUPPORTED;
+    }
     int clusters = (int)((T + 3) / 4);  // a task meets four tokens at a time
     if (clusters > most) clusters = most;
-    cudaError_t e = cudaMemsetAsync(a.counter, 0, 256, st);
+    cudaError_t e = cudaMemsetAsync(a.counter, 0, kRouterWordBytes, st);
     if (e != cudaSuccess) return launch_failed(e);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * kCs), 1, 1);
@@ -697,6 +727,7 @@ dmr_status_t launch_router_fused(const float *params, const dmr_router_cfg_t &c,
     cfg.numAttrs = 2;
     e = cudaLaunchKernelEx(&cfg, kernel, a);
     if (e != cudaSuccess) return launch_failed(e);
+    if (!sure) *done = reinterpret_cast<const int32_t *>(a.counter + 1);
     return check_launch();
 }
 

@@ -13,8 +13,8 @@
 // Arithmetic: fp32 throughout (CUDA cores; fused multiply-adds), so that the probabilities agree with a binary64
 // evaluation to about 1e-6 and the comparison against a threshold is stable.  The model is small (14 M parameters at
 // d = 384 and 8 layers) and runs once per agent step, next to a language-model call of tens of milliseconds.
-// Calls of up to kRouterFusedMaxTokens tokens with a head width of 16, 32, 64 or 128 are one launch (router_fused.cu); this file has the
-// layer-by-layer kernels for the others: positions added; per layer a linear (QKV; tiled, or one feature per warp when there are at
+// Calls with a head width of 16, 32, 64 or 128 and not too many tokens are one launch (router_fused.cu, which says how many); this file has the
+// layer-by-layer kernels for the others, which return at once where that launch has found few enough valid tokens: positions added; per layer a linear (QKV; tiled, or one feature per warp when there are at
 // most 32 tokens), one CTA per (sequence, head) for the attention, a linear with the residual added, a layer norm, two linears (ReLU;
 // residual), a layer norm; then pooling, head and softmax.
 #include "sm100.cuh"
@@ -28,10 +28,18 @@ constexpr float kLnEps = 1e-5f;
 // Lengths come from the caller's device memory and are not checked on the host: keep every index in range.
 __device__ __forceinline__ int valid_len(int n, int L) { return n < 1 ? 1 : (n > L ? L : n); }
 
+// Waits for the kernel before this one (all are launched as programmatic dependents: 58 that have nothing to do take 60 us instead of 155);
+// whether the one-launch kernel has taken the call (done: the word it writes; nullptr: it was not asked).
+__device__ __forceinline__ bool answered(const int32_t *done) {
+    pdl_wait();
+    return done && *done != 0;
+}
+
 // H[b][l][:] = Z[b][l][:] + P[l][:] for the valid steps, zero behind them.
 __global__ void __launch_bounds__(256) router_embed_kernel(const float *__restrict__ Z, const float *__restrict__ pos,
                                                            const int32_t *__restrict__ lengths, int B, int L, int d,
-                                                           float *__restrict__ H) {
+                                                           float *__restrict__ H, const int32_t *done) {
+    if (answered(done)) return;
     const long long total = (long long)B * L * (d / 4);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
         const int c4 = (int)(i % (d / 4));
@@ -53,7 +61,8 @@ constexpr int LBM = 64, LBN = 64, LBK = 16;
 template <bool RELU, bool RESID>
 __global__ void __launch_bounds__(256) router_linear_kernel(const float *__restrict__ X, const float *__restrict__ W,
                                                             const float *__restrict__ bias, const float *__restrict__ R,
-                                                            int T, int N, int K, float *__restrict__ Y) {
+                                                            int T, int N, int K, float *__restrict__ Y, const int32_t *done) {
+    if (answered(done)) return;
     __shared__ float xs[LBK][LBM + 4];
     __shared__ float ws[LBK][LBN + 4];
     const int t0 = blockIdx.y * LBM, n0 = blockIdx.x * LBN;
@@ -113,7 +122,8 @@ constexpr int kSmallT = 32;
 template <bool RELU, bool RESID>
 __global__ void __launch_bounds__(256) router_linear_small_kernel(const float *__restrict__ X, const float *__restrict__ W,
                                                                   const float *__restrict__ bias, const float *__restrict__ R,
-                                                                  int T, int N, int K, float *__restrict__ Y) {
+                                                                  int T, int N, int K, float *__restrict__ Y, const int32_t *done) {
+    if (answered(done)) return;
     __shared__ float part[2][4][kSmallT];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int f = warp >> 2, ks = warp & 3;
@@ -158,7 +168,8 @@ __global__ void __launch_bounds__(256) router_linear_small_kernel(const float *_
 constexpr int kAttWarps = 4, kAttMaxL = 128;
 __global__ void __launch_bounds__(kAttWarps * 32) router_attention_kernel(const float *__restrict__ QKV,
                                                                           const int32_t *__restrict__ lengths, int L, int d,
-                                                                          int dh, float *__restrict__ O) {
+                                                                          int dh, float *__restrict__ O, const int32_t *done) {
+    if (answered(done)) return;
     extern __shared__ float att_smem[];
     const int b = blockIdx.x, h = blockIdx.y;
     const int n = valid_len(lengths[b], L);
@@ -226,7 +237,8 @@ __global__ void __launch_bounds__(kAttWarps * 32) router_attention_kernel(const 
 // One warp per token: H[t][:] = (x - mean) / sqrt(var + eps) * g + b over the d features of S[t][:] (d <= 1024).
 __global__ void __launch_bounds__(256) router_layernorm_kernel(const float *__restrict__ S, const float *__restrict__ g,
                                                                const float *__restrict__ bta, int T, int d,
-                                                               float *__restrict__ H) {
+                                                               float *__restrict__ H, const int32_t *done) {
+    if (answered(done)) return;
     const int t = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (t >= T) return;
@@ -262,7 +274,8 @@ __global__ void __launch_bounds__(256) router_layernorm_kernel(const float *__re
 __global__ void __launch_bounds__(32) router_head_kernel(const float *__restrict__ H, const int32_t *__restrict__ lengths,
                                                          const float *__restrict__ wc, const float *__restrict__ bc, int L,
                                                          int d, int classes, int score_class, float *__restrict__ probs,
-                                                         float *__restrict__ scores) {
+                                                         float *__restrict__ scores, const int32_t *done) {
+    if (answered(done)) return;
     const int b = blockIdx.x, lane = threadIdx.x;
     const float *hstar = H + ((size_t)b * L + (valid_len(lengths[b], L) - 1)) * d;
     float mine = -INFINITY;  // lane c keeps the logit of class c
@@ -287,12 +300,12 @@ __global__ void __launch_bounds__(32) router_head_kernel(const float *__restrict
 
 template <bool RELU, bool RESID>
 dmr_status_t launch_linear(const float *X, const float *W, const float *bias, const float *R, int T, int N, int K, float *Y,
-                           cudaStream_t st) {
+                           const int32_t *done, cudaStream_t st) {
     if (T <= kSmallT) {
-        router_linear_small_kernel<RELU, RESID><<<(N + 1) / 2, 256, 0, st>>>(X, W, bias, R, T, N, K, Y);
+        (void)launch_pdl(router_linear_small_kernel<RELU, RESID>, dim3((unsigned)((N + 1) / 2)), dim3(256), 0, st, X, W, bias, R, T, N, K, Y, done);
     } else {
         dim3 grid((unsigned)((N + LBN - 1) / LBN), (unsigned)((T + LBM - 1) / LBM), 1);
-        router_linear_kernel<RELU, RESID><<<grid, 256, 0, st>>>(X, W, bias, R, T, N, K, Y);
+        (void)launch_pdl(router_linear_kernel<RELU, RESID>, grid, dim3(256), 0, st, X, W, bias, R, T, N, K, Y, done);
     }
     return check_launch();
 }
@@ -307,18 +320,19 @@ size_t router_param_floats(const dmr_router_cfg_t &c) {
 
 size_t router_workspace_bytes(const dmr_router_cfg_t &c, int B, int L) {
     const size_t T = (size_t)B * L;
-    const size_t fused = 7 * T * (size_t)c.d * sizeof(float) + 256;  // input rows, two buffers of QKV, a counter
+    const size_t fused = 7 * T * (size_t)c.d * sizeof(float);  // input rows, two buffers of QKV
     const size_t layered = T * (size_t)(6 * c.d + c.ffn) * sizeof(float);
-    return round_up(fused > layered ? fused : layered, 256);
+    return round_up(fused > layered ? fused : layered, 256) + kRouterWordBytes;  // the words lie behind what either way writes
 }
 
 size_t router_attention_smem(int L, int dh) { return ((size_t)2 * L * (dh + 1) + (size_t)kAttWarps * L + (size_t)kAttWarps * dh) * sizeof(float); }
 
 dmr_status_t launch_router_forward(const float *params, const dmr_router_cfg_t &c, const float *Z, const int32_t *lengths, int B,
                                    int L, float *probs, float *scores, int score_class, float *ws, cudaStream_t st) {
+    const int32_t *done = nullptr;
     if (router_fused_supported(c, B, L)) {
-        const dmr_status_t rf = launch_router_fused(params, c, Z, lengths, B, L, probs, scores, score_class, ws, st);
-        if (rf != DMR_ERR_UNSUPPORTED) return rf;
+        const dmr_status_t rf = launch_router_fused(params, c, Z, lengths, B, L, probs, scores, score_class, ws, &done, st);
+        if (rf != DMR_ERR_UNSUPPORTED && (rf != DMR_OK || !done)) return rf;
     }
     const int d = c.d, f = c.ffn, T = B * L, dh = c.d / c.heads;
     float *H = ws;                        // [T][d]   the layer's input and output
@@ -333,7 +347,7 @@ dmr_status_t launch_router_forward(const float *params, const dmr_router_cfg_t &
         const long long total = (long long)T * (d / 4);
         long long blocks = (total + 255) / 256;
         if (blocks > 148 * 16) blocks = 148 * 16;
-        router_embed_kernel<<<(int)blocks, 256, 0, st>>>(Z, params, lengths, B, L, d, H);
+        router_embed_kernel<<<(int)blocks, 256, 0, st>>>(Z, params, lengths, B, L, d, H, done);
         if ((r = check_launch()) != DMR_OK) return r;
     }
     const float *p = params + (size_t)c.l_max * d;
@@ -343,21 +357,21 @@ dmr_status_t launch_router_forward(const float *params, const dmr_router_cfg_t &
         const float *ln1_g = bo + d, *ln1_b = ln1_g + d, *w1 = ln1_b + d, *b1 = w1 + (size_t)f * d;
         const float *w2 = b1 + f, *b2 = w2 + (size_t)d * f, *ln2_g = b2 + d, *ln2_b = ln2_g + d;
         p = ln2_b + d;
-        if ((r = launch_linear<false, false>(H, wqkv, bqkv, nullptr, T, 3 * d, d, QKV, st)) != DMR_OK) return r;
+        if ((r = launch_linear<false, false>(H, wqkv, bqkv, nullptr, T, 3 * d, d, QKV, done, st)) != DMR_OK) return r;
         // few sequences: split a sequence's query rows over several CTAs (each loads the head's keys and values again)
         int zsplit = (4 * 148) / (B * c.heads);
         zsplit = zsplit < 1 ? 1 : (zsplit > (L + kAttWarps - 1) / kAttWarps ? (L + kAttWarps - 1) / kAttWarps : zsplit);
-        router_attention_kernel<<<dim3((unsigned)B, (unsigned)c.heads, (unsigned)zsplit), kAttWarps * 32, att_smem, st>>>(QKV, lengths, L, d, dh, ATT);
+        (void)launch_pdl(router_attention_kernel, dim3((unsigned)B, (unsigned)c.heads, (unsigned)zsplit), dim3(kAttWarps * 32), att_smem, st, (const float *)QKV, lengths, L, d, dh, ATT, done);
         if ((r = check_launch()) != DMR_OK) return r;
-        if ((r = launch_linear<false, true>(ATT, wo, bo, H, T, d, d, SUM, st)) != DMR_OK) return r;
-        router_layernorm_kernel<<<ln_blocks, 256, 0, st>>>(SUM, ln1_g, ln1_b, T, d, H);
+        if ((r = launch_linear<false, true>(ATT, wo, bo, H, T, d, d, SUM, done, st)) != DMR_OK) return r;
+        (void)launch_pdl(router_layernorm_kernel, dim3((unsigned)ln_blocks), dim3(256), 0, st, (const float *)SUM, ln1_g, ln1_b, T, d, H, done);
         if ((r = check_launch()) != DMR_OK) return r;
-        if ((r = launch_linear<true, false>(H, w1, b1, nullptr, T, f, d, FF, st)) != DMR_OK) return r;
-        if ((r = launch_linear<false, true>(FF, w2, b2, H, T, d, f, SUM, st)) != DMR_OK) return r;
-        router_layernorm_kernel<<<ln_blocks, 256, 0, st>>>(SUM, ln2_g, ln2_b, T, d, H);
+        if ((r = launch_linear<true, false>(H, w1, b1, nullptr, T, f, d, FF, done, st)) != DMR_OK) return r;
+        if ((r = launch_linear<false, true>(FF, w2, b2, H, T, d, f, SUM, done, st)) != DMR_OK) return r;
+        (void)launch_pdl(router_layernorm_kernel, dim3((unsigned)ln_blocks), dim3(256), 0, st, (const float *)SUM, ln2_g, ln2_b, T, d, H, done);
         if ((r = check_launch()) != DMR_OK) return r;
     }
-    router_head_kernel<<<B, 32, 0, st>>>(H, lengths, p, p + (size_t)c.classes * d, L, d, c.classes, score_class, probs, scores);
+    (void)launch_pdl(router_head_kernel, dim3((unsigned)B), dim3(32), 0, st, (const float *)H, lengths, p, p + (size_t)c.classes * d, L, d, c.classes, score_class, probs, scores, done);
     return check_launch();
 }
 

@@ -69,3 +69,26 @@ def test_features_that_some_ctas_have_none_of_after_a_kernel_that_left_nans(ffn)
         dmr.dmr_dense_linear(X, W)
         got, _ = dmr.dmr_router_forward(params, cfg, Zd, nd)
         assert np.abs(got.cpu().numpy() - want).max() <= TOL
+
+
+@pytest.mark.parametrize("cfg_kw,B,L,ways", [
+    (dict(d=96, heads=6, ffn=96, layers=12, l_max=64, classes=2), 8, 32, 1),     # few tokens: one launch
+    (dict(d=96, heads=6, ffn=96, layers=12, l_max=64, classes=2), 8, 64, 0),     # layer by layer
+    (dict(d=256, heads=4, ffn=1024, layers=6, l_max=64, classes=2), 16, 64, 2),  # one launch or layer by layer, as the lengths are
+    (dict(d=64, heads=4, ffn=128, layers=2, l_max=64, classes=3), 16, 64, 0),
+    (dict(d=384, heads=6, ffn=1536, layers=8, l_max=64, classes=2), 24, 64, 2),
+])
+def test_choice_between_one_launch_and_layer_by_layer(cfg_kw, B, L, ways):
+    """Both ways of a call whose lengths decide between them, in turn on one workspace; which kernels are enqueued depends on the sizes only."""
+    cfg = RouterCfg(**cfg_kw)
+    p = inputs.router_params(**cfg_kw, seed=B)
+    Z = inputs.router_embeddings(B, L, cfg_kw["d"], seed=L)
+    params, Zd = dmr.pack_router_params(p, cfg), torch.from_numpy(Z).cuda()
+    ws = torch.full((dmr.lib().dmr_router_workspace_bytes(cfg, B, L),), 255, dtype=torch.uint8, device="cuda")
+    layered = 2 + 7 * cfg_kw["layers"]
+    for n in (np.full(B, L, np.int32), inputs.router_lengths(B, L, seed=L), np.ones(B, np.int32), np.full(B, L, np.int32)):
+        before = dmr.dmr_launch_count()
+        got, _ = dmr.dmr_router_forward(params, cfg, Zd, torch.from_numpy(n).cuda(), workspace=ws)
+        assert dmr.dmr_launch_count() - before == (layered, 1, layered + 1)[ways]
+        few = slice(0, B, max(1, B // 8))  # (sequences do not depend on one another)
+        assert np.abs(got.cpu().numpy()[few] - oracle.router_forward(Z[few], n[few], p, cfg_kw["heads"])).max() <= TOL
