@@ -16,18 +16,19 @@ namespace {
 
 // Workspace layout (all offsets multiples of 256 bytes):
 //   [0, 256)   status word
+//   then       counters of the small-batch and the streaming kernel, one set for each half of a routed call (in every layout)
 //   routed:    counts {n_high, n_low} (256 B), idx_high [M], idx_low [M]
 //   routed, tensor-core path: gathered activations of the low rows [M][K], then of the high rows
-//   split-K:   fp32 partial sums [splits][M][N] (shared by the two halves of a routed call)
-//   decode:    feature-group counters and per-CTA partial sums of the streaming kernel
+//   low-bit, large batches:   prepared activations and their row scales
+//   then       fp32 partial sums: of the shares (small-batch kernel), [splits][M][N] (large batches), per CTA (streaming kernel)
 struct Scratch {
     int32_t *status = nullptr;
     int32_t *counts = nullptr, *idx_high = nullptr, *idx_low = nullptr;
     uint16_t *xg_low = nullptr, *xg_high = nullptr;
     void *prefill_scratch = nullptr;  // prepared fp16 activations and row scales of the prefill kernel
     float *partial = nullptr;
-    int32_t *counters = nullptr, *counters_high = nullptr;  // small-batch kernel: shares of a tile that are done
-    void *stream_scratch = nullptr;  // counters + partial sums of the streaming decode kernel
+    int32_t *counters = nullptr, *counters_high = nullptr;  // small-batch and streaming kernel: shares of a tile that are done
+    void *stream_scratch = nullptr;  // partial sums of the streaming decode kernel
     uint16_t *xg_stream = nullptr;   // routed, decode path: the gathered activation rows of one chunk
     // routed calls run their two halves on two streams: the high-precision half gets its own scratch
     float *partial_high = nullptr;
@@ -81,10 +82,9 @@ Scratch carve(void *workspace, dmr_op_t op, int M, int N, int K, dmr_qformat_t f
     Scratch s;
     char *base = reinterpret_cast<char *>(workspace);
     size_t off = kWsStatusBytes;
-    // at a place of their own in every layout, so that no other call's scratch ever lies on them
     s.counters = reinterpret_cast<int32_t *>(base + off);
-    s.counters_high = s.counters + kSmallMaxTiles;
-    off += 2 * (size_t)kSmallMaxTiles * sizeof(int32_t);
+    s.counters_high = s.counters + kWsCounters;
+    off += 2 * kWsCounters * sizeof(int32_t);
     s.status = reinterpret_cast<int32_t *>(base);
     const int g = format_ok(K, f) ? group_of(K, f) : K;
     const bool low_pair = op != DMR_OP_DENSE_LINEAR && use_pair(M, N, K, f.bits, g);
@@ -212,7 +212,7 @@ dmr_status_t run_lowbit(const uint16_t *X, int M, RowSel sel, const uint32_t *qw
             Xc = ws.xg_stream;
         }
         dmr_status_t r = launch_stream(Xc, mc, s, qweight, scales, zeros, N, K, f.bits, g, Yc, out, ws.stream_scratch,
-                                       ws.status, st, M);
+                                       ws.counters, ws.status, st, M);
         if (r != DMR_OK) return r;
     }
     return DMR_OK;
@@ -257,7 +257,7 @@ dmr_status_t run_dense(const uint16_t *X, int M, RowSel sel, const uint16_t *W, 
             if (rg != DMR_OK) return rg;
             Xc = ws.xg_stream;
         }
-        dmr_status_t r = launch_stream(Xc, mc, s, W, nullptr, nullptr, N, K, 16, K, Yc, out, ws.stream_scratch, ws.status, st, M);
+        dmr_status_t r = launch_stream(Xc, mc, s, W, nullptr, nullptr, N, K, 16, K, Yc, out, ws.stream_scratch, ws.counters, ws.status, st, M);
         if (r != DMR_OK) return r;
     }
     return DMR_OK;

@@ -56,8 +56,11 @@ struct RowSel {
 
 // ---- workspace layout --------------------------------------------------------------------
 // [0, 256)            status word (int32) + padding
-// [256, ...)          routed: counts[2] (+pad to 256), idx_high[Mpad], idx_low[Mpad]
-// then                compacted activations / split-K partial sums, op dependent
+// [256, ...)          counters of the low-precision half (and of calls without halves), then of the high-precision half: at a place of their
+//                     own in every layout, so that no other call's scratch ever lies on them; zero between calls
+// then                routed: counts[2] (+pad to 256), idx_high[Mpad], idx_low[Mpad]
+// then                compacted activations / partial sums, op dependent
+constexpr size_t kWsCounters = 8192;  // words for each half
 constexpr size_t kWsStatusBytes = 256;
 
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -71,13 +74,10 @@ dmr_status_t launch_dequantize(const uint32_t *qweight, const uint16_t *scales, 
                                cudaStream_t st);
 
 // Streaming decode kernel (M <= 32 per launch): persistent, one or two CTAs per SM, weights read once.  `bits` is 4 or 8
-// for packed codes and 16 for bf16 weights.  `scratch` holds stream_scratch_bytes(N) bytes that are
-// zero before the first use (the kernel leaves its counters zeroed again).
+// for packed codes and 16 for bf16 weights.  `scratch` holds stream_scratch_bytes(N) bytes, `counters` kWsCounters words that are zero
+// before and after every call.
 constexpr int kMaxStreamCtas = 512;
-// Feature-group counters sit one per 128-byte line: counts into different groups then never queue up
-// behind each other in the L2.
-constexpr int kCounterStride = 32;  // int32 words between counters
-// Scratch layout: per-CTA partial sums [kMaxStreamCtas][2][16 slots][128 features] fp32 first, the counters after them.
+// Per-CTA partial sums [kMaxStreamCtas][2][16 slots][128 features], fp32.
 constexpr size_t kStreamPartialBytes = (size_t)kMaxStreamCtas * 2 * 16 * 128 * sizeof(float);
 size_t stream_scratch_bytes(int N);
 bool stream_supported(int M, int N, int K, int bits, int g);
@@ -86,7 +86,7 @@ bool stream_supported(int M, int N, int K, int bits, int g);
 // summation order) whichever chunk it falls into - a routed call moves rows between chunks.
 dmr_status_t launch_stream(const uint16_t *X, int M, RowSel sel, const void *weights, const uint16_t *scales,
                            const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out,
-                           void *scratch, int32_t *status, cudaStream_t st, int batch_rows = 0);
+                           void *scratch, int32_t *counters, int32_t *status, cudaStream_t st, int batch_rows = 0);
 
 // Decode kernel for 4-bit codes (M <= 16 per launch): every CTA owns whole output features and streams their codes
 // through warp-private TMA rings; no scratch memory beyond the status word.  sel.idx / sel.count select and
@@ -116,7 +116,7 @@ dmr_status_t launch_prefill(const uint16_t *X, int M, RowSel sel, const void *qw
                             void *scratch, float *partial, int32_t *status, cudaStream_t st);
 
 // Batches of up to 64 rows, and of up to 128 on layers of up to kNarrow features with 4- and 8-bit codes (bits == 0: bf16 weights).  X holds M rows (for a routed call: the gathered rows); `partial` holds
-// small_plan().partial_bytes, `counters` kSmallMaxTiles words that are zero before and after every call.
+// small_plan().partial_bytes, `counters` kWsCounters words that are zero before and after every call.
 constexpr int kSmallMaxTiles = 4096;
 constexpr int kNarrow = 15 * 128;  // k and v projections
 struct SmallPlan {

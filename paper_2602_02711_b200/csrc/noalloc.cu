@@ -12,12 +12,12 @@ namespace dmr {
 
 namespace {
 
-// Limits of the fixed scratch: enough for N <= kNoallocMaxN output features on a GPU with up to
+// Limits of the fixed scratch: enough for N <= kNoallocMaxN output features (512 counters) on a GPU with up to
 // kMaxStreamCtas / 2 SMs.  Every GPU that loads the library holds this array until the process exits.
 constexpr int kNoallocMaxN = 65536;
 constexpr size_t kNoallocStatusBytes = 256;
 constexpr size_t kNoallocScratchBytes =
-    kNoallocStatusBytes + kStreamPartialBytes + (size_t)(kNoallocMaxN / 128) * kCounterStride * sizeof(int32_t);
+    kNoallocStatusBytes + kStreamPartialBytes + kWsCounters * sizeof(int32_t);  // partial sums first: a counter's address never depends on N
 
 // In host code this name is only a handle for cudaGetSymbolAddress, never a device address.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
@@ -84,7 +84,8 @@ dmr_status_t dmr_lowbit_linear_noalloc(const void *X_bf16, int M, const void *qw
     RowSel sel = {nullptr, nullptr, 0};
     return launch_stream(reinterpret_cast<const uint16_t *>(X_bf16), M, sel, qweight, reinterpret_cast<const uint16_t *>(scales),
                          reinterpret_cast<const uint8_t *>(zeros), N, K, f.bits, group_of(K, f), Y, out,
-                         reinterpret_cast<char *>(base) + kNoallocStatusBytes, reinterpret_cast<int32_t *>(base), st);
+                         reinterpret_cast<char *>(base) + kNoallocStatusBytes,
+                         reinterpret_cast<int32_t *>(reinterpret_cast<char *>(base) + kNoallocStatusBytes + kStreamPartialBytes), reinterpret_cast<int32_t *>(base), st);
 }
 
 }  // extern "C"

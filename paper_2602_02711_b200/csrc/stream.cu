@@ -126,7 +126,8 @@ struct StreamArgs {
     const uint8_t *zeros;     // low-bit only
     void *Y;
     float *partial;           // [ctas][2][16 slots][128 features] fp32
-    int32_t *counters;        // [feature groups][kCounterStride], zero on entry and on exit
+    int32_t *counters;        // [feature groups][counter_stride], zero on entry and on exit
+    int counter_stride;
     int32_t *status;
     int M, coff, N, K, g_size;
     int g_shift;              // log2(g_size) when it is a power of two, else -1
@@ -353,18 +354,18 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_cons
         int old0 = 0, old1 = 0;
         if (n_ev > 0) {
             if (!mbar_wait(pub_bar(0), 0u, a.status)) return;
-            old0 = atom_add_acq_rel(a.counters + (size_t)rg0 * kCounterStride, 1);
+            old0 = atom_add_acq_rel(a.counters + (size_t)rg0 * a.counter_stride, 1);
         }
         if (n_ev > 1) {
             if (!mbar_wait(pub_bar(1), 0u, a.status)) return;
-            old1 = atom_add_acq_rel(a.counters + (size_t)rg1 * kCounterStride, 1);
+            old1 = atom_add_acq_rel(a.counters + (size_t)rg1 * a.counter_stride, 1);
         }
         for (int e = 0; e < n_ev; ++e) {
             const int rg = e == 0 ? rg0 : rg1;
             int c_first, c_last;
             sharers(rg, c_first, c_last);
             const bool last = (e == 0 ? old0 : old1) == c_last - c_first;
-            if (last) a.counters[(size_t)rg * kCounterStride] = 0;  // every sharer has counted in: ready for the next call
+            if (last) a.counters[(size_t)rg * a.counter_stride] = 0;  // every sharer has counted in: ready for the next call
             is_last[e] = last ? 1 : 0;
             mbar_arrive(role_bar(e));
         }
@@ -981,7 +982,7 @@ dmr_status_t launch_stream_nt(const CUtensorMap &wmap, const CUtensorMap &xmap, 
 
 size_t stream_scratch_bytes(int N) {
     const size_t groups = (size_t)(N + kTileRows - 1) / kTileRows;
-    return kStreamPartialBytes + groups * kCounterStride * sizeof(int32_t);
+    return kStreamPartialBytes + (groups > kWsCounters ? groups * sizeof(int32_t) : 0);
 }
 
 void stream_plan(int M, int N, int K, int bits, int *tiles, long long *steps, int *cluster) {
@@ -1002,7 +1003,7 @@ bool stream_supported(int M, int N, int K, int bits /*16 = bf16 weights*/, int g
 
 dmr_status_t launch_stream(const uint16_t *X, int M, RowSel sel, const void *weights, const uint16_t *scales,
                            const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out,
-                           void *scratch, int32_t *status, cudaStream_t st, int batch_rows) {
+                           void *scratch, int32_t *counters, int32_t *status, cudaStream_t st, int batch_rows) {
     const int step_k = 1024 / bits;
     StreamArgs a;
     const int call_rows = batch_rows > M ? batch_rows : M;
@@ -1013,11 +1014,15 @@ dmr_status_t launch_stream(const uint16_t *X, int M, RowSel sel, const void *wei
     a.zeros = zeros;
     a.Y = Y;
     const size_t groups = (size_t)(N + kTileRows - 1) / kTileRows;
-    // The partial sums come first (a fixed size) and the counters after them, so that a counter's address never
-    // depends on N: layers of different widths can share one scratch area without one layer's partial sums
-    // landing on words that another layer needs to find zero.
     a.partial = reinterpret_cast<float *>(scratch);
-    a.counters = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(scratch) + kStreamPartialBytes);
+    a.counters = counters;
+    // one counter per 128-byte line, so that counts into different groups never queue up behind each other in the L2, while the lines last
+    for (a.counter_stride = 32; a.counter_stride > 1 && groups * a.counter_stride > kWsCounters;) a.counter_stride /= 2;
+    if (groups > kWsCounters) {  // (more than a million features) behind the partial sums, where other calls' scratch may have been
+        a.counters = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(scratch) + kStreamPartialBytes);
+        const cudaError_t e = cudaMemsetAsync(a.counters, 0, groups * sizeof(int32_t), st);
+        if (e != cudaSuccess) return launch_failed(e);
+    }
     a.status = status;
     a.M = M;
     a.coff = sel.offset;

@@ -86,3 +86,31 @@ def test_calls_one_after_the_other(bits, M):
     for _ in range(20):
         again = [f() for f in layers for _ in range(2)]
         assert all(torch.equal(y, first[i // 2]) for i, y in enumerate(again))
+
+
+def test_one_workspace_for_calls_of_all_kernels():
+    """Zeroed once, a workspace serves calls of any sizes in any order: one kernel's partial sums and gathered rows must not lie on the
+    counters that another one expects to be zero."""
+    def case(op, M, N, K, bits=0, group=0):
+        W, X = to_dev_bf16(inputs.weights(N, K, seed=N)), to_dev_bf16(inputs.activations(M, K, seed=K))
+        q = dmr.dmr_quantize(W, QFormat(bits, group)) if bits else None
+        mask = torch.from_numpy(inputs.precision_mask(M, 0.4, seed=M)).cuda()
+        call = {OP_DENSE: lambda **k: dmr.dmr_dense_linear(X, W, OUT_F32, **k), OP_LOWBIT: lambda **k: dmr.dmr_lowbit_linear(X, q, OUT_F32, **k),
+                OP_ROUTED: lambda **k: dmr.dmr_routed_linear(X, mask, W, q, OUT_F32, **k)}[op]
+        return call, dmr.dmr_workspace_bytes(op, M, N, K, QFormat(bits or 4, group))
+
+    cases = [case(OP_DENSE, 64, 4096, 4096),            # partial sums of 148 shares
+             case(OP_DENSE, 16, 2304, 8200),            # streaming kernel, feature groups shared by CTAs
+             case(OP_LOWBIT, 300, 4096, 11008, 4, 128),  # prepared activations, split along k
+             case(OP_LOWBIT, 8, 4096, 8256, 8, 192),    # streaming kernel
+             case(OP_ROUTED, 64, 1024, 5120, 4, 128),
+             case(OP_ROUTED, 20, 2304, 8256, 8, 192),   # streaming kernel, low half
+             case(OP_ROUTED, 20, 2304, 8224, 4, 32),    # streaming kernel, high half
+             case(OP_LOWBIT, 13, 4096, 4096, 8, 0)]
+    want = [call() for call, _ in cases]
+    ws = torch.zeros(max(n for _, n in cases), dtype=torch.uint8, device="cuda")
+    for _ in range(3):
+        for order in (range(len(cases)), reversed(range(len(cases)))):
+            for i in order:
+                assert torch.equal(cases[i][0](workspace=ws), want[i])
+    assert int(ws[:4].view(torch.int32).item()) == 0
