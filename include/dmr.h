@@ -112,7 +112,7 @@ dmr_status_t dmr_dequantize(const void *qweight, const void *scales, const void 
 /*
  * Low-precision linear layer (the W4A16 model's Linear, Sec. 5; also 8-bit and 3-bit codes): Y = X . dequant(Wq)^T
  * with fp32 accumulation.  Up to 16 rows of 3- and 4-bit codes run the decode kernels, larger batches and 8-bit codes the tensor-core
- * kernels.  Kernels of up to 64 rows start fetching qweight, scales and zeros before the preceding kernel
+ * kernels.  Calls of up to 32 rows start fetching qweight, scales and zeros before the preceding kernel
  * of `stream` has finished (programmatic dependent launch): these three must be complete when the
  * call is enqueued, or be written by kernels that do not release their dependents early (dmr_quantize
  * and every ordinary kernel launch qualify).  X may be produced by the preceding kernel.
@@ -124,7 +124,7 @@ dmr_status_t dmr_lowbit_linear(const void *X_bf16, int M, const void *qweight, c
                                void *stream);
 
 /* High-precision linear layer (the bf16 reference model, Sec. 5): Y = X . W^T, fp32 accumulation.  W is fetched ahead of the preceding
- * kernel's end as the codes above are. */
+ * kernel's end as the codes above are, up to 32 rows; larger calls may take another call's output as W. */
 dmr_status_t dmr_dense_linear(const void *X_bf16, int M, const void *W_bf16, int N, int K, void *Y,
                               dmr_out_t out, void *workspace, size_t workspace_bytes, void *stream);
 

@@ -220,7 +220,8 @@ def _out_tensor(M, N, out, device, Y):
 
 def dmr_lowbit_linear(X: torch.Tensor, q: QuantizedLinear, out: int = OUT_BF16, Y=None, workspace=None,
                       stream=None) -> torch.Tensor:
-    """Y = X . dequant(Wq)^T."""
+    """Y = X . dequant(Wq)^T.  Up to 32 rows the codes, scales and zero points are read before the kernel ahead on the stream has ended: they must
+    be complete when the call is made, or come from dmr_quantize or a kernel of another library."""
     L = lib()
     if Y is not None and workspace is not None:
         f = q.fmt
@@ -243,7 +244,8 @@ def dmr_lowbit_linear(X: torch.Tensor, q: QuantizedLinear, out: int = OUT_BF16, 
 
 def dmr_dense_linear(X: torch.Tensor, W: torch.Tensor, out: int = OUT_BF16, Y=None, workspace=None,
                      stream=None) -> torch.Tensor:
-    """Y = X . W^T with bf16 weights."""
+    """Y = X . W^T with bf16 weights.  Up to 32 rows W is read before the kernel ahead on the stream has ended: it must be complete when the call
+    is made, or come from a kernel of another library (not from another call of a linear)."""
     L = lib()
     if Y is not None and workspace is not None:
         r = _calls.dense(X, W, Y, out, workspace, None if stream is None else stream.cuda_stream)
@@ -266,7 +268,7 @@ def dmr_dense_linear(X: torch.Tensor, W: torch.Tensor, out: int = OUT_BF16, Y=No
 
 def dmr_routed_linear(X: torch.Tensor, mask: torch.Tensor, W: torch.Tensor, q: QuantizedLinear,
                       out: int = OUT_BF16, Y=None, workspace=None, stream=None) -> torch.Tensor:
-    """Rows with mask != 0 use the bf16 weights, the others the low-bit weights; Y keeps step order."""
+    """Rows with mask != 0 use the bf16 weights, the others the low-bit weights; Y keeps step order.  Weights as for the two calls above."""
     L = lib()
     if Y is not None and workspace is not None:
         f = q.fmt

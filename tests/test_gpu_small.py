@@ -114,3 +114,22 @@ def test_one_workspace_for_calls_of_all_kernels():
             for i in order:
                 assert torch.equal(cases[i][0](workspace=ws), want[i])
     assert int(ws[:4].view(torch.int32).item()) == 0
+
+
+@pytest.mark.parametrize("M", [33, 48, 64])
+def test_weights_written_by_the_call_before(M):
+    """From 33 rows on a call's weights may be another call's output, which the kernel before still writes when this one's starts (it takes eight
+    of the SMs, so this one finds free ones at once)."""
+    A, B = to_dev_bf16(inputs.activations(64, 1024, seed=1)), to_dev_bf16(inputs.weights(1024, 1024, seed=2))
+    X = to_dev_bf16(inputs.activations(M, 1024, seed=3))
+    W = dmr.dmr_dense_linear(A, B)
+    torch.cuda.synchronize()
+    want = dmr.dmr_dense_linear(X, W, OUT_F32)
+    ws = [dmr.new_workspace(OP_DENSE, 64, 1024, 1024, QFormat(4, 0)) for _ in range(2)]
+    Y = torch.empty_like(want)
+    for _ in range(20):
+        W.zero_()
+        torch.cuda.synchronize()
+        dmr.dmr_dense_linear(A, B, Y=W, workspace=ws[0])
+        dmr.dmr_dense_linear(X, W, OUT_F32, Y=Y, workspace=ws[1])
+        assert torch.equal(Y, want)
