@@ -29,17 +29,13 @@ const at::Tensor *device_tensor(PyObject *o, at::ScalarType type, int dims = -1)
     return t && t->is_cuda() && t->scalar_type() == type && (dims < 0 || t->dim() == dims) && t->is_contiguous() ? t : nullptr;
 }
 
-// Addresses of tensors; false where one has none to give.
+// Addresses of tensors; false where one is missing.
 bool addresses(std::initializer_list<const at::Tensor *> tensors, void **out) {
-    try {
-        for (const at::Tensor *t : tensors) {
-            if (!t) return false;
-            *out++ = t->data_ptr();
-        }
-        return true;
-    } catch (const std::exception &) {
-        return false;
+    for (const at::Tensor *t : tensors) {
+        if (!t) return false;
+        *out++ = t->data_ptr();
     }
+    return true;
 }
 
 // The stream a call is enqueued on: the given handle, or (None) the current one.
@@ -67,8 +63,18 @@ PyObject *refused() {
     return PyLong_FromLong(-1);
 }
 
+// A tensor that cannot say its size, order or address (compressed sparse, symbolic or jagged sizes, no storage) throws when it is asked.
+template <PyObject *take(PyObject *const *, Py_ssize_t)>
+PyObject *guarded(PyObject *, PyObject *const *args, Py_ssize_t n) {
+    try {
+        return take(args, n);
+    } catch (const std::exception &) {
+        return refused();
+    }
+}
+
 template <class F>
-PyObject *call(F f) {  // other Python threads run meanwhile
+PyObject *call(F f) noexcept {  // other Python threads run meanwhile
     int r;
     Py_BEGIN_ALLOW_THREADS
     r = (int)f();
@@ -89,7 +95,7 @@ PyObject *bind(PyObject *, PyObject *const *args, Py_ssize_t n) {
 at::ScalarType out_type(int out) { return out == DMR_OUT_F32 ? at::kFloat : at::kBFloat16; }
 
 // lowbit(X, qweight, scales, zeros, N, K, bits, group, Y, out, workspace, stream)
-PyObject *lowbit(PyObject *, PyObject *const *args, Py_ssize_t n) {
+PyObject *lowbit(PyObject *const *args, Py_ssize_t n) {
     if (n != 12 || !g_lowbit) return refused();
     const at::Tensor *X = device_tensor(args[0], at::kBFloat16, 2), *ws = tensor(args[10]);
     int v[4], out;
@@ -103,7 +109,7 @@ PyObject *lowbit(PyObject *, PyObject *const *args, Py_ssize_t n) {
 }
 
 // dense(X, W, Y, out, workspace, stream)
-PyObject *dense(PyObject *, PyObject *const *args, Py_ssize_t n) {
+PyObject *dense(PyObject *const *args, Py_ssize_t n) {
     if (n != 6 || !g_dense) return refused();
     const at::Tensor *X = device_tensor(args[0], at::kBFloat16, 2), *W = device_tensor(args[1], at::kBFloat16, 2), *ws = tensor(args[4]);
     int out;
@@ -116,7 +122,7 @@ PyObject *dense(PyObject *, PyObject *const *args, Py_ssize_t n) {
 }
 
 // routed(X, mask, W, qweight, scales, zeros, N, K, bits, group, Y, out, workspace, stream)
-PyObject *routed(PyObject *, PyObject *const *args, Py_ssize_t n) {
+PyObject *routed(PyObject *const *args, Py_ssize_t n) {
     if (n != 14 || !g_routed) return refused();
     const at::Tensor *X = device_tensor(args[0], at::kBFloat16, 2), *mask = device_tensor(args[1], at::kByte), *W = device_tensor(args[2], at::kBFloat16, 2);
     const at::Tensor *ws = tensor(args[12]);
@@ -136,9 +142,9 @@ PyObject *routed(PyObject *, PyObject *const *args, Py_ssize_t n) {
 
 PyMethodDef g_methods[] = {
     {"bind", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(bind)), METH_FASTCALL, nullptr},
-    {"lowbit", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(lowbit)), METH_FASTCALL, nullptr},
-    {"dense", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(dense)), METH_FASTCALL, nullptr},
-    {"routed", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(routed)), METH_FASTCALL, nullptr},
+    {"lowbit", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<lowbit>)), METH_FASTCALL, nullptr},
+    {"dense", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<dense>)), METH_FASTCALL, nullptr},
+    {"routed", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<routed>)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };
 PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};
