@@ -269,7 +269,8 @@ dmr_status_t dmr_router_forward(const float *params, dmr_router_cfg_t cfg, const
 dmr_status_t dmr_selftest_wait_timeout(void *workspace, size_t workspace_bytes, void *stream);
 
 /* Reads the status word a previous call may have set in `workspace` (DMR_OK or DMR_ERR_TIMEOUT).
- * Synchronises `stream`. */
+ * Synchronises `stream`.  After DMR_ERR_TIMEOUT the outputs of the calls on that workspace since it was zero-filled are not
+ * valid; the caller zero-fills it (all of it: counters may be left too) before using it again. */
 dmr_status_t dmr_workspace_status(const void *workspace, void *stream);
 
 /*

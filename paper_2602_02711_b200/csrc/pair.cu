@@ -205,6 +205,8 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
                     else if (weights) tma_load_2d(p_tile(s), &map_w, full, BITS == 3 ? kb * (Cfg::P_ROW / 2) : kb * Cfg::P_ROW, n0);
                 }
             }
+            // no copy is left in flight, even where a wait has run out
+            for (uint32_t i = it > (uint32_t)S ? it - (uint32_t)S : 0u; i < it; ++i) (void)mbar_wait(full_bar(i % F), (i / F) & 1, a.status);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -244,6 +246,7 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
                 if (ok && lane == 0) umma2_commit_both(tfull_bar(buf));
                 __syncwarp();
             }
+            if (it > 0) (void)mbar_wait(empty_bar((it - 1) % S), ((it - 1) / S) & 1, a.status);  // no MMA is left in flight
         } else if (BITS == 0 && lane == 0) {
             uint32_t it = 0;
             bool ok = true;

@@ -69,7 +69,6 @@ struct SmallArgs {
     int g_units, half;           // units per quantization group; half: two groups per unit
     uint32_t g_mul;              // group of a tile's unit k = k g_mul / 2^32 (0: k itself)
     int units, k_units;          // in all; per tile
-    int early;                   // the weights may be read before the kernel ahead of this one has ended
     int shares;                  // the units are cut into this many equal shares; a CTA works through one or, in a routed call, two
 };
 
@@ -162,11 +161,13 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
     constexpr int S = Cfg::S, MW = Cfg::MW;
     // Counting a CTA into a shared tile means a fence and the counter's way to the L2 and back, which hold the scale warps up, and with them the
     // MMAs: it is left until all units are done (routed 14B layer, M = 64, 259 us instead of 278; bf16 M = 64 96 instead of 103).  The instances
-    // for few rows of 8-bit codes, whose scale warps have little to do, are the faster for counting at once (32B layer, M = 13, 65 instead of 67).
+    // for few rows of 8-bit codes, whose scale warps have little to do, are the faster for counting at once (M = 1 / 13 / 32, 7B layer 63.5 / 66.4 / 71.3
+    // instead of 66.6 / 68.6 / 74.9, 14B layer 98 / 102 / 112 instead of 103 / 107 / 117, groups of 64 and 128 1 to 3 %).
     constexpr bool COUNT_NOW = BITS == 8 && BN < 64;
     constexpr int W_SCALE = Cfg::UW, W_MMA = Cfg::UW + Cfg::EW, W_COPY = W_MMA + MW;  // first warp of each role
     extern __shared__ uint8_t smem_dyn[];
     __shared__ int shared_tile[kMaxShared], n_shared;  // tiles that this CTA has a part of, later those that it finished last
+    __shared__ int share_range[2], n_all;               // for where a wait has run out: its shares (kept here: registers are short), all such tiles
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -235,6 +236,7 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
     const uint32_t d_cols = 256u / (uint32_t)nd, half_cols = d_cols / 2;
     // this CTA's shares and units (consecutive ones), and the first unit's tile and place in it
     const int share_lo = (int)((uint32_t)a.shares * (uint32_t)cta / (uint32_t)ctas), share_hi = (int)((uint32_t)a.shares * (uint32_t)(cta + 1) / (uint32_t)ctas);
+    if (threadIdx.x == 0) share_range[0] = share_lo, share_range[1] = share_hi;
     const int lo = first_unit(share_lo), hi = first_unit(share_hi);
     const int lo_tile = lo / a.k_units, lo_ku = lo - lo_tile * a.k_units;
 
@@ -242,7 +244,7 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
     // for what the caller's earlier work wrote, they run ahead of the number of rows as well).  Elsewhere that kernel may still be writing them, and
     // they come as far as the L2 (four 7B linears, bf16, 64 rows: 105.5 us without that, 102 with it, 97 if they were copied at once).
     const int first = min(hi - lo, S);
-    if (!a.early) {
+    if (BN >= 64 && !a.count) {
         if (warp == W_COPY && lane == 0) {
             for (int i = 0; i < first; ++i) {
                 const int u = lo + i, tile = u / a.k_units, ku = u - tile * a.k_units;
@@ -459,7 +461,8 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
         int i = 0;  // units done
         uint32_t phases = 0;  // bit w: phase of tfull w
         int tile = lo_tile, ku = lo_ku, share = share_lo, share_end = first_unit(share_lo + 1);
-        for (int u = work ? lo : hi; u < hi;) {
+        int u = work ? lo : hi;
+        while (u < hi) {
             while (share_end <= u) share_end = first_unit(++share + 1);
             const int n = tile * kSm + r, nc = min(n, a.N - 1);
             const int mine = min(share_end - u, a.k_units - ku), ku_end = ku + mine;  // the share's units of the tile
@@ -520,7 +523,10 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
                 if (!ok) break;
                 i += run;
             }
-            if (!ok) break;
+            if (!ok) {
+                if (!COUNT_NOW && warp == W_SCALE && lane == 0) n_shared = -1;  // not all of the shared tiles are listed
+                break;
+            }
             if (mine < a.k_units) {
                 // one of several shares that have units of this tile
                 float *part = slot_of(tile, share) + r;
@@ -555,7 +561,21 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
                 ++tile;
             }
         }
-        if constexpr (!COUNT_NOW) __threadfence();  // the partial sums, before the CTA counts itself
+        // Where a wait has run out (the status says so) the CTA counts itself into its shared tiles all the same, so that the counters are zero again
+        // after the call, and where they meet at each of them the scale warps still do.
+        if constexpr (COUNT_NOW) {
+            while (u < hi) {
+                const int share_of_u = (int)((((uint32_t)u + 1) * (uint32_t)a.shares - 1) / (uint32_t)a.units), t = u / a.k_units;
+                const int next = min(first_unit(share_of_u + 1), (t + 1) * a.k_units), from = max(first_unit(share_of_u), t * a.k_units);
+                if (next - from < a.k_units) {
+                    asm volatile("bar.sync 1, %0;" ::"n"(Cfg::EW * 32) : "memory");
+                    if (warp == W_SCALE && lane == 0) (void)count_in(t);
+                }
+                u = next;
+            }
+        } else {
+            __threadfence();  // the partial sums, before the CTA counts itself
+        }
         __syncwarp();
     }
 
@@ -569,11 +589,22 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
     // layer, M = 64, 311 us instead of 279.)
     if constexpr (!COUNT_NOW) {
         if (n_shared == 0) return;
-        if ((int)threadIdx.x < n_shared && !count_in(shared_tile[threadIdx.x])) shared_tile[threadIdx.x] = -1;
+        if (n_shared < 0) {  // a wait has run out before all of them were listed: list them from the CTA's shares
+            if (threadIdx.x == 0) {
+                n_all = 0;
+                for (int c = share_range[0]; c < share_range[1]; ++c)
+                    for (int u = first_unit(c), next; u < first_unit(c + 1); u = next) {
+                        next = min(first_unit(c + 1), (u / a.k_units + 1) * a.k_units);
+                        if (next - u < a.k_units) shared_tile[n_all++] = u / a.k_units;
+                    }
+            }
+            __syncthreads();
+        }
+        if ((int)threadIdx.x < (n_shared < 0 ? n_all : n_shared) && !count_in(shared_tile[threadIdx.x])) shared_tile[threadIdx.x] = -1;
         __syncthreads();
     }
     constexpr int RW = BN >= 64 ? 4 : BN / 16, CU = BN == 16 ? 8 : BN == 128 ? 2 : 4;  // rows of a warp, and CTAs, at a time (as registers allow)
-    for (int e = 0; e < n_shared; ++e) {
+    for (int e = 0; e < (n_shared < 0 ? n_all : n_shared); ++e) {
         if (shared_tile[e] < 0) continue;
         const int tile = shared_tile[e], n4 = tile * kSm + 4 * lane;
         int c_first, c_last;
@@ -732,7 +763,6 @@ SmallArgs small_args(const SmallPlan &p, int M, RowSel sel, const uint16_t *scal
     a.units = p.units;
     a.k_units = (K + kSk - 1) / kSk;  // (half a unit past the end: zero activations)
     a.shares = p.shares;
-    a.early = M <= 32 || sel.count ? 1 : 0;
     a.G = bits == 0 ? 1 : K / g;
     a.half = bits != 0 && g == 64 ? 1 : 0;
     a.g_units = bits == 0 || g == K ? a.k_units : a.half ? 1 : g / kSk;
