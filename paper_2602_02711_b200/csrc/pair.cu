@@ -37,35 +37,39 @@ constexpr int kPk = 64;          // k per stage
 constexpr int kMaxRows = 256;    // activation rows per tile at most
 constexpr int kRowGroup = 8;     // row tiles visited per feature tile
 
-template <int BITS>  // 0: bf16 weights
+template <int BITS, bool WORDS = false>  // BITS 0: bf16 weights; WORDS: the unpack threads fetch the codes' words from global memory themselves
 struct PairCfg {
     static constexpr int A_BYTES = kPm * kPk * 2;                       // 16 KB
     static constexpr int B_BYTES = kMaxRows / 2 * kPk * 2;              // 16 KB
     // Packed codes of a stage.  A k block of 3-bit codes is 24 bytes a row, which no TMA box can be: two k blocks share a box of 48
-    // bytes, in a slot of its own beside the ring (S / 2 of them).
-    static constexpr int P_ROW = BITS == 3 ? 48 : kPk * BITS / 8;
+    // bytes, in a slot of its own beside the ring (S / 2 of them).  Rows of an odd number of k blocks (no multiple of 16 bytes, so that no tensor map
+    // describes them) are read word by word (WORDS): 2880 x 2880, groups of 64, M = 300 / 700 / 2048 26 / 32 / 58 us (M = 300, 700 on the CUDA cores:
+    // 2680, 6145); 3000 x 4544, M = 200 29.
+    static constexpr bool BOX3 = BITS == 3 && !WORDS;
+    static constexpr int P_ROW = BOX3 ? 48 : WORDS ? 0 : kPk * BITS / 8;
     static constexpr int P_BYTES = BITS == 0 ? 0 : kPm * P_ROW;
-    static constexpr int STAGE = A_BYTES + B_BYTES + (BITS == 3 ? 0 : P_BYTES);
+    static constexpr int STAGE = A_BYTES + B_BYTES + (BOX3 ? 0 : P_BYTES);
     static constexpr int S_RAW = (225 * 1024) / STAGE;
-    static constexpr int S = BITS == 3 ? 6 : S_RAW > 8 ? 8 : S_RAW;
+    static constexpr int S = BOX3 ? 6 : S_RAW > 8 ? 8 : S_RAW;
     // Barriers the copies of the k blocks complete on, in turn.  Where a stage comes round to the unpack groups alternately there are two per
     // stage, so that each is always waited for by the same group, phase after phase: a group that did not wait for the phase before takes
     // a parity it waits for as already there.  (An even number of stages would do too: 8-bit, 32B layer, M = 500, 4 stages for 5: 381 us
     // instead of 345; 3-bit, 7B layer, M = 1024, 4 for 6: 423 instead of 395.)
     static constexpr int F = BITS == 8 || BITS == 3 ? 2 * S : S;
-    static constexpr int RING = S * STAGE + (BITS == 3 ? S / 2 * P_BYTES : 0);
+    static constexpr int RING = S * STAGE + (BOX3 ? S / 2 * P_BYTES : 0);
     static constexpr int UW = BITS == 0 ? 0 : 8;                        // unpack warps
     static constexpr int EW = 8;                                        // epilogue warps
     static constexpr int THREADS = 32 * (2 + UW + EW);
     static constexpr size_t SMEM = (size_t)RING + 1024 /*alignment*/ + 512 /*barriers*/;
     static_assert(SMEM <= 227 * 1024, "stages exceed an SM's shared memory");
-    static_assert(UW == 0 || F / (BITS == 3 ? 2 : 1) % (UW / 4) == 0, "a barrier belongs to one group of unpack warps");
+    static_assert(UW == 0 || F / (BOX3 ? 2 : 1) % (UW / 4) == 0, "a barrier belongs to one group of unpack warps");
     static_assert(S <= 8 && F <= 32, "room for the barriers");
 };
 
 struct PairArgs {
     const uint16_t *scales;
     const uint8_t *zeros;
+    const uint32_t *words;     // 3-bit codes of rows that no tensor map describes
     const float *xscale;       // codes: power of two each prepared activation row was divided by
     void *Y;
     const int32_t *idx;        // routed: output row of batch slot m (nullptr = identity)
@@ -121,11 +125,12 @@ __device__ __forceinline__ TilePos tile_pos(int item, int n_tiles, int m_tiles, 
     return p;
 }
 
-template <int BITS, bool OUT_F32, bool SPLITK>
-__global__ void __launch_bounds__(PairCfg<BITS>::THREADS, 1)
+template <int BITS, bool WORDS, bool OUT_F32, bool SPLITK>
+__global__ void __launch_bounds__(PairCfg<BITS, WORDS>::THREADS, 1)
 pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const PairArgs a) {
-    using Cfg = PairCfg<BITS>;
+    using Cfg = PairCfg<BITS, WORDS>;
     constexpr int S = Cfg::S, F = Cfg::F;
+    constexpr bool BOX3 = Cfg::BOX3;
     extern __shared__ uint8_t smem_dyn[];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -136,7 +141,7 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
     auto a_tile = [&](int s) { return base + (uint32_t)s * Cfg::STAGE; };
     auto b_tile = [&](int s) { return base + (uint32_t)s * Cfg::STAGE + Cfg::A_BYTES; };
     auto p_tile = [&](int s) {
-        return BITS == 3 ? base + (uint32_t)(S * Cfg::STAGE + s / 2 * Cfg::P_BYTES) : base + (uint32_t)s * Cfg::STAGE + Cfg::A_BYTES + Cfg::B_BYTES;
+        return BOX3 ? base + (uint32_t)(S * Cfg::STAGE + s / 2 * Cfg::P_BYTES) : base + (uint32_t)s * Cfg::STAGE + Cfg::A_BYTES + Cfg::B_BYTES;
     };
     const uint32_t bar_base = base + (uint32_t)Cfg::RING;
     auto full_bar = [&](int f) { return bar_base + 256u + 8u * f; };     // this CTA's copies have landed, k block it: f = it % F
@@ -197,12 +202,12 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
                         ok = false;
                         break;
                     }
-                    const bool weights = BITS != 3 || (kb & 1) == 0;  // work items start at an even k block and have an even number of them
+                    const bool weights = !WORDS && (!BOX3 || (kb & 1) == 0);  // work items start at an even k block and have an even number of them
                     const uint32_t full = full_bar(it % F);
                     mbar_expect_tx(full, tx_x + (weights ? tx_w : 0u));
                     tma_load_2d(b_tile(s), &map_x, full, kb * kPk, m0);
                     if constexpr (BITS == 0) tma_load_2d(a_tile(s), &map_w, full, kb * kPk, n0);
-                    else if (weights) tma_load_2d(p_tile(s), &map_w, full, BITS == 3 ? kb * (Cfg::P_ROW / 2) : kb * Cfg::P_ROW, n0);
+                    else if (weights) tma_load_2d(p_tile(s), &map_w, full, BOX3 ? kb * (Cfg::P_ROW / 2) : kb * Cfg::P_ROW, n0);
                 }
             }
             // no copy is left in flight, even where a wait has run out
@@ -279,9 +284,9 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
                 const int kb_lo = k_lo(p), kb_hi = k_hi(p);
                 const int n = min((p.n * 2 + (int)rank) * kPm + r, a.N - 1);
                 UnpackRow<BITS> row;
-                row.begin(a.scales + (size_t)n * G, a.zeros + (size_t)n * G, G, nullptr);
+                row.begin(a.scales + (size_t)n * G, a.zeros + (size_t)n * G, G, WORDS ? a.words + (size_t)n * (a.K / 32 * 3) : nullptr);
                 // a group's k blocks: every NG-th, or (3 bits) both of every NG-th pair
-                constexpr int RUN = BITS == 3 ? 2 : 1;
+                constexpr int RUN = BOX3 ? 2 : 1;
                 int kb = kb_lo + RUN * (int)(((uint32_t)grp_id + (uint32_t)NG - it0 / RUN % (uint32_t)NG) % (uint32_t)NG);
                 auto next_kb = [&](int k) { return RUN == 1 || (k & 1) ? k + RUN * (NG - 1) + 1 : k + 1; };
                 uint32_t w3[12];  // 3-bit codes: a pair's words, in registers when its first k block is handed on
@@ -297,7 +302,7 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
                         break;
                     }
                     const uint32_t src = p_tile(s) + r * Cfg::P_ROW;
-                    if constexpr (BITS == 3) {
+                    if constexpr (BOX3) {
                         if ((kb & 1) == 0) {
 #pragma unroll
                             for (int i = 0; i < 3; ++i)
@@ -390,10 +395,10 @@ pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ C
     }
 }
 
-template <int BITS, bool OUT_F32, bool SPLITK>
+template <int BITS, bool WORDS, bool OUT_F32, bool SPLITK>
 dmr_status_t launch_pair_t(const CUtensorMap &map_w, const CUtensorMap &map_x, const PairArgs &a, int ctas, cudaStream_t st) {
-    using Cfg = PairCfg<BITS>;
-    auto kernel = pair_kernel<BITS, OUT_F32, SPLITK>;
+    using Cfg = PairCfg<BITS, WORDS>;
+    auto kernel = pair_kernel<BITS, WORDS, OUT_F32, SPLITK>;
     if (!ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), Cfg::SMEM)) return DMR_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ctas, 1, 1);
@@ -413,18 +418,18 @@ dmr_status_t launch_pair_t(const CUtensorMap &map_w, const CUtensorMap &map_x, c
     return check_launch();
 }
 
-template <int BITS>
+template <int BITS, bool WORDS = false>
 dmr_status_t launch_pair_bits(const CUtensorMap &map_w, const CUtensorMap &map_x, const PairArgs &a, int ctas, dmr_out_t out, cudaStream_t st) {
-    if (a.splits > 1) return launch_pair_t<BITS, true, true>(map_w, map_x, a, ctas, st);
-    if (out == DMR_OUT_F32) return launch_pair_t<BITS, true, false>(map_w, map_x, a, ctas, st);
-    return launch_pair_t<BITS, false, false>(map_w, map_x, a, ctas, st);
+    if (a.splits > 1) return launch_pair_t<BITS, WORDS, true, true>(map_w, map_x, a, ctas, st);
+    if (out == DMR_OUT_F32) return launch_pair_t<BITS, WORDS, true, false>(map_w, map_x, a, ctas, st);
+    return launch_pair_t<BITS, WORDS, false, false>(map_w, map_x, a, ctas, st);
 }
 
 }  // namespace
 
 bool pair_supported(int M, int N, int K, int bits, int g) {
     (void)N;
-    if (M <= 32 || K % (bits == 3 ? 2 * kPk : kPk) != 0) return false;  // (3-bit codes: rows of whole 48-byte boxes)
+    if (M <= 32 || K % kPk != 0) return false;
     return bits == 0 || ((bits == 3 || bits == 4 || bits == 8) && g % kPk == 0 && K <= 32768);
 }
 
@@ -448,7 +453,7 @@ PairPlan pair_plan(int M, int N, int K, int bits) {
         for (int sp = 1; sp <= 8; ++sp) {
             if (sp > 1 && (tiles >= pairs || nkb / sp < 16)) break;
             int per = (nkb + sp - 1) / sp;
-            if (bits == 3) per = (per + 1) / 2 * 2;  // two k blocks share a box
+            if (bits == 3 && nkb % 2 == 0) per = (per + 1) / 2 * 2;  // two k blocks share a box
             const int splits = (nkb + per - 1) / per;
             const int rounds = (tiles * splits + pairs - 1) / pairs;
             double cost = rounds * (per * kb_cycles + 1500.0);
@@ -478,9 +483,12 @@ dmr_status_t launch_pair(const uint16_t *X, int M, RowSel sel, const float *xsca
                             (uint64_t)K * 2, (uint32_t)(p.rows / 2), kPk, TmaSwizzle::k128B))
         return DMR_ERR_CUDA;
     const uint64_t row_bytes = (uint64_t)K * bits / 8;
+    const bool words = bits == 3 && K % (2 * kPk) != 0;
     if (bits == 0) {
         if (!make_tensor_map_2d(&map_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, weights, (uint64_t)N, (uint64_t)K, (uint64_t)K * 2, kPm, kPk, TmaSwizzle::k128B))
             return DMR_ERR_CUDA;
+    } else if (words) {
+        map_w = map_x;  // (not used)
     } else if (!make_tensor_map_2d(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, weights, (uint64_t)N, row_bytes, row_bytes, kPm,
                                    (uint32_t)(bits == 3 ? 48 : kPk * bits / 8), TmaSwizzle::kNone)) {
         return DMR_ERR_CUDA;
@@ -488,6 +496,7 @@ dmr_status_t launch_pair(const uint16_t *X, int M, RowSel sel, const float *xsca
     PairArgs a = {};
     a.scales = scales;
     a.zeros = zeros;
+    a.words = words ? reinterpret_cast<const uint32_t *>(weights) : nullptr;
     a.xscale = xscale;
     a.Y = Y;
     a.idx = sel.idx;
@@ -504,6 +513,7 @@ dmr_status_t launch_pair(const uint16_t *X, int M, RowSel sel, const float *xsca
     a.kb_per_split = p.kb_per_split;
     dmr_status_t r;
     if (bits == 0) r = launch_pair_bits<0>(map_w, map_x, a, p.ctas, out, st);
+    else if (words) r = launch_pair_bits<3, true>(map_w, map_x, a, p.ctas, out, st);
     else if (bits == 3) r = launch_pair_bits<3>(map_w, map_x, a, p.ctas, out, st);
     else if (bits == 4) r = launch_pair_bits<4>(map_w, map_x, a, p.ctas, out, st);
     else r = launch_pair_bits<8>(map_w, map_x, a, p.ctas, out, st);

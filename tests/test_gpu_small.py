@@ -32,7 +32,7 @@ def test_dense(M, N, K):
                                                                                         (65, 1024, 512, 128), (128, 1920, 384, 64), (100, 250, 576, 192)])
 def test_low_bit(M, N, K, bits, group):
     if bits == 3 and (M > 64 or K % 128 != 0):
-        pytest.skip("other kernels")
+        pytest.skip("the SM-pair kernel (test_gpu_pair.py), or up to 32 rows the one for any shape (test_gpu_w3.py)")
     W, X = inputs.weights(N, K, seed=K), inputs.activations(M, K, seed=N, outlier_frac=0.01)
     q = dmr.dmr_quantize(to_dev_bf16(W), QFormat(bits, group))
     want = oracle.lowbit_linear(X, *oracle.quantize(W, bits=bits, group=group), bits=bits, group=group)
