@@ -74,7 +74,7 @@ int decode_max_m(int bits) {
 // M = 128 148 -> 136; 8-bit 32B layer M = 65 191 -> 155; 3-bit 7B layer M = 128 174 -> 141.)
 bool use_small(int M, int N, int K, int bits, int g) { return M > decode_max_m(bits) && small_supported(M, N, K, bits, g); }
 bool use_pair(int M, int N, int K, int bits, int g) {
-    const bool exact = (bits == 4 || bits == 8) && M <= 128 && N <= kNarrow;
+    const bool exact = (bits == 4 || bits == 8) && M <= kExactRows && N <= kNarrow;
     return M > decode_max_m(bits) && !exact && !use_small(M, N, K, bits, g) && pair_supported(M, N, K, bits, g);
 }
 

@@ -66,8 +66,8 @@ struct SmallArgs {
     int32_t *counters;           // [tiles], zero between calls
     int32_t *status;
     int M, N, K, G;
-    int g_units, half;           // units per quantization group; half: two groups per unit
-    uint32_t g_mul;              // group of a tile's unit k = k g_mul / 2^32 (0: k itself)
+    int g_units, half;           // units per quantization group; half: two groups per unit (or two pieces of 64 inputs of longer ones)
+    uint32_t g_mul;              // group of a tile's unit (half: piece) k = k g_mul / 2^32 (0: k itself)
     int units, k_units;          // in all; per tile
     int shares;                  // the units are cut into this many equal shares; a CTA works through one or, in a routed call, two
 };
@@ -228,6 +228,7 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
         }
     };
     auto group_of = [&](int ku) -> int { return a.g_mul ? (int)__umulhi((uint32_t)ku, a.g_mul) : ku; };
+    auto piece_group = [&](int piece) -> int { return BN >= 64 ? group_of(piece) : piece; };  // (up to 32 rows: groups of 64 only)
     // Unit i of the CTA's share belongs to MMA warp and accumulator i % nd.  A quantization group that ends with its unit is read when the unit
     // is done; a longer one (or a tile of bf16 weights) when all warps are through with their units of it, their accumulators added in order; a
     // group of half a unit has an accumulator of its own beside the other half's.
@@ -377,8 +378,8 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
                 auto zeros_of = [&](uint32_t &z0, uint32_t &z1) {
                     const uint8_t *zp = a.zeros + (size_t)min(tile * kSm + r, a.N - 1) * a.G;
                     if (half_groups) {
-                        z0 = __ldg(zp + 2 * ku);
-                        z1 = __ldg(zp + min(2 * ku + 1, a.G - 1));
+                        z0 = __ldg(zp + piece_group(2 * ku));
+                        z1 = __ldg(zp + min(piece_group(2 * ku + 1), a.G - 1));
                     } else {
                         z0 = z1 = __ldg(zp + group_of(ku));
                     }
@@ -470,13 +471,13 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
 #pragma unroll
             for (int c = 0; c < CW; ++c) acc[c] = 0.f;
             const uint16_t *sp = a.scales + (size_t)nc * a.G;
-            int grp = group_of(ku), left = a.g_units - (ku - grp * a.g_units);  // group, and units left in it
+            int grp = BN >= 64 && half_groups ? ku : group_of(ku), left = a.g_units - (ku - grp * a.g_units);  // group, and units left in it
             uint32_t sb0 = 0, sb1 = 0;
             auto scale_of = [&](int k, int g) {
                 if (BITS == 0) return;
                 if (half_groups) {
-                    sb0 = __ldg(sp + 2 * k);
-                    sb1 = __ldg(sp + min(2 * k + 1, a.G - 1));
+                    sb0 = __ldg(sp + piece_group(2 * k));
+                    sb1 = __ldg(sp + min(piece_group(2 * k + 1), a.G - 1));
                 } else {
                     sb0 = __ldg(sp + g);
                 }
@@ -764,22 +765,29 @@ SmallArgs small_args(const SmallPlan &p, int M, RowSel sel, const uint16_t *scal
     a.k_units = (K + kSk - 1) / kSk;  // (half a unit past the end: zero activations)
     a.shares = p.shares;
     a.G = bits == 0 ? 1 : K / g;
-    a.half = bits != 0 && g == 64 ? 1 : 0;
+    a.half = bits != 0 && g != K && g % kSk != 0 ? 1 : 0;
     a.g_units = bits == 0 || g == K ? a.k_units : a.half ? 1 : g / kSk;
-    a.g_mul = a.g_units > 1 ? (uint32_t)((0x100000000ull + (uint64_t)a.g_units - 1) / (uint64_t)a.g_units) : 0u;  // exact for the unit numbers that occur
+    const int per_group = a.half ? g / 64 : a.g_units;
+    a.g_mul = per_group > 1 ? (uint32_t)((0x100000000ull + (uint64_t)per_group - 1) / (uint64_t)per_group) : 0u;  // exact for the numbers that occur
     return a;
 }
 
 }  // namespace
 
+// 4- and 8-bit codes that pair.cu would round to fp16 where they have always been multiplied exactly: more than 32 rows on narrow layers (k and v
+// projections).
+static bool exact_only(int M, int N, int bits) { return (bits == 4 || bits == 8) && M > 32 && M <= kExactRows && N <= kNarrow; }
+
 bool small_supported(int M, int N, int K, int bits, int g) {
     const int tiles = (N + kSm - 1) / kSm;
-    // narrow layers (k and v projections) with 4- and 8-bit codes: up to 128 rows, so that they are multiplied exactly
-    if (M < 1 || M > ((bits == 4 || bits == 8) && N <= kNarrow ? 128 : 64)) return false;
+    const bool exact = exact_only(M, N, bits);
+    if (M < 1 || (M > 64 && !exact)) return false;
     if (K % (bits == 3 ? kSk : kSk / 2) != 0) return false;  // (3-bit codes: rows of whole 48-byte boxes)
     if (tiles > kSmallMaxTiles || K > 131072) return false;  // (units x shares stay below 2^32)
-    // a unit is one group, part of one, or two; two of 64 have an accumulator each, which is as many as there are
-    return bits == 0 || ((bits == 3 || bits == 4 || bits == 8) && (g % 128 == 0 || g == 64 || g == K));
+    // a unit is one group, part of one, or two pieces of 64 inputs with an accumulator each, which is as many as there are; groups of other odd
+    // multiples of 64 than one take the piecewise way only where nothing else multiplies them exactly (1024 x 960, 4 bits, groups of 320,
+    // M = 48 / 128: 9.6 / 12.5 us, on the CUDA cores 83 / 208)
+    return bits == 0 || ((bits == 3 || bits == 4 || bits == 8) && (g % 128 == 0 || g == 64 || g == K || (exact && g % 64 == 0)));
 }
 
 SmallPlan small_plan(int M, int N, int K) {

@@ -29,11 +29,13 @@ def test_dense(M, N, K):
 
 @pytest.mark.parametrize("bits", [3, 4, 8])
 @pytest.mark.parametrize("M,N,K,group", [s + (g,) for s in SHAPES for g in (64, 0)] + [(20, 700, 1024, 128), (64, 129, 1536, 256), (33, 128, 768, 384),
-                                                                                        (65, 1024, 512, 128), (128, 1920, 384, 64), (100, 250, 576, 192)])
+                                                                                        (65, 1024, 512, 128), (128, 1920, 384, 64), (100, 250, 576, 192),
+                                                                                        (33, 1024, 960, 320), (64, 100, 960, 192), (128, 1920, 2880, 576)])
 def test_low_bit(M, N, K, bits, group):
     if bits == 3 and (M > 64 or K % 128 != 0):
         pytest.skip("the SM-pair kernel (test_gpu_pair.py), or up to 32 rows the one for any shape (test_gpu_w3.py)")
     W, X = inputs.weights(N, K, seed=K), inputs.activations(M, K, seed=N, outlier_frac=0.01)
+    assert M <= 16 or dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, group))["kernel"] != "simple"
     q = dmr.dmr_quantize(to_dev_bf16(W), QFormat(bits, group))
     want = oracle.lowbit_linear(X, *oracle.quantize(W, bits=bits, group=group), bits=bits, group=group)
     Y = dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_F32)
@@ -41,10 +43,9 @@ def test_low_bit(M, N, K, bits, group):
     assert torch.equal(dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_BF16), Y.to(torch.bfloat16))
 
 
-@pytest.mark.parametrize("bits,group", [(4, 128), (4, 64), (8, 0), (3, 128)])
+@pytest.mark.parametrize("bits,group,K", [(4, 128, 1024), (4, 64, 1024), (8, 0, 1024), (3, 128, 1024), (4, 320, 960)])
 @pytest.mark.parametrize("M,high,N", [(2, 1, 700), (16, 5, 128), (17, 0, 700), (40, 40, 130), (64, 63, 700), (64, 20, 2304), (100, 30, 700)])
-def test_routed_rows_equal_unrouted_ones(M, high, N, bits, group):
-    K = 1024
+def test_routed_rows_equal_unrouted_ones(M, high, N, bits, group, K):
     W, X = to_dev_bf16(inputs.weights(N, K, seed=1)), to_dev_bf16(inputs.activations(M, K, seed=2))
     q = dmr.dmr_quantize(W, QFormat(bits, group))
     mask = np.zeros(M, dtype=np.uint8)
