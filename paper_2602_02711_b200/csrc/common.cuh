@@ -115,11 +115,13 @@ dmr_status_t launch_prefill(const uint16_t *X, int M, RowSel sel, const void *qw
                             const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out,
                             void *scratch, float *partial, int32_t *status, cudaStream_t st);
 
-// Batches of up to 64 rows, and of up to kExactRows on layers of up to kNarrow features with 4- and 8-bit codes (bits == 0: bf16 weights).  X holds M rows (for a routed call: the gathered rows); `partial` holds
+// Batches of up to 64 rows; with 4- and 8-bit codes also of up to kExactRows on layers of up to kNarrow features, and of any size, kExactRows a
+// launch, with more than kPairMaxK inputs (bits == 0: bf16 weights).  X holds M rows (for a routed call: the gathered rows); `partial` holds
 // small_plan().partial_bytes, `counters` kWsCounters words that are zero before and after every call.
 constexpr int kSmallMaxTiles = 4096;
 constexpr int kNarrow = 15 * 128;  // k and v projections
 constexpr int kExactRows = 128;
+constexpr int kPairMaxK = 32768;   // inputs of codes that the large batches' activation preparation takes at most
 struct SmallPlan {
     int bn, tiles, units, shares;
     size_t partial_bytes;

@@ -430,7 +430,7 @@ dmr_status_t launch_pair_bits(const CUtensorMap &map_w, const CUtensorMap &map_x
 bool pair_supported(int M, int N, int K, int bits, int g) {
     (void)N;
     if (M <= 32 || K % kPk != 0) return false;
-    return bits == 0 || ((bits == 3 || bits == 4 || bits == 8) && g % kPk == 0 && K <= 32768);
+    return bits == 0 || ((bits == 3 || bits == 4 || bits == 8) && g % kPk == 0 && K <= kPairMaxK);
 }
 
 PairPlan pair_plan(int M, int N, int K, int bits) {

@@ -67,6 +67,7 @@ struct SmallArgs {
     int32_t *status;
     int M, N, K, G;
     int g_units, half;           // units per quantization group; half: two groups per unit (or two pieces of 64 inputs of longer ones)
+    int offset;                  // routed: batch slots before this launch's first one
     uint32_t g_mul;              // group of a tile's unit (half: piece) k = k g_mul / 2^32 (0: k itself)
     int units, k_units;          // in all; per tile
     int shares;                  // the units are cut into this many equal shares; a CTA works through one or, in a routed call, two
@@ -266,7 +267,7 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
     int rows = a.M;
     if (a.count) {
         pdl_wait();
-        rows = min(*a.count, a.M);
+        rows = min(*a.count - a.offset, a.M);
     }
     const bool work = rows > 0;
 
@@ -755,6 +756,7 @@ SmallArgs small_args(const SmallPlan &p, int M, RowSel sel, const uint16_t *scal
     a.Y = Y;
     a.idx = sel.idx;
     a.count = sel.count;
+    a.offset = sel.offset;
     a.partial = partial;
     a.counters = counters;
     a.status = status;
@@ -774,16 +776,20 @@ SmallArgs small_args(const SmallPlan &p, int M, RowSel sel, const uint16_t *scal
 
 }  // namespace
 
-// 4- and 8-bit codes that pair.cu would round to fp16 where they have always been multiplied exactly: more than 32 rows on narrow layers (k and v
-// projections).
-static bool exact_only(int M, int N, int bits) { return (bits == 4 || bits == 8) && M > 32 && M <= kExactRows && N <= kNarrow; }
+// 4- and 8-bit codes that have always been multiplied exactly where pair.cu would round them to fp16, or does not take them: more than 32 rows, up
+// to kExactRows on narrow layers (k and v projections), any number, kExactRows a launch, of rows too long for its activation preparation
+// (4096 x 40960, 4 bits, groups of 128, M = 300: 225 us; 902 in chunks of 16 rows on the decode kernel).
+static bool exact_only(int M, int N, int K, int bits) {
+    return (bits == 4 || bits == 8) && M > 32 && ((N <= kNarrow && M <= kExactRows) || K > kPairMaxK);
+}
 
 bool small_supported(int M, int N, int K, int bits, int g) {
-    const int tiles = (N + kSm - 1) / kSm;
-    const bool exact = exact_only(M, N, bits);
+    const long long tiles = ((long long)N + kSm - 1) / kSm, k_units = ((long long)K + kSk - 1) / kSk;
+    const bool exact = exact_only(M, N, K, bits);
     if (M < 1 || (M > 64 && !exact)) return false;
     if (K % (bits == 3 ? kSk : kSk / 2) != 0) return false;  // (3-bit codes: rows of whole 48-byte boxes)
-    if (tiles > kSmallMaxTiles || K > 131072) return false;  // (units x shares stay below 2^32)
+    // units x shares stay below 2^32, pieces of 64 inputs where the multiplication that finds their group is exact
+    if (tiles > kSmallMaxTiles || k_units > 16384 || tiles * k_units * device_sm_count() >= 0x100000000ll) return false;
     // a unit is one group, part of one, or two pieces of 64 inputs with an accumulator each, which is as many as there are; groups of other odd
     // multiples of 64 than one take the piecewise way only where nothing else multiplies them exactly (1024 x 960, 4 bits, groups of 320,
     // M = 48 / 128: 9.6 / 12.5 us, on the CUDA cores 83 / 208)
@@ -803,14 +809,27 @@ SmallPlan small_plan(int M, int N, int K) {
 
 dmr_status_t launch_small(const uint16_t *X, int M, RowSel sel, const void *weights, const uint16_t *scales, const uint8_t *zeros, int N, int K,
                           int bits, int g, void *Y, dmr_out_t out, float *partial, int32_t *counters, int32_t *status, cudaStream_t st) {
-    const SmallPlan p = small_plan(M, N, K);
-    SmallMaps m;
-    if (!small_maps(&m, X, M, weights, N, K, bits, p.bn)) return DMR_ERR_CUDA;
-    const SmallArgs a = small_args(p, M, sel, scales, zeros, N, K, bits, g, Y, partial, counters, status);
-    if (bits == 0) return launch_small_bits<0>(p.bn, m.w, m.x, a, p.shares, out, st);
-    if (bits == 3) return launch_small_bits<3>(p.bn, m.w, m.x, a, p.shares, out, st);
-    if (bits == 4) return launch_small_bits<4>(p.bn, m.w, m.x, a, p.shares, out, st);
-    return launch_small_bits<8>(p.bn, m.w, m.x, a, p.shares, out, st);
+    const SmallPlan p = small_plan(M, N, K);  // (one tile of rows for all launches: a row's sums do not depend on the launch it is in)
+    for (int m0 = 0; m0 < M; m0 += kExactRows) {
+        const int rows = M - m0 < kExactRows ? M - m0 : kExactRows;
+        RowSel s = sel;
+        void *Yc = Y;
+        if (sel.idx) {
+            s.idx = sel.idx + m0;
+            s.offset = sel.offset + m0;
+        } else {
+            Yc = reinterpret_cast<char *>(Y) + (size_t)m0 * N * (out == DMR_OUT_F32 ? 4 : 2);
+        }
+        SmallMaps m;
+        if (!small_maps(&m, X + (size_t)m0 * K, rows, weights, N, K, bits, p.bn)) return DMR_ERR_CUDA;
+        const SmallArgs a = small_args(p, rows, s, scales, zeros, N, K, bits, g, Yc, partial, counters, status);
+        const dmr_status_t r = bits == 0   ? launch_small_bits<0>(p.bn, m.w, m.x, a, p.shares, out, st)
+                               : bits == 3 ? launch_small_bits<3>(p.bn, m.w, m.x, a, p.shares, out, st)
+                               : bits == 4 ? launch_small_bits<4>(p.bn, m.w, m.x, a, p.shares, out, st)
+                                           : launch_small_bits<8>(p.bn, m.w, m.x, a, p.shares, out, st);
+        if (r != DMR_OK) return r;
+    }
+    return DMR_OK;
 }
 
 dmr_status_t launch_small_routed(const uint16_t *Xh, const uint16_t *Xl, int M, RowSel high, RowSel low, const uint16_t *W, const void *qweight,

@@ -134,3 +134,19 @@ def test_weights_written_by_the_call_before(M):
         dmr.dmr_dense_linear(A, B, Y=W, workspace=ws[0])
         dmr.dmr_dense_linear(X, W, OUT_F32, Y=Y, workspace=ws[1])
         assert torch.equal(Y, want)
+
+
+@pytest.mark.parametrize("bits,group", [(4, 128), (4, 64), (8, 320), (8, 0)])
+@pytest.mark.parametrize("M,N", [(40, 2000), (65, 300), (128, 2000), (300, 130)])
+def test_rows_longer_than_the_large_batches_take(M, N, bits, group):
+    """More than 32768 inputs: exact for any number of rows, in launches of 128; routed rows are the unrouted ones whichever launch they fall into."""
+    K = 40960
+    assert dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, group))["kernel"] not in ("simple", "stream", "decode_w4")
+    W, X = inputs.weights(N, K, seed=N), inputs.activations(M, K, seed=M, outlier_frac=0.01)
+    q, Xd, Wd = dmr.dmr_quantize(to_dev_bf16(W), QFormat(bits, group)), to_dev_bf16(X), to_dev_bf16(W)
+    Y = dmr.dmr_lowbit_linear(Xd, q, OUT_F32)
+    want = Xd.double() @ dmr.dmr_dequantize(q).double().T
+    assert float((Y.double() - want).abs().max() / want.abs().max()) <= TOL
+    mask = torch.from_numpy(inputs.precision_mask(M, 0.4, seed=M)).cuda()
+    Yr = dmr.dmr_routed_linear(Xd, mask, Wd, q, OUT_F32)
+    assert torch.equal(Yr, torch.where(mask[:, None] != 0, dmr.dmr_dense_linear(Xd, Wd, OUT_F32), Y))
