@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 from dataclasses import dataclass
 
 import torch
@@ -106,9 +107,10 @@ def lib() -> ctypes.CDLL:
     L.dmr_launch_count.restype = ctypes.c_uint64
     try:
         from . import _calls as calls
-    except ImportError as e:
-        raise DmrError(-1, f"{e}: run `python -m paper_2602_02711_b200.build`") from e
-    calls.bind(*(ctypes.cast(getattr(L, f), vp).value for f in ("dmr_lowbit_linear", "dmr_dense_linear", "dmr_routed_linear")))
+        calls.bind(*(ctypes.cast(getattr(L, f), vp).value for f in ("dmr_lowbit_linear", "dmr_dense_linear", "dmr_routed_linear")))
+    except ImportError as e:  # the same calls through ctypes
+        calls = None
+        warnings.warn(f"{e}: the linears' calls take about twice as long on the host; run `python -m paper_2602_02711_b200.build`")
     _calls, _lib = calls, L
     return L
 
@@ -223,7 +225,7 @@ def dmr_lowbit_linear(X: torch.Tensor, q: QuantizedLinear, out: int = OUT_BF16, 
     """Y = X . dequant(Wq)^T.  Up to 32 rows the codes, scales and zero points are read before the kernel ahead on the stream has ended: they must
     be complete when the call is made, or come from dmr_quantize or a kernel of another library."""
     L = lib()
-    if Y is not None and workspace is not None:
+    if Y is not None and workspace is not None and _calls is not None:
         f = q.fmt
         r = _calls.lowbit(X, q.qweight, q.scales, q.zeros, q.N, q.K, f.bits, f.group_size, Y, out, workspace, None if stream is None else stream.cuda_stream)
         if r >= 0:
@@ -247,7 +249,7 @@ def dmr_dense_linear(X: torch.Tensor, W: torch.Tensor, out: int = OUT_BF16, Y=No
     """Y = X . W^T with bf16 weights.  Up to 32 rows W is read before the kernel ahead on the stream has ended: it must be complete when the call
     is made, or come from a kernel of another library (not from another call of a linear)."""
     L = lib()
-    if Y is not None and workspace is not None:
+    if Y is not None and workspace is not None and _calls is not None:
         r = _calls.dense(X, W, Y, out, workspace, None if stream is None else stream.cuda_stream)
         if r >= 0:
             if r:
@@ -270,7 +272,7 @@ def dmr_routed_linear(X: torch.Tensor, mask: torch.Tensor, W: torch.Tensor, q: Q
                       out: int = OUT_BF16, Y=None, workspace=None, stream=None) -> torch.Tensor:
     """Rows with mask != 0 use the bf16 weights, the others the low-bit weights; Y keeps step order.  Weights as for the two calls above."""
     L = lib()
-    if Y is not None and workspace is not None:
+    if Y is not None and workspace is not None and _calls is not None:
         f = q.fmt
         r = _calls.routed(X, mask, W, q.qweight, q.scales, q.zeros, q.N, q.K, f.bits, f.group_size, Y, out, workspace, None if stream is None else stream.cuda_stream)
         if r >= 0:

@@ -1,5 +1,5 @@
 """The linears' native marshalling away from a GPU: tensors that cannot say their size or address are refused with -1, for the Python code to
-name the error, and end no process."""
+name the error, and end no process; without the module the library loads all the same."""
 import os
 import subprocess
 import sys
@@ -34,3 +34,18 @@ with FakeTensorMode(shape_env=env):  # tensors on a GPU, as far as anyone can as
 def test_arguments_that_throw_are_refused():
     r = subprocess.run([sys.executable, "-c", SCRIPT], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, (r.stdout.split()[-1:], r.stderr[-2000:])
+
+
+def test_the_library_loads_without_the_module():
+    script = """
+import sys, warnings
+sys.modules["paper_2602_02711_b200._calls"] = None  # an import of it fails
+import paper_2602_02711_b200 as dmr
+from paper_2602_02711_b200 import binding
+with warnings.catch_warnings(record=True) as said:
+    warnings.simplefilter("always")
+    assert dmr.lib().dmr_workspace_bytes(0, 1, 128, 128, dmr.QFormat(4, 64)) > 0 and binding._calls is None
+assert len(said) == 1 and "build" in str(said[0].message)
+"""
+    r = subprocess.run([sys.executable, "-c", script], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]

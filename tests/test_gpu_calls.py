@@ -4,15 +4,19 @@ import pytest
 import torch
 
 import paper_2602_02711_b200 as dmr
-from paper_2602_02711_b200 import QFormat, OUT_BF16, OUT_F32
+from paper_2602_02711_b200 import binding, QFormat, OUT_BF16, OUT_F32
 from paper_2602_02711_b200.binding import OP_DENSE, OP_LOWBIT, OP_ROUTED
 
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("native", [True, False])
 @pytest.mark.parametrize("M", [0, 1, 40])
 @pytest.mark.parametrize("out", [OUT_BF16, OUT_F32])
-def test_given_outputs_workspaces_and_streams(M, out):
+def test_given_outputs_workspaces_and_streams(M, out, native, monkeypatch):
+    dmr.lib()
+    if not native:
+        monkeypatch.setattr(binding, "_calls", None)
     N, K = 200, 256
     X, W = torch.randn(M, K, device="cuda").bfloat16(), torch.randn(N, K, device="cuda").bfloat16()
     q, mask = dmr.dmr_quantize(W, QFormat(4, 64)), torch.ones(M, dtype=torch.uint8, device="cuda")
