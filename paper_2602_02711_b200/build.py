@@ -11,6 +11,7 @@ import subprocess
 import sys
 import sysconfig
 from concurrent.futures import ThreadPoolExecutor
+from importlib import metadata
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -19,6 +20,7 @@ OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdmr.so")
 CALLS_SRC = os.path.join(CSRC, "calls.cpp")
 CALLS = os.path.join(PKG, "_calls.so")
+CALLS_STAMP = os.path.join(OBJ, "calls.txt")  # what CALLS was built for
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -45,8 +47,22 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _calls_made_for() -> str:
+    return f"torch {metadata.version('torch')}, Python {sys.version_info[0]}.{sys.version_info[1]}"
+
+
+def _calls_stale() -> bool:
+    # the module is bound to the torch and Python it was built with, whatever the files' times say
+    try:
+        with open(CALLS_STAMP) as f:
+            made_for = f.read()
+    except OSError:
+        return True
+    return made_for != _calls_made_for() or _stale(CALLS, [CALLS_SRC] + headers())
+
+
 def needs_build() -> bool:
-    return _stale(LIB, sources() + headers()) or _stale(CALLS, [CALLS_SRC] + headers())
+    return _stale(LIB, sources() + headers()) or _calls_stale()
 
 
 def _calls_command() -> list:
@@ -71,7 +87,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         return src, r
 
-    calls = subprocess.Popen(_calls_command()) if force or _stale(CALLS, [CALLS_SRC] + hdrs) else None
+    calls = subprocess.Popen(_calls_command()) if force or _calls_stale() else None
     with ThreadPoolExecutor(max_workers=min(8, max(1, len(todo)))) as pool:
         for src, r in pool.map(compile_one, todo):
             if verbose or r.returncode != 0:
@@ -80,8 +96,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
                 raise subprocess.CalledProcessError(r.returncode, f"nvcc {src}")
     objs = [_obj(s) for s in sources()]
     subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "--shared", "-o", LIB] + objs, check=True)
-    if calls is not None and calls.wait() != 0:
-        raise subprocess.CalledProcessError(calls.returncode, f"{calls.args[0]} {CALLS_SRC}")
+    if calls is not None:
+        if calls.wait() != 0:
+            raise subprocess.CalledProcessError(calls.returncode, f"{calls.args[0]} {CALLS_SRC}")
+        with open(CALLS_STAMP, "w") as f:
+            f.write(_calls_made_for())
     return LIB
 
 

@@ -1,8 +1,10 @@
 """The linears' native marshalling away from a GPU: tensors that cannot say their size or address are refused with -1, for the Python code to
-name the error, and end no process; without the module the library loads all the same."""
+name the error, and end no process; without the module the library loads all the same; and it is built again for another torch."""
 import os
 import subprocess
 import sys
+
+from paper_2602_02711_b200 import build
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -49,3 +51,14 @@ assert len(said) == 1 and "build" in str(said[0].message)
 """
     r = subprocess.run([sys.executable, "-c", script], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+def test_the_module_is_stale_for_another_torch(monkeypatch, tmp_path):
+    stamp = tmp_path / "calls.txt"
+    monkeypatch.setattr(build, "CALLS_STAMP", str(stamp))
+    monkeypatch.setattr(build, "_stale", lambda target, deps: False)
+    assert build.needs_build()  # nobody knows what it was built for
+    stamp.write_text(build._calls_made_for())
+    assert not build.needs_build()
+    monkeypatch.setattr(build.metadata, "version", lambda name: "99.0")
+    assert build.needs_build()
