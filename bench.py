@@ -488,7 +488,7 @@ def run_extra_sections(sections, rank, dev, torch, dmr, inputs, fmt, peaks, l2_b
         # all four linears at M = 8192 as one figure for the tensor-core roofline
         out["roofline_prefill"] = {"bound": "tensor", "achieved": per_m[8192]["tflops"], "peak": peaks["bf16_tflops"],
                                    "unit": "TFLOP/s", "frac": per_m[8192]["tflops"] / peaks["bf16_tflops"], "traffic": None,
-                                   "us": per_m[8192]["us"], "kernel": "prefill_kernel", "peak_source": peaks["_source"] + " (burst)",
+                                   "us": per_m[8192]["us"], "kernel": "pair_kernel", "peak_source": peaks["_source"] + " (burst)",
                                    "frac_by_M": {str(M): round(v["tflops"] / peaks["bf16_tflops"], 3) for M, v in per_m.items()},
                                    "workload": "7B-class layer, four linears, INT4 g=128, bf16 out; headline figure at M=8192"}
 
@@ -644,7 +644,9 @@ def run_extra_sections(sections, rank, dev, torch, dmr, inputs, fmt, peaks, l2_b
             n = torch.from_numpy(inputs.router_lengths(B, L, seed=0)).to(dev)
             wsr = torch.empty(dmr.lib().dmr_router_workspace_bytes(cfg, B, L), dtype=torch.uint8, device=dev)
             g = torch.cuda.CUDAGraph()
+            launches = dmr.dmr_launch_count()
             dmr.dmr_router_forward(params, cfg, Z, n, 1, workspace=wsr)
+            launches = dmr.dmr_launch_count() - launches
             torch.cuda.synchronize()
             with torch.cuda.graph(g, stream=stream):
                 dmr.dmr_router_forward(params, cfg, Z, n, 1, workspace=wsr)
@@ -652,7 +654,7 @@ def run_extra_sections(sections, rank, dev, torch, dmr, inputs, fmt, peaks, l2_b
             T = B * L
             flops = 2.0 * T * kw["layers"] * (4 * kw["d"] * kw["d"] + 2 * kw["d"] * kw["ffn"])
             rt[f"B{B}"] = {"ms_per_call": t * 1e3, "tokens": T, "tflops_fp32": flops / t / 1e12,
-                           "frac_fp32_fma_peak": flops / t / 1e12 / 74.5, "launches_per_call": 2 + 7 * kw["layers"]}
+                           "frac_fp32_fma_peak": flops / t / 1e12 / 74.5, "launches_per_call": launches}
         rt["config"] = dict(kw, note="sizes are this library's reading; the paper prints none")
         rt["paper_t_router_ms_per_call"] = "17.13-29.15 (A6000, router plus frozen sentence encoder)"
         emit_section("router_forward", rt)
@@ -660,8 +662,7 @@ def run_extra_sections(sections, rank, dev, torch, dmr, inputs, fmt, peaks, l2_b
 
     if "crossover" in sections:
         # 32B-class gate and down linears, INT4 g=64 and INT8 per-channel, M = 1 .. 256, 1 % outlier channels x20,
-        # with the library's default dispatch (decode kernels up to 32 rows, tensor-core kernels above): where
-        # the bandwidth-bound family hands over to the compute-bound one.  Two weight copies exceed 3 x L2 for INT8
+        # with the library's default dispatch: where the bandwidth-bound kernels hand over to the compute-bound one.  Two weight copies exceed 3 x L2 for INT8
         # (141 MB each) and come close for INT4 g64 (77 MB each; three copies are used).
         cx = {"dispatch": f"DMR_DECODE_MAX_M={os.environ.get('DMR_DECODE_MAX_M', 'default')}"}
         summary = {}
@@ -683,13 +684,13 @@ def run_extra_sections(sections, rank, dev, torch, dmr, inputs, fmt, peaks, l2_b
                     b = qs[0].weight_bytes()
                     kern = dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, f5)["kernel"]
                     cx[f"{lname}_{fname}_M{M}"] = {"us": t * 1e6, "gbs": b / t / 1e9, "tflops": 2.0 * M * N * K / t / 1e12, "kernel": kern}
-                    if kern in ("decode_w4", "stream"):
+                    if kern != "pair":
                         best = M
                 summary[f"{lname}_{fname}"] = {
                     "M1_frac_hbm": round(cx[f"{lname}_{fname}_M1"]["gbs"] / peaks["hbm_gbs"], 3),
                     "M16_frac_hbm": round(cx[f"{lname}_{fname}_M16"]["gbs"] / peaks["hbm_gbs"], 3),
                     "M256_tflops": round(cx[f"{lname}_{fname}_M256"]["tflops"], 1),
-                    "last_M_on_decode_kernels": best}
+                    "last_M_on_bandwidth_bound_kernels": best}
                 del qs
         emit_section("crossover_32b", cx)
         out["crossover_32b"] = summary

@@ -145,7 +145,7 @@ def dmr_launch_count() -> int:
 
 def dmr_describe_dispatch(op: int, M: int, N: int, K: int, fmt: QFormat = None) -> dict:
     """Which kernel family and launch shape the library would use, as a dict such as
-    {"kernel": "prefill", "bits": 4, "bn": 256, "tiles": 3072, "ctas": 148}."""
+    {"kernel": "pair", "bits": 4, "rows": 256, "splits": 1, "tiles": 768, "ctas": 148}."""
     buf = ctypes.create_string_buffer(256)
     n = lib().dmr_describe_dispatch(op, M, N, K, fmt if fmt is not None else QFormat(4, 0), buf, 256)
     if n < 0:

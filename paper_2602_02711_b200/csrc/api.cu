@@ -508,18 +508,14 @@ int dmr_describe_dispatch(dmr_op_t op, int M, int N, int K, dmr_qformat_t f, cha
     if (op != DMR_OP_LOWBIT_LINEAR && op != DMR_OP_DENSE_LINEAR) return -1;
     if (!dense && !format_ok(K, f)) return -1;
     const int bits = dense ? 0 : f.bits, g = dense ? K : group_of(K, f);
-    if (use_pair(M, N, K, bits, g)) {  // tiles counted per CTA: 128 features each
+    if (use_pair(M, N, K, bits, g)) {
         const PairPlan p = pair_plan(M, N, K, bits);
-        return snprintf(buf, buf_bytes, "%s bits=%d bn=256 rows=%d splits=%d tiles=%d ctas=%d", dense ? "gemm" : "prefill", bits, p.rows, p.splits,
-                        (N + 127) / 128 * (p.tiles / p.n_tiles), p.ctas);
+        return snprintf(buf, buf_bytes, "pair bits=%d rows=%d splits=%d tiles=%d ctas=%d", bits, p.rows, p.splits, p.tiles, p.ctas);
     }
     if (use_small(M, N, K, bits, g)) {
-        // the family a batch of this size belongs to; one kernel serves them all, one unit of 128 features x 128 inputs after the other
         const SmallPlan p = small_plan(M, N, K);
-        if (!dense && M > 32) return snprintf(buf, buf_bytes, "prefill bits=%d bn=%d splits=1 tiles=%d ctas=%d", bits, p.bn, p.tiles, p.shares);
-        if (dense && M > 32) return snprintf(buf, buf_bytes, "gemm bits=0 bn=%d splits=1 tiles=%d ctas=%d", p.bn, p.tiles, p.shares);
-        if (!dense && bits != 8) return snprintf(buf, buf_bytes, "decode_w%d rows=%d tile=128 ctas=%d chunks=1", bits, p.bn, p.shares);
-        return snprintf(buf, buf_bytes, "stream bits=%d rows=%d steps=%d cluster=0 chunks=1", dense ? 16 : 8, p.bn, dense ? 2 * p.units : p.units);
+        return snprintf(buf, buf_bytes, "small bits=%d rows=%d tiles=%d units=%d ctas=%d chunks=%d", bits, p.bn, p.tiles, p.units, p.shares,
+                        (M + kExactRows - 1) / kExactRows);
     }
     if (!dense && bits == 3 && decode_w3_supported(M < kDecodeChunk ? M : kDecodeChunk, N, K, g)) {
         int nt, r, warps;

@@ -3,8 +3,9 @@
 The oracle cannot run these layers in full within seconds, so every case compares a few thousand seeded output
 coordinates, one whole output row and one whole output column with oracle.sampled_linear (each output costs only K
 multiply-adds), and asserts through dmr_describe_dispatch that the intended kernel instance is the one that ran:
-the persistent prefill kernel with 256-row activation tiles and several tiles per CTA, the streaming kernel with
-feature groups split across CTAs (no clusters) for bf16 and 8-bit weights, the 4-bit decode kernel, the routed call.
+the SM-pair kernel with several tiles per pair and split along k, the small-batch kernel with several tiles per CTA and with tiles
+that several CTAs share, the streaming kernel with feature groups split across CTAs (no clusters) for bf16 and 8-bit weights of the
+shapes it takes, the 4-bit decode kernel, the routed call.
 """
 import numpy as np
 import pytest
@@ -56,18 +57,18 @@ def quantized_layer(N, K, bits, group, seed):
     return _layers[key]
 
 
-# ---------------- prefill: 7B-class shapes, the 256-row instance, several tiles per CTA ----------------
+# ---------------- prefill: 7B-class shapes, several tiles per pair of SMs ----------------
 
 @pytest.mark.parametrize("name,M,bits,group", [
-    ("o", 2048, 4, 128),       # 32 x 8 = 256 tiles of 128 x 256 on 148 CTAs
-    ("qkv", 2048, 4, 128),     # 768 tiles: more than five per CTA
+    ("o", 2048, 4, 128),       # 16 x 8 tiles or more on 74 pairs
+    ("qkv", 2048, 4, 128),     # 48 x 8 tiles: more than five per pair
     ("qkv", 1900, 4, 128),     # M not a multiple of 256: a ragged last row tile
     ("o", 2048, 8, 0),         # INT8 per-channel
 ])
 def test_prefill_7b_shapes(name, M, bits, group):
     N, K = inputs.LAYER_7B[name]
     plan = dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, group))
-    assert plan["kernel"] == "prefill" and plan["bn"] == 256 and plan["tiles"] > plan["ctas"]
+    assert plan["kernel"] == "pair" and plan["splits"] == 1 and 2 * plan["tiles"] > plan["ctas"]
     W, q, ref = quantized_layer(N, K, bits, group, seed=40)
     X = inputs.activations(M, K, seed=40, index=M)
     Xd = to_dev_bf16(X)
@@ -78,27 +79,27 @@ def test_prefill_7b_shapes(name, M, bits, group):
     assert torch.equal(Y16, Y32.to(torch.bfloat16))
 
 
-def test_prefill_many_tiles_per_cta_with_ragged_features():
-    # N not a multiple of 128 and M = 700: 3 row tiles x 44 feature tiles (the last one ragged), and a layer with
-    # 1024 rows x 12288 features where every CTA runs two or three tiles back to back
+def test_prefill_many_tiles_per_pair_with_ragged_features():
+    # N not a multiple of 256 and M = 700: 3 row tiles or more x 22 feature tiles (the last one ragged), and a layer with
+    # 1024 rows x 12288 features where every pair runs two or three tiles back to back
     for (M, N, K) in [(700, 5600, 1024), (1024, 12288, 4096)]:
         plan = dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(4, 128))
-        assert plan["kernel"] == "prefill" and plan["bn"] == 256
+        assert plan["kernel"] == "pair"
         W, q, ref = quantized_layer(N, K, 4, 128, seed=41)
         X = inputs.activations(M, K, seed=41, index=M)
         Y32 = dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_F32)
         ms, ns, want, scale = sampled_reference(X, M, N, 41, qweight=ref[0], scales=ref[1], zeros=ref[2], bits=4, group=128)
         check(Y32, ms, ns, want, scale, TOL_PREFILL)
-    assert dmr.dmr_describe_dispatch(OP_LOWBIT, 1024, 12288, 4096, QFormat(4, 128))["tiles"] >= 2 * 148
+    assert dmr.dmr_describe_dispatch(OP_LOWBIT, 1024, 12288, 4096, QFormat(4, 128))["tiles"] >= 2 * 74
 
 
 def test_prefill_split_k_over_two_row_tiles():
-    # 300 rows = two 256-row tiles (the second ragged) x 32 feature tiles leave SMs idle: every tile's k range is split in
-    # two work items, fp32 partial sums added in split order by the second kernel
+    # 300 rows = two row tiles x 16 feature tiles leave pairs idle: every tile's k range is split in two work items, fp32
+    # partial sums added in split order by the second kernel
     name, M = "down", 300
     N, K = inputs.LAYER_7B[name]
     plan = dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(4, 128))
-    assert plan["kernel"] == "prefill" and plan["bn"] == 256 and plan["splits"] == 2 and plan["tiles"] == 64
+    assert plan["kernel"] == "pair" and plan["splits"] == 2 and plan["tiles"] == 32
     W, q, ref = quantized_layer(N, K, 4, 128, seed=40)
     X = inputs.activations(M, K, seed=44, index=M)
     Xd = to_dev_bf16(X)
@@ -110,24 +111,24 @@ def test_prefill_split_k_over_two_row_tiles():
 
 
 @pytest.mark.parametrize("bits", [4, 3])
-def test_prefill_64_row_tile_several_tiles_per_cta(bits):
-    # up to 64 rows run the 64-row instance; 40000 features = 313 feature tiles (the last one ragged) on 148 CTAs,
-    # no split along k: every CTA runs two or three tiles back to back through both accumulators
+def test_64_row_tile_several_tiles_per_cta(bits):
+    # up to 64 rows run the small-batch kernel's 64-row instance; 40000 features = 313 feature tiles (the last one ragged) on
+    # 148 CTAs: every CTA has one whole tile or two, and a part of one or two more, all of them eight units long
     M, N, K = 50, 40000, 1024
     plan = dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, 128))
-    assert plan["kernel"] == "prefill" and plan["bn"] == 64 and plan["splits"] == 1 and plan["tiles"] > 2 * plan["ctas"]
+    assert plan["kernel"] == "small" and plan["rows"] == 64 and plan["tiles"] > 2 * plan["ctas"]
     W, q, ref = quantized_layer(N, K, bits, 128, seed=43)
     X = inputs.activations(M, K, seed=43, index=M)
     Y32 = dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_F32)
     ms, ns, want, scale = sampled_reference(X, M, N, 43, qweight=ref[0], scales=ref[1], zeros=ref[2], bits=bits, group=128)
-    check(Y32, ms, ns, want, scale, TOL_PREFILL)
+    check(Y32, ms, ns, want, scale, TOL_SUMS)
 
 
 # ---------------- streaming kernel with feature groups split across CTAs (no clusters) ----------------
 
 @pytest.mark.parametrize("M,out", [(1, OUT_F32), (16, OUT_BF16), (27, OUT_F32)])
 def test_dense_decode_contiguous_split(M, out):
-    N, K = 2304, 8192     # 18 feature groups x 128 steps of 64 bf16 weights = 2304 steps
+    N, K = 2304, 8200     # (not a multiple of 64) 18 feature groups x 129 steps of 64 bf16 weights = 2322 steps
     plan = dmr.dmr_describe_dispatch(OP_DENSE, M, N, K)
     assert plan["kernel"] == "stream" and plan["cluster"] == 0 and plan["steps"] > 2100
     W = inputs.weights(N, K, seed=42, index=1)
@@ -140,9 +141,9 @@ def test_dense_decode_contiguous_split(M, out):
 
 
 @pytest.mark.parametrize("M,N,K,group,out", [
-    (8, 4096, 8192, 0, OUT_F32),      # INT8 per-channel, 32 groups x 64 steps
-    (16, 4096, 8192, 0, OUT_BF16),
-    (32, 2048, 16384, 128, OUT_F32),  # INT8 grouped, the 32-row instance
+    (8, 4096, 8256, 192, OUT_F32),    # INT8, groups of 192: 32 feature groups x 65 steps
+    (16, 4096, 8256, 192, OUT_BF16),
+    (32, 2048, 16320, 192, OUT_F32),  # the 32-row instance
 ])
 def test_int8_decode_contiguous_split(M, N, K, group, out):
     plan = dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(8, group))
@@ -159,23 +160,23 @@ def test_int8_decode_contiguous_split(M, N, K, group, out):
 def test_streaming_chain_on_one_workspace_is_repeatable():
     """bf16 and 8-bit layers of different widths, all split across CTAs, launched back to back on one workspace
     (programmatic dependent launch; counters and partial sums reused): every repetition gives the first bits."""
-    shapes = [(2304, 8192, 16, 1), (4096, 8192, 8, 8), (4608, 4096, 16, 27), (2048, 16384, 8, 16)]   # N, K, bits, M
+    shapes = [(2304, 8200, 16, 1), (4096, 8256, 8, 8), (4608, 4104, 16, 27), (2048, 16320, 8, 16)]   # N, K, bits, M
     cases = []
     for (N, K, bits, M) in shapes:
         X = to_dev_bf16(inputs.activations(M, K, seed=44, index=M))
         W = inputs.weights(N, K, seed=44, index=N)
-        layer = to_dev_bf16(W) if bits == 16 else dmr.dmr_quantize(to_dev_bf16(W), QFormat(8, 0))
+        layer = to_dev_bf16(W) if bits == 16 else dmr.dmr_quantize(to_dev_bf16(W), QFormat(8, 192))
         op = OP_DENSE if bits == 16 else OP_LOWBIT
-        plan = dmr.dmr_describe_dispatch(op, M, N, K, QFormat(8, 0))
+        plan = dmr.dmr_describe_dispatch(op, M, N, K, QFormat(8, 192))
         assert plan["kernel"] == "stream" and plan["cluster"] == 0
         Xb = inputs.activations(M, K, seed=44, index=M)
         if bits == 16:
             ref = sampled_reference(Xb, M, N, 44, count=500, W=W)
         else:
-            r = oracle.quantize(W, bits=8, group=0)
-            ref = sampled_reference(Xb, M, N, 44, count=500, qweight=r[0], scales=r[1], zeros=r[2], bits=8, group=0)
+            r = oracle.quantize(W, bits=8, group=192)
+            ref = sampled_reference(Xb, M, N, 44, count=500, qweight=r[0], scales=r[1], zeros=r[2], bits=8, group=192)
         cases.append((X, layer, bits, M, N, ref))
-    ws = dmr.new_workspace(OP_LOWBIT, 32, 4608, 16384, QFormat(8, 0), "cuda")
+    ws = dmr.new_workspace(OP_LOWBIT, 32, 4608, 16320, QFormat(8, 192), "cuda")
 
     def run_all():
         outs = []
@@ -197,6 +198,31 @@ def test_streaming_chain_on_one_workspace_is_repeatable():
     assert dmr.lib().dmr_workspace_status(ws.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
 
 
+# ---------------- bf16 and 8-bit decoding: the small-batch kernel with tiles that several CTAs share ----------------
+
+@pytest.mark.parametrize("M,N,K,bits,out", [
+    (1, 2304, 8192, 0, OUT_F32), (16, 2304, 8192, 0, OUT_BF16), (27, 2304, 8192, 0, OUT_F32),
+    (8, 4096, 8192, 8, OUT_F32), (16, 4096, 8192, 8, OUT_BF16), (32, 2048, 16384, 8, OUT_F32),
+])
+def test_small_batches_with_shared_tiles(M, N, K, bits, out):
+    fmt = QFormat(bits or 4, 0)
+    plan = dmr.dmr_describe_dispatch(OP_LOWBIT if bits else OP_DENSE, M, N, K, fmt)
+    assert plan["kernel"] == "small" and plan["tiles"] < plan["ctas"] and plan["chunks"] == 1
+    X = inputs.activations(M, K, seed=42, index=M)
+    Xd = to_dev_bf16(X)
+    if bits:
+        W, q, ref = quantized_layer(N, K, bits, 0, seed=43)
+        layer, call = dict(qweight=ref[0], scales=ref[1], zeros=ref[2], bits=bits, group=0), lambda: dmr.dmr_lowbit_linear(Xd, q, out)
+    else:
+        W = inputs.weights(N, K, seed=42, index=1)
+        Wd = to_dev_bf16(W)
+        layer, call = dict(W=W), lambda: dmr.dmr_dense_linear(Xd, Wd, out)
+    Y = call()
+    ms, ns, want, scale = sampled_reference(X, M, N, 42, **layer)
+    check(Y, ms, ns, want, scale, TOL_SUMS if out == OUT_F32 else 2 ** -8 + TOL_SUMS)
+    assert torch.equal(call(), Y)
+
+
 # ---------------- 4-bit decode kernel at 14B- and 32B-class sizes ----------------
 
 @pytest.mark.parametrize("N,K,group,M,outlier", [
@@ -208,7 +234,7 @@ def test_streaming_chain_on_one_workspace_is_repeatable():
 ])
 def test_decode_w4_large_layers(N, K, group, M, outlier):
     plan = dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(4, group))
-    assert plan["kernel"] == "decode_w4"
+    assert plan["kernel"] == ("decode_w4" if M <= 16 else "small")
     W, q, ref = quantized_layer(N, K, 4, group, seed=45)
     X = inputs.activations(M, K, seed=45, index=M, outlier_frac=outlier)
     Y32 = dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_F32)

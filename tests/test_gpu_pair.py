@@ -33,7 +33,7 @@ def test_dense(M, N, K):
 @pytest.mark.parametrize("bits,group", [(4, 64), (8, 0), (3, 64)])
 @pytest.mark.parametrize("M,N,K", SHAPES)
 def test_low_bit(M, N, K, bits, group):
-    assert dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, group))["kernel"] != "simple"
+    assert dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, group))["kernel"] == "pair"
     W, X = inputs.weights(N, K, seed=K), inputs.activations(M, K, seed=N, outlier_frac=0.01)
     q = dmr.dmr_quantize(to_dev_bf16(W), QFormat(bits, group))
     want = oracle.lowbit_linear(X, *oracle.quantize(W, bits=bits, group=group), bits=bits, group=group)
@@ -46,7 +46,7 @@ def test_low_bit(M, N, K, bits, group):
 # to all k blocks, the fewest rows
 @pytest.mark.parametrize("M,N,K,group", [(129, 256, 64, 64), (33, 100, 192, 64), (64, 300, 2880, 320), (65, 257, 2880, 0), (300, 640, 4544, 64), (1100, 2600, 960, 192)])
 def test_3_bit_rows_that_are_not_whole_boxes(M, N, K, group):
-    assert dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(3, group))["kernel"] != "simple"
+    assert dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(3, group))["kernel"] == "pair"
     W, X = inputs.weights(N, K, seed=K), inputs.activations(M, K, seed=N, outlier_frac=0.01)
     q = dmr.dmr_quantize(to_dev_bf16(W), QFormat(3, group))
     want = oracle.lowbit_linear(X, *oracle.quantize(W, bits=3, group=group), bits=3, group=group)

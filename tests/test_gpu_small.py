@@ -35,7 +35,7 @@ def test_low_bit(M, N, K, bits, group):
     if bits == 3 and (M > 64 or K % 128 != 0):
         pytest.skip("the SM-pair kernel (test_gpu_pair.py), or up to 32 rows the one for any shape (test_gpu_w3.py)")
     W, X = inputs.weights(N, K, seed=K), inputs.activations(M, K, seed=N, outlier_frac=0.01)
-    assert M <= 16 or dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, group))["kernel"] != "simple"
+    assert M <= 16 or dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, group))["kernel"] == "small"
     q = dmr.dmr_quantize(to_dev_bf16(W), QFormat(bits, group))
     want = oracle.lowbit_linear(X, *oracle.quantize(W, bits=bits, group=group), bits=bits, group=group)
     Y = dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_F32)
@@ -141,7 +141,7 @@ def test_weights_written_by_the_call_before(M):
 def test_rows_longer_than_the_large_batches_take(M, N, bits, group):
     """More than 32768 inputs: exact for any number of rows, in launches of 128; routed rows are the unrouted ones whichever launch they fall into."""
     K = 40960
-    assert dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, group))["kernel"] not in ("simple", "stream", "decode_w4")
+    assert dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(bits, group))["kernel"] == "small"
     W, X = inputs.weights(N, K, seed=N), inputs.activations(M, K, seed=M, outlier_frac=0.01)
     q, Xd, Wd = dmr.dmr_quantize(to_dev_bf16(W), QFormat(bits, group)), to_dev_bf16(X), to_dev_bf16(W)
     Y = dmr.dmr_lowbit_linear(Xd, q, OUT_F32)
