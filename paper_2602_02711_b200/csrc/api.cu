@@ -40,7 +40,8 @@ struct Scratch {
 constexpr int kStreamChunk = 32;  // rows one launch of the streaming decode kernel takes at most
 
 // The warp-ring decode kernel takes the 4-bit decode batches unless the environment says DMR_DECODE_KERNEL=stream
-// (the shared-memory ring kernel, kept for 8-bit codes, bf16 weights and for comparison).
+// (the shared-memory ring kernel, kept for what the others do not take - bf16 weights with K not a multiple of 64, other 8-bit groups than 64, multiples of
+// 128 and whole rows - for dmr_lowbit_linear_noalloc and for comparison).
 bool decode_w4_enabled() {
     static int v = -1;
     if (v < 0) {

@@ -135,7 +135,7 @@ dmr_status_t launch_small_routed(const uint16_t *Xh, const uint16_t *Xl, int M, 
                                  const uint16_t *scales, const uint8_t *zeros, int N, int K, int bits, int g, void *Y, dmr_out_t out, float *partial_high,
                                  float *partial_low, int32_t *counters_high, int32_t *counters_low, int32_t *status, cudaStream_t st);
 
-// Large batches (M > 32) on pairs of SMs: bf16 weights (bits == 0) and packed codes.  X is the bf16 matrix, or for codes the
+// Large batches (more than 32 rows that the small-batch kernel does not take) on pairs of SMs: bf16 weights (bits == 0) and packed codes.  X is the bf16 matrix, or for codes the
 // prepared fp16 one with its row scales.
 struct PairPlan {
     int n_tiles, rows, splits, kb_per_split, tiles, ctas;

@@ -183,8 +183,8 @@ __device__ __noinline__ KlThread kl_redo(const uint8_t *ra, const uint8_t *rb, i
 // Bound by HBM and, with bf16 logits, as much by the two exponentials per element (16 per clock and SM: 52 us for 777 x 151936
 // against 72 for the bytes).  So: 64 warps on an SM (at most 32 registers, one vector of each row in flight per thread; two in
 // flight, or 48 warps, measured no better: 89 and 92 us), no test per element for logits that are not finite, bf16x2 maxima, unaligned
-// rows (V not a multiple of 8) with 16-byte loads too.  777 x 151936 bf16: 102 -> 90 us (5.2 TB/s); 100 x 99997: 45 -> 25.5;
-// 250 x 151936 fp32: 64 -> 53 (5.8 TB/s).
+// rows (V not a multiple of 8) with 16-byte loads too.  777 x 151936 bf16: 106 -> 95 us (5.0 TB/s); 100 x 99997: 30 -> 21;
+// 250 x 151936 fp32: 64 -> 48 (6.3 TB/s).
 template <bool F32, bool ALIGNED>
 __global__ void __launch_bounds__(kKlThreads, 4)
 kl_token_kernel(const void *__restrict__ high, const void *__restrict__ low, int V, int parts, int ctas, float *__restrict__ kl_token) {
