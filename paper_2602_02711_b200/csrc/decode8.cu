@@ -1,0 +1,635 @@
+// Decode-time linears of 4-bit codes, a few rows: the weight matrix is read exactly once.
+// Decoding re-streams the model weights for every generated token and is limited by memory bandwidth, which is where weight-only
+// quantization pays (App. "Evaluation protocol", discussion of output length; App. "Latency coefficients").
+//
+// What bounds it.  HBM, if the arithmetic keeps out of the way.  A code among the low eleven bits of a 16-bit word IS an fp16 number, exactly: up to 2^11
+// the bits count in steps of 2^-24, through the subnormals and the first binade above.  So the pairs of 4-bit codes of a word are an AND each,
+// in place, with one byte permute for half of them, and the otherwise idle FMA pipe does the rest (code_pair): 4 integer instructions for 8 codes where bf16
+// numbers 128 + q need 7.  Nothing is rounded and no offset is added: the tensor cores (mma.m16n8k16, the weights as the 16-row operand) sum x q, and per chunk of inputs, which never crosses a quantization group,
+//     sum_k x_k s (q_k - z) = s (sum_k x_k q_k - z sum_k x_k)
+// is formed in fp32 (errors against 64 bits: 1e-7 of the outputs' 2-norm, 2.5e-6 with the offset).  Activations are converted to fp16 once per CTA, after scaling a
+// row's inputs of a box by the power of two that brings the largest to [2^14, 2^15): exact for all that are above 2^-31 of it, and to 2^-39 of the largest for
+// the others.
+// Measured: four 7B linears, groups of 128, one row 39.4 -> 33.9 us, of 64 45.9 -> 37.9 (kernel chosen in decode8_supported).  A tile of 32 x 4096 takes 2950 cycles
+// there, the HBM rate; the rest is a launch's beginning and end.  (mma.m16n8k32 on e4m3 numbers, which 4-bit codes in bytes of their own are as well, is carried
+// out by conversions to fp16 on this GPU: 43.6 us.)
+//
+// Work decomposition.  A cluster of c CTAs (1, 2, 4 or 8) owns tiles of 32 c output features.  Each CTA takes a c-th of the inputs for
+// all of them, so that it converts and keeps a c-th of the activations only (c is the smallest that makes them fit).  Its warps are c groups of
+// rows times WARPS / c pieces of its inputs: a warp owns 32 features and every (WARPS / c)-th box of 128 bytes a row.  The 32 features of row group i are
+// finished by CTA i: every warp sends its sums there (plain stores for c = 1, st.async through distributed shared memory otherwise),
+// where they are added in a fixed order that depends on the instance and the layer's shape only, so a row's result never depends
+// on the batch around it.  No sum goes through global memory.  The hand-over is by mbarrier and one tile late, so that no warp waits for another one's
+// tile.
+//
+// Data movement.  Every warp has a ring of its own in shared memory that one of its lanes keeps full with TMA boxes of [32 rows x 128
+// bytes] of packed codes (rows past N read as zero; 128-byte swizzle); nobody else
+// reads it, so the only synchronisation is the warp's own mbarrier per stage.  Scales and zero points are fetched into registers a box ahead.
+//
+// Launch chains.  The kernel lets its successor start at once (programmatic dependent launch) and asks for more than half of an SM's shared
+// memory, so that an SM never holds two CTAs of these kernels: the successor's CTA moves in when this kernel's CTA on that SM has finished,
+// fills its rings and only then waits for its predecessor.  Weights, scales and zero points are read before the wait: they must not be
+// produced by a kernel that releases its dependents early (the library's own kernels that write weights never do).
+#include <cuda_bf16.h>
+
+#include <cstdlib>
+
+#include "sm100.cuh"
+
+namespace dmr {
+
+namespace {
+
+struct Decode8Args {
+    const uint16_t *X;        // [*][K] bf16
+    const int32_t *idx;       // routed: row of X / Y for batch slot s (nullptr = identity)
+    const int32_t *count;     // routed: valid slots in the whole list (nullptr = M)
+    const uint16_t *scales;   // [N][G] bf16
+    const uint8_t *zeros;     // [N][G]
+    void *Y;                  // [*][N]
+    int32_t *status;          // set to DMR_ERR_TIMEOUT if a bounded wait runs out
+    int M, coff, N, K, G;
+    int out_f32;
+    int nboxes, nchunks;      // of the whole k range
+    int log_c;                // CTAs per cluster
+    int tiles_each, tiles_more;  // of ceil(N / (32 c)): a cluster's, and how many of the first clusters have one more
+    uint32_t g_mul;           // quantization group of chunk k = k g_mul / 2^32 (0: k itself)
+    int sz_vec;               // a box's scales and zero points are side by side and aligned
+    int off_b, off_t, off_red, off_bar;  // shared memory: activations, their sums and scales, sums of a tile, barriers
+};
+
+// Sends 16 bytes to a CTA of the cluster, whose barrier `bar` counts them when they are there.
+__device__ __forceinline__ void st_async_v4(uint32_t addr, float x, float y, float z, float w, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1,%2,%3,%4}, [%5];" ::"r"(addr), "f"(x), "f"(y), "f"(z),
+                 "f"(w), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// Warp-level 16 x 8 x 16 product of fp16 numbers with fp32 sums; the first of a chunk starts from zero.
+template <bool ZERO>
+__device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    if constexpr (ZERO) {
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+            : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+    } else {
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+            : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+    }
+}
+__device__ __forceinline__ uint32_t bf16x2_mul(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+// A chunk's inputs are dealt to the four lanes of a row in blocks; a block's word of eight codes becomes four pairs of fp16 numbers, codes (0, 4), (1, 5),
+// (2, 6), (3, 7), all times 16: the tensor cores line up products by the exponents as they stand, so that small subnormal numbers cost as many bits of the sum as
+// they have leading zeros (without the factor, activations with outliers: errors of 4.1e-6 of the outputs' 2-norm where they are 1.3e-7 with it).  The
+// factor, and the fourth pair, are the FMA pipe's work.
+__device__ __forceinline__ uint32_t code_pair(const uint32_t *w, int i) {
+    const uint32_t u = i % 4 < 2 ? w[i / 4] : __byte_perm(w[i / 4], 0u, 0x4341u);
+    if (i % 4 == 1) return u & 0x00F000F0u;
+    const uint32_t lo = u & 0x000F000Fu;
+    return i & 1 ? f16x2_sub(u, lo) : f16x2_mul(lo, 0x4C004C00u);
+}
+
+constexpr size_t kMinSmem = 116 * 1024;   // more than half of the 228 KB of an SM
+constexpr size_t kMaxSmem = 227 * 1024;
+
+constexpr int WARPS = 16, LOG_WARPS = 4;
+constexpr int D = 2;                          // stages of a warp's ring
+constexpr int kBoxRow = 128, kBoxK = 256;     // a box: bytes of a row, inputs
+constexpr int kStage = 32 * kBoxRow;
+
+// GK: inputs per chunk (64 for groups of 64, else 128).
+template <int GK>
+struct Decode8Cfg {
+    static constexpr int CPB = kBoxK / GK;    // chunks per box
+    static constexpr int BLK = GK / 4;        // inputs of a chunk that a lane meets
+    static constexpr int PIECES = BLK / 8;    // 16-byte pieces (two MMAs) of its operand
+};
+
+// Eight activations (bf16 in order) as fp16, scaled by 2^(field - 127), in the pairs of a word of codes.  Returns their sum.
+__device__ __forceinline__ float convert_octet(const uint4 &x, uint32_t field, uint4 &o) {
+    const uint32_t factor = field << 7 | field << 23, in[4] = {x.x, x.y, x.z, x.w};
+    float f[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t v = bf16x2_mul(in[i], factor);
+        f[2 * i] = __uint_as_float(v << 16);
+        f[2 * i + 1] = __uint_as_float(v & 0xFFFF0000u);
+    }
+    o = make_uint4(pack_f16x2_rn(f[0], f[4]), pack_f16x2_rn(f[1], f[5]), pack_f16x2_rn(f[2], f[6]), pack_f16x2_rn(f[3], f[7]));
+    return ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
+}
+__device__ __forceinline__ uint32_t abs_max8(const uint4 &x) {  // both half-words
+    return __vmaxu2(__vmaxu2(x.x & 0x7FFF7FFFu, x.y & 0x7FFF7FFFu), __vmaxu2(x.z & 0x7FFF7FFFu, x.w & 0x7FFF7FFFu));
+}
+// 2^(field - 127) brings a row's largest activation (`top`, its bits without the sign) to [2^14, 2^15).  undo: what reverses it, and 2^8 of the
+// codes' 2^20 (the rest comes at the end: neither leaves the range); NaN for a row that is not finite.
+__device__ __forceinline__ uint32_t scale_field(uint32_t top) { return min(268u - (top >> 7), 253u); }
+__device__ __forceinline__ float undo_of(uint32_t top) {
+    return top >= 0x7F80u ? __uint_as_float(0x7FC00000u) : __uint_as_float((262u - scale_field(top)) << 23);
+}
+
+template <int GK>
+__global__ void __launch_bounds__(WARPS * 32, 1) decode8_kernel(const __grid_constant__ CUtensorMap wmap, const Decode8Args a) {
+    using Cfg = Decode8Cfg<GK>;
+    constexpr int CPB = Cfg::CPB, BLK = Cfg::BLK, PIECES = Cfg::PIECES, NW = BLK / 8;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const uint32_t base = smem_u32(smem);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane >> 2, t = lane & 3;
+    const int pg = (g >> 1) | ((g & 1) << 2);  // box row of fragment row g: 0, 4, 1, 5, ... (bank-conflict-free under the swizzle)
+    const int c = 1 << a.log_c, log_kw = LOG_WARPS - a.log_c, kw_n = 1 << log_kw;
+    const int rank = a.log_c ? (int)cluster_ctarank() : 0, cid = (int)blockIdx.x >> a.log_c;
+    const int rg = warp >> log_kw, kw = warp & (kw_n - 1);  // row group, and piece of the CTA's inputs
+    const int slot = (rank << log_kw) + kw;                 // of WARPS that add up to the row group's sums
+    const int t0 = cid * a.tiles_each + min(cid, a.tiles_more), t1 = t0 + a.tiles_each + (cid < a.tiles_more ? 1 : 0);
+    const int b_lo = (a.nboxes * rank) >> a.log_c, b_hi = (a.nboxes * (rank + 1)) >> a.log_c;  // this CTA's boxes
+    const uint32_t ring = base + (uint32_t)warp * (D * kStage);
+    const uint32_t bars = base + (uint32_t)a.off_bar + (uint32_t)warp * (D * 8);
+    const uint32_t full = base + (uint32_t)a.off_bar + WARPS * D * 8;  // [2] a tile's sums are here
+    const uint32_t freed = full + 16;                                  // [2] clusters: every warp of it has read them
+    const uint32_t red_buf = (uint32_t)(WARPS * 128) * (uint32_t)a.M;  // bytes of a tile's sums
+
+    if (threadIdx.x == 0) prefetch_tensor_map(&wmap);
+    if (lane == 0) {
+#pragma unroll
+        for (int d = 0; d < D; ++d) mbar_init(bars + 8 * d, 1);
+        if (warp == 0) {
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                mbar_init(full + 8 * d, c == 1 ? WARPS : 1);
+                mbar_init(freed + 8 * d, WARPS << a.log_c);
+            }
+        }
+        fence_barrier_init();
+    }
+    __syncwarp();
+    pdl_launch_dependents();
+
+    // ---- this warp's boxes: tiles t0, t0 + 1, ...; boxes b_lo + kw, + kw_n, ... of each ----
+    const bool has_boxes = b_lo + kw < b_hi;
+    bool ok = true;  // false once a bounded wait ran out: the warp stops copying and waiting but still takes part in everything else
+    int i_tile = t0, i_box = b_lo + kw, issued = 0;  // the next box to request
+    auto issue = [&]() {
+        if (!has_boxes || i_tile >= t1 || !ok) return;
+        if (lane == 0) {
+            const int d = issued % D;
+            mbar_expect_tx(bars + 8 * d, kStage);
+            tma_load_2d(ring + d * kStage, &wmap, bars + 8 * d, i_box * kBoxRow, ((i_tile << a.log_c) + rg) * 32);
+        }
+        ++issued;
+        i_box += kw_n;
+        if (i_box >= b_hi) {
+            i_box = b_lo + kw;
+            ++i_tile;
+        }
+    };
+    // scales and zero points of a box's chunks, as they lie in the tables
+    struct Sz {
+        uint32_t s[2][2][(CPB + 1) / 2], z[2][2];
+    };
+    auto load_sz = [&](Sz &v, int tile, int box) {
+        const int row0 = ((tile << a.log_c) + rg) * 32 + pg;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const size_t row = (size_t)min(row0 + r * 16 + h * 8, a.N - 1) * a.G;
+                if (a.sz_vec) {
+                    const size_t o = row + box * CPB;
+                    if constexpr (CPB == 4) {
+                        const uint2 s = __ldg(reinterpret_cast<const uint2 *>(a.scales + o));
+                        v.s[r][h][0] = s.x;
+                        v.s[r][h][(CPB + 1) / 2 - 1] = s.y;
+                        v.z[r][h] = __ldg(reinterpret_cast<const uint32_t *>(a.zeros + o));
+                    } else if constexpr (CPB == 2) {
+                        v.s[r][h][0] = __ldg(reinterpret_cast<const uint32_t *>(a.scales + o));
+                        v.z[r][h] = __ldg(reinterpret_cast<const uint16_t *>(a.zeros + o));
+                    } else {
+                        v.s[r][h][0] = __ldg(a.scales + o);
+                        v.z[r][h] = __ldg(a.zeros + o);
+                    }
+                } else {
+                    v.z[r][h] = 0;
+#pragma unroll
+                    for (int q = 0; q < CPB; ++q) {
+                        const uint32_t k = (uint32_t)min(box * CPB + q, a.nchunks - 1);
+                        const size_t o = row + (a.g_mul ? __umulhi(k, a.g_mul) : k);
+                        const uint32_t s = __ldg(a.scales + o);
+                        v.s[r][h][q / 2] = (q & 1) ? v.s[r][h][q / 2] | s << 16 : s;
+                        v.z[r][h] |= (uint32_t)__ldg(a.zeros + o) << (8 * q);
+                    }
+                }
+            }
+    };
+    Sz next;
+    // The requests that the first box waits for go first, and no more than a box per warp before the activations: 64 KB an SM keep the memory
+    // busy, and what is requested behind 128 KB comes 5800 cycles later.
+    if (has_boxes && t0 < t1) load_sz(next, t0, b_lo + kw);
+    issue();
+    if (c > 1) {
+        if (threadIdx.x == 0)
+            for (int d = 0; d < 2; ++d)
+                if (t0 + d < t1) mbar_expect_tx(full + 8 * d, red_buf);
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    } else {
+        __syncthreads();  // the barriers that the warps share are set up
+    }
+
+    pdl_wait();
+    const int rows = a.count ? min(*a.count - a.coff, a.M) : a.M;
+    if (rows <= 0 || t1 <= t0) {
+        // nothing to do (a routed call without rows of this kind): let the copies already under way land first
+        for (int d = 0; d < D && d < issued; ++d) (void)mbar_wait(bars + 8 * d, 0u, a.status);
+        if (c > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        return;
+    }
+
+    // ---- the activations of this warp's boxes as MMA operands: [chunk][piece][batch row][lane t] 16 bytes; the row groups share the work ----
+    const int ch_lo = b_lo * CPB, ms = (a.M + 1) & ~1;
+    const uint32_t piece = (uint32_t)a.M * 64, chunk_bytes = PIECES * piece, ops = base + (uint32_t)a.off_b;
+    float *sums = reinterpret_cast<float *>(smem + a.off_t);                             // [chunk][ms] sum of the activations
+    float *undo = sums + ((a.nboxes + c - 1) >> a.log_c) * CPB * ms;                    // [box][ms] power of two that undoes their scale
+    {
+        if (rows == 1) {
+            // a lane takes eight inputs of a box: piece q of lane ct's block (a fifth of the steps of the way below, which three quarters of the lanes would idle through)
+            const int sub = lane / (GK / 8), ct = lane % (GK / 8) / PIECES, q = lane % PIECES;
+            const uint4 *x = reinterpret_cast<const uint4 *>(a.X + (size_t)(a.idx ? a.idx[0] : 0) * a.K) + lane;
+            auto load_x = [&](int box) { return box < b_hi && box * CPB + sub < a.nchunks ? __ldg(x + box * (kBoxK / 8)) : make_uint4(0u, 0u, 0u, 0u); };
+            int box = b_lo + (rg == 0 ? kw : a.nboxes);
+            uint4 nxt = load_x(box);
+#pragma unroll
+            for (int d = 1; d < D; ++d) issue();  // (behind the activations)
+#pragma unroll 1
+            for (; box < b_hi; box += kw_n) {
+                const uint4 cur = nxt;
+                nxt = load_x(box + kw_n);
+                const int bl = box - b_lo;
+                uint32_t top = abs_max8(cur);
+                top = __reduce_max_sync(0xFFFFFFFFu, max(top >> 16, top & 0xFFFFu));
+                uint4 v;
+                float sum = convert_octet(cur, scale_field(top), v);
+                *reinterpret_cast<uint4 *>(smem + a.off_b + (uint32_t)(bl * CPB + sub) * chunk_bytes + q * piece + 16 * ct) = v;
+#pragma unroll
+                for (int d = 1; d < GK / 8; d <<= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
+                if (lane % (GK / 8) == 0) sums[(bl * CPB + sub) * ms] = sum * 0x1p-20f;
+                if (lane == 0) undo[bl * ms] = undo_of(top);
+            }
+        } else {
+            constexpr int LPR = 4 * CPB, RPI = 32 / LPR;  // lanes that share a row's inputs of a box; rows at a time
+            const int sub = (lane % LPR) >> 2, lm = lane / LPR;
+            auto load_x = [&](uint4 (&w)[PIECES], int box, int m0) {
+                const int m = min(m0 + lm, rows - 1), ch = box * CPB + sub;
+                const uint4 *x = reinterpret_cast<const uint4 *>(a.X + (size_t)(a.idx ? a.idx[m] : m) * a.K + (size_t)ch * GK) + t * PIECES;
+#pragma unroll
+                for (int i = 0; i < PIECES; ++i) w[i] = ch < a.nchunks ? __ldg(x + i) : make_uint4(0u, 0u, 0u, 0u);
+            };
+            int box = b_lo + kw, m0 = rg * RPI;
+            if (m0 >= rows) box = b_hi;
+            int l_box = box, l_m0 = m0;  // the rows to request
+            auto next_rows = [&](int &b, int &m) {
+                m += RPI << a.log_c;
+                if (m >= rows) {
+                    m = rg * RPI;
+                    b += kw_n;
+                }
+            };
+            uint4 cur[PIECES], nxt[PIECES];
+            if (l_box < b_hi) load_x(cur, l_box, l_m0);
+            next_rows(l_box, l_m0);
+            if (l_box < b_hi) load_x(nxt, l_box, l_m0);
+#pragma unroll
+            for (int d = 1; d < D; ++d) issue();  // (behind the activations)
+#pragma unroll 1
+            while (box < b_hi) {
+                uint32_t top = abs_max8(cur[0]);
+#pragma unroll
+                for (int i = 1; i < PIECES; ++i) top = __vmaxu2(top, abs_max8(cur[i]));
+                top = max(top >> 16, top & 0xFFFFu);
+#pragma unroll
+                for (int d = 1; d < LPR; d <<= 1) top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, d));
+                const int m = m0 + lm, bl = box - b_lo;
+                float part[PIECES];
+#pragma unroll
+                for (int i = 0; i < PIECES; ++i) {
+                    uint4 v;
+                    part[i] = convert_octet(cur[i], scale_field(top), v);
+                    if (m < rows) *reinterpret_cast<uint4 *>(smem + a.off_b + (uint32_t)(bl * CPB + sub) * chunk_bytes + i * piece + (uint32_t)(64 * m + 16 * t)) = v;
+                }
+                // (added in the order of the way above: a routed call may have one row where its caller has several)
+                float sum = PIECES == 4 ? (part[0] + part[1]) + (part[PIECES - 2] + part[PIECES - 1]) : part[0] + part[1];
+                sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
+                sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
+                if (t == 0 && m < rows) sums[(bl * CPB + sub) * ms + m] = sum * 0x1p-20f;
+                if (lane % LPR == 0 && m < rows) undo[bl * ms + m] = undo_of(top);
+                next_rows(box, m0);
+                next_rows(l_box, l_m0);
+#pragma unroll
+                for (int i = 0; i < PIECES; ++i) cur[i] = nxt[i];
+                if (l_box < b_hi) load_x(nxt, l_box, l_m0);
+            }
+        }
+        if (c == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + kw), "r"(32 << a.log_c) : "memory");
+    }
+    // this lane's column (columns past the batch read the first one: their products are never used)
+    const uint32_t bcol = ops + (uint32_t)((g < rows ? g : 0) * 64 + t * 16);
+    const int mcol = min(2 * t, ms - 2);
+    auto lds = [&](uint32_t addr) -> uint4 { return *reinterpret_cast<const uint4 *>(smem + (addr - base)); };
+    if (c > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // the other CTAs' barriers are set up
+
+    float acc[2][4];  // rows g (two) and g + 8 (two) of each 16-row block, batch rows 2 t, 2 t + 1
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
+
+    // Adds up the row group that this CTA finishes of the cluster's tile `tile` (its number `tl`) and writes the outputs.
+    auto finish_tile = [&](int tile, int tl) {
+        const uint32_t par = (uint32_t)((tl >> 1) & 1);
+        if (ok) ok = c == 1 ? mbar_wait(full + 8 * (tl & 1), par, a.status) : mbar_wait_cluster(full + 8 * (tl & 1), par, a.status);
+        const float *buf = reinterpret_cast<const float *>(smem + a.off_red + (tl & 1) * red_buf);
+        for (int o = threadIdx.x; o < 32 * rows; o += WARPS * 32) {
+            const int m = o >> 5, l = o & 31, lg = l & 7;
+            const float *p = buf + m * 32 + ((lg & 3) << 1 | lg >> 2) * 4 + (l >> 3);
+            float v = p[0];
+#pragma unroll
+            for (int s = 1; s < WARPS; ++s) v += p[s * 32 * a.M];
+            v *= 4096.f;
+            const int n = ((tile << a.log_c) + rank) * 32 + l;
+            if (ok && n < a.N) {
+                const size_t at = (size_t)(a.idx ? a.idx[m] : m) * a.N + n;
+                if (a.out_f32) reinterpret_cast<float *>(a.Y)[at] = v;
+                else reinterpret_cast<__nv_bfloat16 *>(a.Y)[at] = __float2bfloat16_rn(v);
+            }
+        }
+        if (c > 1) {
+            if (threadIdx.x == 0 && tile + 2 < t1) mbar_expect_tx(full + 8 * (tl & 1), red_buf);
+            __syncwarp();
+            if (lane < c) mbar_arrive_cluster(cluster_map(freed + 8 * (tl & 1), (uint32_t)lane));
+        }
+    };
+
+    // this lane's codes of a row and chunk, from the row's place in the box
+    auto load_codes = [&](uint32_t (&w)[NW], uint32_t row, int sub) {
+        if constexpr (GK == 64) {
+            const uint2 v = *reinterpret_cast<const uint2 *>(smem + (row + (uint32_t)((((2 * sub + (t >> 1)) ^ pg) << 4) + 8 * (t & 1)) - base));
+            w[0] = v.x;
+            w[1] = v.y;
+        } else {
+#pragma unroll
+            for (int i = 0; i < NW / 4; ++i) {  // (pg = row mod 8)
+                const uint4 v = lds(row + (uint32_t)(((4 * (NW / 4 * sub + i) + t) ^ pg) << 4));
+                w[4 * i] = v.x;
+                w[4 * i + 1] = v.y;
+                w[4 * i + 2] = v.z;
+                w[4 * i + 3] = v.w;
+            }
+        }
+    };
+    int consumed = 0;
+    for (int tile = t0, tl = 0; tile < t1; ++tile, ++tl) {
+        for (int box = b_lo + kw; box < b_hi; box += kw_n) {
+            const int d = consumed % D;
+            const Sz sz = next;
+            {
+                const bool more = box + kw_n < b_hi;
+                if (more || tile + 1 < t1) load_sz(next, more ? tile : tile + 1, more ? box + kw_n : b_lo + kw);
+            }
+            if (ok) ok = mbar_wait(bars + 8 * d, (uint32_t)((consumed / D) & 1), a.status);
+            ++consumed;
+            const uint32_t stage = ring + d * kStage;
+            const int ch0 = box * CPB - ch_lo, nsub = min(CPB, a.nchunks - box * CPB);
+            float sbox[2][4];  // the box's sums, in units of its rows' scales
+#pragma unroll
+            for (int sub = 0; sub < CPB; ++sub) {
+                if (CPB > 1 && sub >= nsub) break;
+                const uint32_t boff = (uint32_t)(ch0 + sub) * chunk_bytes;
+                uint32_t raw[2][2][NW];  // this lane's codes of rows g and g + 8 of each 16-row block
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) load_codes(raw[r][h], stage + (uint32_t)((r * 16 + h * 8 + pg) * kBoxRow), sub);
+                if (sub == nsub - 1) {  // the stage is in registers: request the box D ahead into it
+                    __syncwarp();
+                    issue();
+                }
+                float gs[2][4];
+#pragma unroll
+                for (int q = 0; q < PIECES; ++q) {
+                    const uint4 b = lds(bcol + boff + q * piece);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)  // MMA 2 q + j of the chunk: pairs 4 q + 2 j, + 1
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            const int i = 4 * q + 2 * j;
+                            const uint32_t a0 = code_pair(raw[r][0], i), a1 = code_pair(raw[r][1], i);
+                            const uint32_t a2 = code_pair(raw[r][0], i + 1), a3 = code_pair(raw[r][1], i + 1);
+                            if (i == 0) mma_f16<true>(gs[r], a0, a1, a2, a3, b.x, b.y);
+                            else mma_f16<false>(gs[r], a0, a1, a2, a3, j ? b.z : b.x, j ? b.w : b.y);
+                        }
+                }
+                // s (sum x q - z sum x)
+                float s[2][2], z[2][2];
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t sw = CPB == 4 && sub >= 2 ? sz.s[r][h][(CPB + 1) / 2 - 1] : sz.s[r][h][0];
+                        s[r][h] = __uint_as_float((sub & 1) ? (sw & 0xFFFF0000u) : (sw << 16));
+                        z[r][h] = (float)((sz.z[r][h] >> (8 * sub)) & 0xFFu);
+                    }
+                const float2 sx = *reinterpret_cast<const float2 *>(sums + (ch0 + sub) * ms + mcol);
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float v = fmaf(-z[r][q >> 1], (q & 1) ? sx.y : sx.x, gs[r][q]);
+                        sbox[r][q] = sub == 0 ? s[r][q >> 1] * v : fmaf(s[r][q >> 1], v, sbox[r][q]);
+                    }
+            }
+            const float2 u = *reinterpret_cast<const float2 *>(undo + (box - b_lo) * ms + mcol);
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[r][q] = fmaf((q & 1) ? u.y : u.x, sbox[r][q], acc[r][q]);
+        }
+        // ---- end of a tile.  A warp first adds up and writes the tile BEFORE (all sums of it have normally come long ago), then
+        // hands over its own.  The buffer it writes is free: alone (c = 1), whoever announced tile t - 1 had read tile t - 2 before, and it
+        // has waited for all of them; in a cluster the readers say so.
+        if (tl > 0) finish_tile(tile - 1, tl - 1);
+        if (c > 1 && tl > 1 && ok) ok = mbar_wait(freed + 8 * (tl & 1), (uint32_t)(((tl >> 1) - 1) & 1), a.status);
+        const uint32_t to = base + (uint32_t)a.off_red + (uint32_t)(tl & 1) * red_buf + (uint32_t)(slot * a.M * 128 + g * 16);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int m = 2 * t + q;
+            const float v0 = acc[0][q], v1 = acc[0][2 + q], v2 = acc[1][q], v3 = acc[1][2 + q];
+            if (m < a.M) {
+                if (c == 1) asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(to + 128 * m), "f"(v0), "f"(v1), "f"(v2), "f"(v3) : "memory");
+                else st_async_v4(cluster_map(to + 128 * m, (uint32_t)rg), v0, v1, v2, v3, cluster_map(full + 8 * (tl & 1), (uint32_t)rg));
+            }
+            acc[0][q] = acc[0][2 + q] = acc[1][q] = acc[1][2 + q] = 0.f;
+        }
+        if (c == 1) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full + 8 * (tl & 1));
+        }
+    }
+    finish_tile(t1 - 1, t1 - 1 - t0);
+    if (c > 1) {  // nothing is sent to a CTA that has left
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+}
+
+struct Decode8Plan {
+    int log_c;  // below 0: the activations do not fit
+    int off_b, off_t, off_red, off_bar;
+    size_t smem;
+};
+
+// The smallest cluster whose CTAs have room for their share of the activations.
+Decode8Plan decode8_plan(int M, int K, int g) {
+    Decode8Plan p = {};
+    const int nboxes = (K + kBoxK - 1) / kBoxK, cpb = g == 64 ? 4 : 2, ms = (M + 1) & ~1;
+    for (p.log_c = 0; p.log_c <= 3; ++p.log_c) {
+        const size_t boxes = (size_t)(nboxes + (1 << p.log_c) - 1) >> p.log_c;
+        size_t off = (size_t)WARPS * D * kStage;
+        p.off_b = (int)off;
+        off += boxes * kBoxK * 2 * M;
+        p.off_t = (int)off;
+        off += round_up(boxes * (cpb + 1) * ms * 4, 16);
+        p.off_red = (int)off;
+        off += (size_t)2 * WARPS * M * 128;
+        p.off_bar = (int)off;
+        off += (size_t)(WARPS * D + 4) * 8;
+        if (off > kMaxSmem) continue;
+        p.smem = off < kMinSmem ? kMinSmem : off;
+        return p;
+    }
+    p.log_c = -1;
+    return p;
+}
+
+// Clusters of c CTAs that the current device holds at once (a CTA takes an SM).
+template <typename Kernel>
+int max_clusters(Kernel kernel, int threads, int log_c) {
+    static std::atomic<int> known[64][4];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+    if (log_c == 0) return device_sm_count();
+    int n = known[dev][log_c].load();
+    if (n > 0) return n;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1u << log_c, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = kMaxSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1u << log_c;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
+        (void)cudaGetLastError();
+        n = device_sm_count() >> (log_c + 1);
+    }
+    known[dev][log_c].store(n);
+    return n;
+}
+
+template <int GK>
+dmr_status_t launch_decode8_t(Decode8Args a, const Decode8Plan &p, const void *qweight, cudaStream_t st) {
+    using Cfg = Decode8Cfg<GK>;
+    auto kernel = decode8_kernel<GK>;
+    if (!ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), kMaxSmem)) return DMR_ERR_CUDA;
+    a.nchunks = a.K / GK;
+    a.nboxes = (a.nchunks + Cfg::CPB - 1) / Cfg::CPB;
+    const int per_group = a.K / a.G / GK;
+    a.g_mul = per_group > 1 ? (uint32_t)((0x100000000ull + (uint64_t)per_group - 1) / (uint64_t)per_group) : 0u;  // exact for the numbers that occur
+    a.sz_vec = per_group == 1 && a.G % Cfg::CPB == 0 && (uintptr_t)a.scales % (2 * Cfg::CPB) == 0 && (uintptr_t)a.zeros % Cfg::CPB == 0;
+    const int tiles = (a.N + (32 << p.log_c) - 1) >> (5 + p.log_c);
+    int clusters = max_clusters(kernel, WARPS * 32, p.log_c);
+    if (clusters > tiles) clusters = tiles;
+    a.tiles_each = tiles / clusters;
+    a.tiles_more = tiles % clusters;
+    CUtensorMap wmap;
+    const uint64_t rb = (uint64_t)a.K / 2;
+    if (!make_tensor_map_2d(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, qweight, (uint64_t)a.N, rb, rb, 32, kBoxRow, TmaSwizzle::k128B))
+        return DMR_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)clusters << p.log_c, 1, 1);
+    cfg.blockDim = dim3(WARPS * 32, 1, 1);
+    cfg.dynamicSmemBytes = p.smem;  // more than half of an SM's: two CTAs of these kernels never share an SM (see above)
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int n_attr = 0;
+    if (tc_pdl_enabled()) {
+        attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (p.log_c) {
+        attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+        attr[n_attr].val.clusterDim.x = 1u << p.log_c;
+        attr[n_attr].val.clusterDim.y = attr[n_attr].val.clusterDim.z = 1;
+        ++n_attr;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = (unsigned)n_attr;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, wmap, a);
+    if (e != cudaSuccess) return launch_failed(e);
+    return check_launch();
+}
+
+}  // namespace
+
+// us, against decode.cu's kernel: four 7B linears, groups of 128, 1 row 33.9 and 39.4, 2 rows 38.0 and 39.9, 4 rows 39.2 and 40.2, 6 rows 42.3 and 40.4 (the conversion of
+// the activations, which every CTA does for itself, grows with the rows); groups of 64, whose chunks cost the other kernel more, 1 row 37.9 and 45.9, 3 rows 44.4
+// and 47.6, 5 rows 48.6 and 48.2; 14B layer, 1 row, groups of 128 63.0 and 71.2; 32B layer, 1 row, groups of 128 49.2 and 61.5, of 64 55.3 and 71.7.  A cluster
+// pays for groups of 64 alone (32B layer, groups of 128, 3 rows: 61.4 and 63.2 with one for one of the linears; 14B layer 74 to 85 and 74 to 77).
+bool decode8_supported(int M, int K, int bits, int g) {
+    if (bits != 4 || M < 1 || M > 4) return false;
+    if (g == 64) return K % 64 == 0 && decode8_plan(M, K, g).log_c >= 0;
+    return g % 128 == 0 && K % 128 == 0 && decode8_plan(M, K, g).log_c == 0;
+}
+
+void decode8_describe(int M, int K, int g, int *warps, int *cluster) {
+    *warps = WARPS;
+    *cluster = 1 << decode8_plan(M, K, g).log_c;
+}
+
+dmr_status_t launch_decode8(const uint16_t *X, int M, RowSel sel, const void *qweight, const uint16_t *scales, const uint8_t *zeros, int N, int K, int g,
+                            void *Y, dmr_out_t out, int32_t *status, cudaStream_t st) {
+    const Decode8Plan p = decode8_plan(M, K, g);
+    if (p.log_c < 0) return DMR_ERR_UNSUPPORTED;
+    Decode8Args a = {};
+    a.X = X;
+    a.idx = sel.idx;
+    a.count = sel.count;
+    a.coff = sel.offset;
+    a.scales = scales;
+    a.zeros = zeros;
+    a.Y = Y;
+    a.status = status;
+    a.M = M;
+    a.N = N;
+    a.K = K;
+    a.G = K / g;
+    a.out_f32 = out == DMR_OUT_F32;
+    a.log_c = p.log_c;
+    a.off_b = p.off_b;
+    a.off_t = p.off_t;
+    a.off_red = p.off_red;
+    a.off_bar = p.off_bar;
+    return g == 64 ? launch_decode8_t<64>(a, p, qweight, st) : launch_decode8_t<128>(a, p, qweight, st);
+}
+
+}  // namespace dmr

@@ -1,0 +1,64 @@
+"""4-bit linears of a few rows against the oracle at the edges of their kernel: fewer features than a tile and ragged ones, half-used last boxes, fewer
+boxes than warps and several per warp, clusters of 2 and 4 CTAs (long rows), scale tables that are not aligned, groups of several chunks, rows of very
+different size, a row that is not finite, and routed calls with fewer rows than the call has."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2602_02711_b200 as dmr
+from paper_2602_02711_b200 import inputs, QFormat, OUT_BF16, OUT_F32
+from paper_2602_02711_b200.binding import OP_LOWBIT
+from helpers import to_dev_bf16
+
+pytestmark = pytest.mark.gpu
+
+# Exact products.  The tensor cores' fp32 sums of a chunk are cut off, not rounded, in each of eight additions: 2^-23 of a sum of x q, which is up to four
+# times (a code of 0 .. 15 against its distance from the zero point) what is left of it where one large activation prevails.  The roundings of scaling and adding
+# up are a quarter of that.
+TOL = 8 * 2.0 ** -23 * 4 * 1.25
+
+
+@pytest.mark.parametrize("M,N,K,group,cluster", [
+    (1, 40, 128, 128, 1), (1, 4800, 384, 128, 1), (3, 100, 640, 128, 1), (4, 1000, 4224, 128, 1), (2, 64, 768, 256, 1), (4, 33, 1024, 0, 1), (1, 70, 11008, 128, 1),
+    (1, 40, 64, 64, 1), (2, 5000, 320, 64, 1), (4, 96, 1088, 64, 1), (3, 130, 5120, 64, 1), (4, 300, 11008, 64, 2), (2, 5000, 27648, 64, 2), (4, 600, 27648, 64, 4),
+])
+def test_few_rows(M, N, K, group, cluster):
+    plan = dmr.dmr_describe_dispatch(OP_LOWBIT, M, N, K, QFormat(4, group))
+    assert plan["kernel"] == "decode_w4" and plan["cluster"] == cluster
+    W, X = inputs.weights(N, K, seed=K), inputs.activations(M, K, seed=N, outlier_frac=0.01)
+    Xf = inputs.bf16_bits_to_f64(X)
+    Xf[-1] *= 2.0 ** -60
+    X = inputs.f64_to_bf16_bits(Xf)
+    q = dmr.dmr_quantize(to_dev_bf16(W), QFormat(4, group))
+    want = oracle.lowbit_linear(X, *oracle.quantize(W, bits=4, group=group), bits=4, group=group)
+    Y = dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_F32)
+    got = Y.cpu().numpy().astype(np.float64)
+    for m in range(M):
+        assert np.linalg.norm(got[m] - want[m]) <= TOL * np.linalg.norm(want[m])
+    assert torch.equal(dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_BF16), Y.to(torch.bfloat16))
+    if M > 1:  # a row of its own, and a row that is not finite
+        Xd = to_dev_bf16(X)
+        Xd[0, K // 2] = float("inf")
+        Yn = dmr.dmr_lowbit_linear(Xd, q, OUT_F32)
+        assert torch.equal(Yn[1:], Y[1:]) and not torch.isfinite(Yn[0]).any()
+        Wd = to_dev_bf16(W)
+        for keep in (1, M - 1):
+            mask = torch.ones(M, dtype=torch.uint8, device="cuda")
+            mask[:keep] = 0
+            assert torch.equal(dmr.dmr_routed_linear(to_dev_bf16(X), mask, Wd, q, OUT_F32)[:keep], Y[:keep])
+
+
+def test_scale_tables_at_odd_addresses():
+    N, K, M = 96, 512, 2
+    W, X = inputs.weights(N, K, seed=3), inputs.activations(M, K, seed=4)
+    q = dmr.dmr_quantize(to_dev_bf16(W), QFormat(4, 128))
+    want = dmr.dmr_lowbit_linear(to_dev_bf16(X), q, OUT_F32)
+    scales, zeros = torch.empty(N * 4 + 1, dtype=torch.bfloat16, device="cuda"), torch.empty(N * 4 + 1, dtype=torch.uint8, device="cuda")
+    scales[1:], zeros[1:] = q.scales.flatten(), q.zeros.flatten()
+    Y, ws = torch.empty_like(want), dmr.new_workspace(OP_LOWBIT, M, N, K, q.fmt)
+    lib, st = dmr.lib(), torch.cuda.current_stream().cuda_stream
+    assert lib.dmr_lowbit_linear(to_dev_bf16(X).data_ptr(), M, q.qweight.data_ptr(), scales[1:].data_ptr(), zeros[1:].data_ptr(), N, K, q.fmt,
+                                 Y.data_ptr(), OUT_F32, ws.data_ptr(), ws.numel(), st) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(Y, want)
