@@ -48,6 +48,10 @@ struct SmallCfg {
     static constexpr int TURN = UW / 4 > MW ? UW / 4 : MW;
     static constexpr int S_RAW = (216 * 1024) / STAGE / TURN * TURN;
     static constexpr int S = S_RAW > 16 ? 16 : S_RAW;
+    // Weights requested ahead of the activations: what is requested behind a whole ring (216 KB an SM) comes late (8 bits, 72 KB, us: 32B layer 13 rows 66.8 ->
+    // 66.3, 7B layer 1 row 65.4 -> 64.3; 4 bits, 20 rows 75.8 -> 75.0; routed 14B layer, 64 rows 256.5 -> 254.4).  bf16 weights of up to 32 rows keep memory busy with
+    // more (7B layer, 3 rows: a ring 80.0, 144 KB 78.8, 72 KB 80.4).
+    static constexpr int AHEAD = ((BITS == 0 && BN < 64 ? 144 : 72) * 1024 + W_BYTES - 1) / W_BYTES;
     static constexpr int EW = BN == 128 ? 8 : 4;                       // scale warps, at most 64 rows of the batch each
     // warps: unpack first, so that groups of four cover the lane quadrants, then scale, MMA, copies
     static constexpr int WARPS = UW + EW + MW + 1;
@@ -245,7 +249,7 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
     // The first weights run ahead of the preceding kernel's end where the interface says so (up to 32 rows; in a routed call, whose split has waited
     // for what the caller's earlier work wrote, they run ahead of the number of rows as well).  Elsewhere that kernel may still be writing them, and
     // they come as far as the L2 (four 7B linears, bf16, 64 rows: 105.5 us without that, 102 with it, 97 if they were copied at once).
-    const int first = min(hi - lo, S);
+    const int first = min(hi - lo, S), ahead = min(first, Cfg::AHEAD);
     if (BN >= 64 && !a.count) {
         if (warp == W_COPY && lane == 0) {
             for (int i = 0; i < first; ++i) {
@@ -258,7 +262,7 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
         pdl_wait();
     }
     if (warp == W_COPY && lane == 0) {
-        for (int i = 0; i < first; ++i) {
+        for (int i = 0; i < ahead; ++i) {
             const int u = lo + i, tile = u / a.k_units;
             copy_w(i, tile, u - tile * a.k_units);
         }
@@ -274,9 +278,9 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
     if (warp == W_COPY) {
         // ================= copies =================
         if (lane == 0) {
-            int issued = first, x_issued = 0;
+            int issued = ahead, x_issued = 0;
             if (work) {
-                int tile = (lo + first) / a.k_units, ku = lo + first - tile * a.k_units, xku = lo_ku;  // the next unit's weights, and activations
+                int tile = (lo + ahead) / a.k_units, ku = lo + ahead - tile * a.k_units, xku = lo_ku;  // the next unit's weights, and activations
                 auto copy_x = [&](int s) {
                     mbar_expect_tx(xfull_bar(s), 2 * Cfg::X_HALF);
                     tma_load_2d(x_tile(s, 0), &map_x, xfull_bar(s), xku * kSk, 0);
@@ -284,7 +288,16 @@ __device__ __forceinline__ void small_body(const CUtensorMap &map_w, const CUten
                     if (++xku == a.k_units) xku = 0;
                 };
                 pdl_wait();
-                for (int i = 0; i < first; ++i) copy_x(i);
+                for (int i = 0; i < ahead; ++i) copy_x(i);
+                for (int i = ahead; i < first; ++i) {
+                    copy_w(i, tile, ku);
+                    if (++ku == a.k_units) {
+                        ku = 0;
+                        ++tile;
+                    }
+                    copy_x(i);
+                }
+                issued = first;
                 for (int u = lo + first, s = 0, par = 0; u < hi; ++u) {
                     if (!mbar_wait(done_bar(s), (uint32_t)par, a.status)) break;
                     copy_w(s, tile, ku);
