@@ -34,9 +34,9 @@ METRIC = "low-bit linear: decode weight GB/s vs HBM peak; prefill TFLOP/s vs bf1
 WORKLOAD = "decode sweep, 7B-class layer (qkv, o, gate_up, down), M in {1,8,16}, INT4 g=128"
 DECODE_MS = (1, 8, 16)
 BITS, GROUP = 4, 128
-# dram__bytes_read.sum + dram__bytes_write.sum per launch of decode_w4_kernel, mean of the four 7B-class
-# linears at M = 1 (ncu capture summarised in profiles/decode_w4_kernel_int4_g128_7b_M1.txt)
-DECODE_TRAFFIC_BYTES_PER_LAUNCH = 26.54e6
+# dram__bytes_read.sum + dram__bytes_write.sum per launch of decode8_kernel, mean of the four 7B-class
+# linears at M = 1 (ncu capture summarised in profiles/decode8_kernel_int4_g128_7b_M1.txt; the same weights are read at M = 8 and 16)
+DECODE_TRAFFIC_BYTES_PER_LAUNCH = 26.56e6
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
@@ -322,7 +322,7 @@ def run_ours(args):
             "gpu_launches": n_launch,
             "roofline": {"bound": "hbm", "achieved": per_gpu, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                          "frac": per_gpu / peaks["hbm_gbs"], "traffic": DECODE_TRAFFIC_BYTES_PER_LAUNCH,
-                         "kernel": "decode_w4_kernel", "peak_source": peaks["_source"],
+                         "kernel": "decode8_kernel (M = 1), decode_w4_kernel (M = 8, 16)", "peak_source": peaks["_source"],
                          "us_per_launch": seconds / n_launch * 1e6,
                          "algorithmic_bytes_per_launch": step_bytes / launches_per_step},
         })
