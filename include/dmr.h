@@ -277,7 +277,7 @@ dmr_status_t dmr_workspace_status(const void *workspace, void *stream);
  * Writes a one-line description of the kernel family and launch shape that dmr_lowbit_linear
  * (op = DMR_OP_LOWBIT_LINEAR) or dmr_dense_linear (DMR_OP_DENSE_LINEAR; f is ignored) would use for these sizes
  * on the current device, e.g. "pair bits=4 rows=256 splits=1 tiles=768 ctas=148" (bits = 0, of "stream" and "simple" 16: bf16 weights; rows: activation rows of a
- * tile; "pair": csrc/pair.cu, "small": small.cu, "decode_w4", "decode_w3": decode.cu, "stream": stream.cu, "simple": simple.cu).  Launches nothing.  Returns the length
+ * tile; "pair": csrc/pair.cu, "small": small.cu, "decode_w4": decode8.cu (with its cluster size) or decode.cu, "decode_w3": decode.cu, "stream": stream.cu, "simple": simple.cu).  Launches nothing.  Returns the length
  * snprintf reports, or -1 for invalid arguments.  For tests and benchmarks that must know which kernel they ran.
  */
 int dmr_describe_dispatch(dmr_op_t op, int M, int N, int K, dmr_qformat_t f, char *buf, size_t buf_bytes);

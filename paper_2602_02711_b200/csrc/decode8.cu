@@ -5,7 +5,8 @@
 // What bounds it.  HBM, if the arithmetic keeps out of the way.  A code among the low eleven bits of a 16-bit word IS an fp16 number, exactly: up to 2^11
 // the bits count in steps of 2^-24, through the subnormals and the first binade above.  So the pairs of 4-bit codes of a word are an AND each,
 // in place, with one byte permute for half of them, and the otherwise idle FMA pipe does the rest (code_pair): 4 integer instructions for 8 codes where bf16
-// numbers 128 + q need 7.  Nothing is rounded and no offset is added: the tensor cores (mma.m16n8k16, the weights as the 16-row operand) sum x q, and per chunk of inputs, which never crosses a quantization group,
+// numbers 128 + q need 7.  Nothing is rounded and no offset is added: the tensor cores (mma.m16n8k16, the weights as the 16-row operand) sum x q, and
+// per chunk of inputs, which never crosses a quantization group,
 //     sum_k x_k s (q_k - z) = s (sum_k x_k q_k - z sum_k x_k)
 // is formed in fp32 (errors against 64 bits: 1e-7 of the outputs' 2-norm, 2.5e-6 with the offset).  Activations are converted to fp16 once per CTA, after scaling a
 // row's inputs of a box by the power of two that brings the largest to [2^14, 2^15): exact for all that are above 2^-31 of it, and to 2^-39 of the largest for
@@ -260,7 +261,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1) decode8_kernel(const __grid_con
     float *undo = sums + ((a.nboxes + c - 1) >> a.log_c) * CPB * ms;                    // [box][ms] power of two that undoes their scale
     {
         if (rows == 1) {
-            // a lane takes eight inputs of a box: piece q of lane ct's block (a fifth of the steps of the way below, which three quarters of the lanes would idle through)
+            // a lane takes eight inputs of a box: piece q of lane ct's block (36.3 -> 32.3 us where the way below, in which three quarters of the lanes idle,
+            // did it; codes not yet times 16)
             const int sub = lane / (GK / 8), ct = lane % (GK / 8) / PIECES, q = lane % PIECES;
             const uint4 *x = reinterpret_cast<const uint4 *>(a.X + (size_t)(a.idx ? a.idx[0] : 0) * a.K) + lane;
             auto load_x = [&](int box) { return box < b_hi && box * CPB + sub < a.nchunks ? __ldg(x + box * (kBoxK / 8)) : make_uint4(0u, 0u, 0u, 0u); };
@@ -322,7 +324,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1) decode8_kernel(const __grid_con
                 for (int i = 0; i < PIECES; ++i) {
                     uint4 v;
                     part[i] = convert_octet(cur[i], scale_field(top), v);
-                    if (m < rows) *reinterpret_cast<uint4 *>(smem + a.off_b + (uint32_t)(bl * CPB + sub) * chunk_bytes + i * piece + (uint32_t)(64 * m + 16 * t)) = v;
+                    const uint32_t at = a.off_b + (uint32_t)(bl * CPB + sub) * chunk_bytes + i * piece + (uint32_t)(64 * m + 16 * t);
+                    if (m < rows) *reinterpret_cast<uint4 *>(smem + at) = v;
                 }
                 // (added in the order of the way above: a routed call may have one row where its caller has several)
                 float sum = PIECES == 4 ? (part[0] + part[1]) + (part[PIECES - 2] + part[PIECES - 1]) : part[0] + part[1];
@@ -591,8 +594,8 @@ dmr_status_t launch_decode8_t(Decode8Args a, const Decode8Plan &p, const void *q
 
 }  // namespace
 
-// us, against decode.cu's kernel: four 7B linears, groups of 128, 1 row 33.9 and 39.4, 2 rows 38.0 and 39.9, 4 rows 39.2 and 40.2, 6 rows 42.3 and 40.4 (the conversion of
-// the activations, which every CTA does for itself, grows with the rows); groups of 64, whose chunks cost the other kernel more, 1 row 37.9 and 45.9, 3 rows 44.4
+// us, against decode.cu's kernel: four 7B linears, groups of 128, 1 row 33.9 and 39.4, 2 rows 38.0 and 39.9, 4 rows 39.2 and 40.2, 6 rows 42.3
+// and 40.4 (the conversion of the activations, which every CTA does for itself, grows with the rows); groups of 64, whose chunks cost the other kernel more, 1 row 37.9 and 45.9, 3 rows 44.4
 // and 47.6, 5 rows 48.6 and 48.2; 14B layer, 1 row, groups of 128 63.0 and 71.2; 32B layer, 1 row, groups of 128 49.2 and 61.5, of 64 55.3 and 71.7.  A cluster
 // pays for groups of 64 alone (32B layer, groups of 128, 3 rows: 61.4 and 63.2 with one for one of the linears; 14B layer 74 to 85 and 74 to 77).
 bool decode8_supported(int M, int K, int bits, int g) {
